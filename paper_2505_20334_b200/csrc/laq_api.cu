@@ -135,7 +135,7 @@ void plan_workspace(const Dims& d, int tiles_per_task, Workspace* w) {
   w->total = off;
 }
 
-static bool use_tensor_core_path(const Dims& d) { return d.D == 128 && d.M <= 256; }
+static bool use_tensor_core_path(const Dims& d) { return d.D <= 128 && d.M <= 256; }
 
 static thread_local int g_last_launches = 0;
 static thread_local cudaEvent_t g_ev_begin = nullptr, g_ev_end = nullptr;

@@ -99,9 +99,11 @@ laq_status selection_source(const Dims& d, const Workspace& w, char* ws, cudaStr
                             int* launches, const float** colsum, Dims* dsel);
 
 // Scoring back ends: both fill colsum (fp32 [U][L_pad]) on `stream`.
-// Tensor-core path (tcgen05 + TMA), head_dim 128, M <= 256.
+// Tensor-core path (tcgen05 + TMA), head_dim <= 128, M <= 256.
 laq_status score_tc_launch(const laq_params& p, const Dims& d, const Workspace& w, const void* q,
                            const void* k, char* ws, cudaStream_t stream, int* launches);
+// Unit whose statistics a test build withholds (-1 in the library).
+int64_t test_withhold_unit();
 // Raw-logit mode (Eq. 4 read literally): one streaming pass over K on CUDA cores.
 laq_status score_raw_launch(const laq_params& p, const Dims& d, const Workspace& w, const void* q,
                             const void* k, char* ws, cudaStream_t stream, int* launches);

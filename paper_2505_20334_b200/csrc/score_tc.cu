@@ -1,5 +1,5 @@
 // Tensor-core scoring kernel for sm_100a: steps 1-3 of the unit computation (Eq. 4 of
-// Section 4.3 read as attention weights) for head_dim 128 and up to 256 softmax rows per unit.
+// Section 4.3 read as attention weights) for head dims up to 128 and up to 256 softmax rows per unit.
 //
 // One persistent CTA per SM pulls tasks from a global ticket counter. A task is one sweep over a
 // chunk of consecutive 128-key tiles of one unit:
@@ -38,6 +38,7 @@
 
 #include "laq_internal.cuh"
 #include "softmax_math.cuh"
+#include "tc_ptx.cuh"
 
 #ifndef LAQ_WAIT_HINT_NS
 #define LAQ_WAIT_HINT_NS 2000  // longest hardware suspension of one mbarrier poll
@@ -47,6 +48,7 @@ namespace laq {
 namespace {
 
 using namespace laq::math;
+using namespace laq::ptx;
 
 constexpr int kSoftmaxWgs = 4;
 constexpr int kSoftmaxWarps = 4 * kSoftmaxWgs;
@@ -85,6 +87,7 @@ struct TcArgs {
   int64_t U;
   int Bt, Hkv, G, W, W_local, L, M, M_pad, n_part, L_pad, n_tiles;
   int tiles_per_task, tasks_per_unit;
+  int boxes, ksteps;    // 64-dim boxes and 16-dim MMA steps per row (2 and 8 for head_dim 128)
   int lag_tasks;        // tasks the second sweep trails the first by
   int tasks_per_layer;  // per-prompt lengths: sweep-1 tasks of one layer (all prompts and KV heads)
   uint32_t total_tickets;
@@ -138,141 +141,6 @@ struct Ctl {
   int task_prefix[LAQ_MAX_RAGGED_BATCH + 1];
 };
 static_assert(sizeof(Ctl) <= kCtlBytes, "control block too large");
-
-// ------------------------------------------------------------------ PTX wrappers
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n.reg .pred p;\n"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      "selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// The same, letting the hardware suspend the thread for up to `ns` nanoseconds while the phase is
-// incomplete (it resumes as soon as the phase completes), so that a long wait polls rarely.
-__device__ __forceinline__ bool mbar_try_wait_for(uint32_t bar, uint32_t parity, uint32_t ns) {
-  uint32_t ok;
-  asm volatile(
-      "{\n.reg .pred p;\n"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
-      "selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity), "r"(ns)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ uint64_t l2_policy_evict_last() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-__device__ __forceinline__ uint64_t l2_policy_evict_first() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-__device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map, uint32_t bar,
-                                            int c0, int c1, int c2, int c3, int c4) {
-  asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes "
-      "[%0], [%1, {%3, %4, %5, %6, %7}], [%2];" ::"r"(dst),
-      "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
-      : "memory");
-}
-__device__ __forceinline__ void tma_load_5d_hint(uint32_t dst, const CUtensorMap* map, uint32_t bar,
-                                                 int c0, int c1, int c2, int c3, int c4,
-                                                 uint64_t policy) {
-  asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint "
-      "[%0], [%1, {%3, %4, %5, %6, %7}], [%2], %8;" ::"r"(dst),
-      "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "l"(policy)
-      : "memory");
-}
-// D[tmem] (+)= A[smem] * B[smem]; the two shared-memory descriptors are passed as (low, high) words.
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo,
-                                          uint32_t desc_hi, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n.reg .pred p;\n.reg .b64 da, db;\n"
-      "mov.b64 da, {%1, %3};\nmov.b64 db, {%2, %3};\n"
-      "setp.ne.b32 p, %5, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n}" ::"r"(d_tmem),
-      "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-               : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-// 32 consecutive fp32 columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
-  uint32_t* r = reinterpret_cast<uint32_t*>(v);
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]),
-        "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
-        "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-}
-// Waits for every tcgen05.ld this thread has issued; the registers of the buffer about to be
-// used are named so that no use of them can move ahead of the wait.
-__device__ __forceinline__ void tmem_ld_wait(float* v) {
-  uint32_t* r = reinterpret_cast<uint32_t*>(v);
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]),
-                 "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]),
-                 "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]),
-                 "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]),
-                 "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]),
-                 "+r"(r[31])
-               :
-               : "memory");
-}
-// Adds to a global fp32 without returning a value.
-__device__ __forceinline__ void red_add(float* p, float v) {
-  asm volatile("red.global.add.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
-}
-
-// Shared-memory matrix descriptor of a K-major operand with 128-byte swizzle, rows of 128 bytes
-// and groups of 8 rows 1024 bytes apart, split into its two words.
-// Low word: start address >> 4 in bits [0,14), leading byte offset (unused by swizzled K-major) in
-// bits [16,30). High word: stride byte offset 1024 >> 4 in bits [32,46), descriptor version 1 of
-// sm_100 at bit 46, 128-byte swizzle (2) at bits [61,64). Advancing the start address by `bytes`
-// (inside one shared-memory window below 256 KiB) is an add of bytes >> 4 to the low word.
-__device__ __forceinline__ uint32_t smem_desc_lo(uint32_t addr) {
-  return ((addr & 0x3FFFFu) >> 4) | (1u << 16);
-}
-constexpr uint32_t kSmemDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
-// Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M x N tile.
-__device__ __forceinline__ uint32_t instr_desc(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
 
 // ------------------------------------------------------------------ bounded waits
 __device__ __noinline__ void record_timeout(const TcArgs& a, Ctl* ctl, int site) {
@@ -558,16 +426,13 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
           const uint32_t qs = qcount & 1u;
           if (!mbar_wait(a, ctl, smem_u32(&ctl->q_empty[qs]), ((qcount >> 1) & 1u) ^ 1u, 3)) break;
           const uint32_t bar = smem_u32(&ctl->q_full[qs]);
-          mbar_expect_tx(bar, (uint32_t)a.M * 256u * (kDup ? 2u : 1u));
-          const uint32_t dst = q_base + qs * q_stage_bytes;
-          tma_load_5d(dst, &tmap_q, bar, 0, 0, task.h * a.G, task.b, task.layer);
-          tma_load_5d(dst + kQRows * 128u, &tmap_q, bar, 64, 0, task.h * a.G, task.b,
-                      task.layer);
-          if (kDup) {
+          mbar_expect_tx(bar, (uint32_t)(a.M * a.boxes) * 128u * (kDup ? 2u : 1u));
+          for (int j = 0; j < a.boxes; ++j) {
+            const uint32_t dst = q_base + qs * q_stage_bytes + (uint32_t)j * (kQRows * 128u);
+            tma_load_5d(dst, &tmap_q, bar, 64 * j, 0, task.h * a.G, task.b, task.layer);
             // a second copy of the rows, 64 rows (8192 bytes: the swizzle pattern repeats) further
-            tma_load_5d(dst + 8192u, &tmap_q, bar, 0, 0, task.h * a.G, task.b, task.layer);
-            tma_load_5d(dst + kQRows * 128u + 8192u, &tmap_q, bar, 64, 0, task.h * a.G,
-                        task.b, task.layer);
+            if (kDup)
+              tma_load_5d(dst + 8192u, &tmap_q, bar, 64 * j, 0, task.h * a.G, task.b, task.layer);
           }
           ++qcount;
         }
@@ -582,12 +447,13 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
             break;
           }
           const uint32_t bar = smem_u32(&ctl->k_full[s]);
-          mbar_expect_tx(bar, kKStageBytes);
+          mbar_expect_tx(bar, (uint32_t)a.boxes * (kKStageBytes / 2));
           const uint32_t dst = k_base + s * kKStageBytes;
           const int key0 = (task.tile0 + i) * TILE_KEYS;
           tma_load_5d_hint(dst, &tmap_k, bar, 0, key0, task.h, task.b, task.layer, pol);
-          tma_load_5d_hint(dst + kKStageBytes / 2, &tmap_k, bar, 64, key0, task.h, task.b, task.layer,
-                           pol);
+          if (a.boxes > 1)
+            tma_load_5d_hint(dst + kKStageBytes / 2, &tmap_k, bar, 64, key0, task.h, task.b, task.layer,
+                             pol);
           ++kcount;
         }
         if (next_ticket < a.total_tickets) decode_ticket(a, prefix, next_ticket, next);
@@ -644,7 +510,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
             for (int rb = 0; rb < RB; ++rb) {
 #pragma unroll
               for (int kk = 0; kk < 8; ++kk)
-                umma_bf16(d_tmem + (uint32_t)rb * 128u,
+                if (kk < a.ksteps) umma_bf16(d_tmem + (uint32_t)rb * 128u,
                           q_lo + (kk >> 2) * q_half16 + (uint32_t)rb * 1024u + (kk & 3) * 2u,
                           k_lo + (kk >> 2) * (kKStageBytes >> 5) + (kk & 3) * 2u, kSmemDescHi,
                           idesc_s1, kk > 0);
@@ -652,7 +518,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
           } else {
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk)
-              umma_bf16(d_tmem, k_lo + (kk >> 2) * (kKStageBytes >> 5) + (kk & 3) * 2u,
+              if (kk < a.ksteps) umma_bf16(d_tmem, k_lo + (kk >> 2) * (kKStageBytes >> 5) + (kk & 3) * 2u,
                         q_lo + (kk >> 2) * q_half16 + (kk & 3) * 2u, kSmemDescHi, idesc_s2, kk > 0);
           }
           umma_commit(smem_u32(&ctl->mma_done[s]));
@@ -980,9 +846,10 @@ EncodeTiledFn get_encode_fn() {
   return fn;
 }
 
-// 5-D bf16 tensor map (dims innermost first) with a 128-byte swizzled box.
-bool make_map(CUtensorMap* map, const void* base, const uint64_t dims[5], const int64_t strides_el[4],
-              const uint32_t box[5]) {
+}  // namespace
+
+bool make_tensor_map(CUtensorMap* map, const void* base, const uint64_t dims[5],
+                     const int64_t strides_el[4], const uint32_t box[5]) {
   EncodeTiledFn fn = get_encode_fn();
   if (!fn) return false;
   cuuint64_t gdim[5], gstride[4];
@@ -998,14 +865,17 @@ bool make_map(CUtensorMap* map, const void* base, const uint64_t dims[5], const 
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+namespace {
+
 #ifdef LAQ_TEST_HOOKS
 std::atomic<long long> g_withhold_unit{-1};
+}  // namespace
 int64_t test_withhold_unit() { return g_withhold_unit.load(); }
 #else
+}  // namespace
 int64_t test_withhold_unit() { return -1; }
 #endif
 
-}  // namespace
 }  // namespace laq
 
 #ifdef LAQ_TEST_HOOKS
@@ -1073,6 +943,8 @@ laq_status score_tc_launch(const laq_params& p, const Dims& d, const Workspace& 
   if (lag_tasks > n_stream) lag_tasks = n_stream;
   a.lag_tasks = (int)lag_tasks;
   a.scale_log2 = d.scale * kLog2e;
+  a.boxes = (d.D + 63) / 64;
+  a.ksteps = (d.D + 15) / 16;
   a.hdr = (int32_t*)(ws + w.off_hdr);
   a.cnt = (int32_t*)(ws + w.off_cnt);
   a.part = (float2*)(ws + w.off_part);
@@ -1084,13 +956,13 @@ laq_status score_tc_launch(const laq_params& p, const Dims& d, const Workspace& 
   const bool dup = w.M_pad <= 64;  // sweep 1 holds every query row twice, on lanes r and 64 + r
 
   CUtensorMap tmap_q, tmap_k;
-  const uint64_t qdims[5] = {128, (uint64_t)d.W, (uint64_t)d.Hq, (uint64_t)d.Bt, (uint64_t)d.NL};
+  const uint64_t qdims[5] = {(uint64_t)d.D, (uint64_t)d.W, (uint64_t)d.Hq, (uint64_t)d.Bt, (uint64_t)d.NL};
   const int64_t qstr[4] = {p.q_stride_pos, p.q_stride_head, p.q_stride_batch, p.q_stride_layer};
   const uint32_t qbox[5] = {64, (uint32_t)d.W, (uint32_t)d.G, 1, 1};
-  const uint64_t kdims[5] = {128, (uint64_t)d.L, (uint64_t)d.Hkv, (uint64_t)d.Bt, (uint64_t)d.NL};
+  const uint64_t kdims[5] = {(uint64_t)d.D, (uint64_t)d.L, (uint64_t)d.Hkv, (uint64_t)d.Bt, (uint64_t)d.NL};
   const int64_t kstr[4] = {p.k_stride_pos, p.k_stride_head, p.k_stride_batch, p.k_stride_layer};
   const uint32_t kbox[5] = {64, TILE_KEYS, 1, 1, 1};
-  if (!make_map(&tmap_q, q, qdims, qstr, qbox) || !make_map(&tmap_k, k, kdims, kstr, kbox))
+  if (!make_tensor_map(&tmap_q, q, qdims, qstr, qbox) || !make_tensor_map(&tmap_k, k, kdims, kstr, kbox))
     return score_simt_launch(p, d, w, q, k, ws, stream, launches);  // layout TMA cannot describe
 
   const size_t smem = kCtlBytes + 2u * (size_t)q_rows * 256u + (size_t)n_slots * kKStageBytes;
