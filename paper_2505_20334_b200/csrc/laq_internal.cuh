@@ -102,6 +102,10 @@ laq_status selection_source(const Dims& d, const Workspace& w, char* ws, cudaStr
 // Tensor-core path (tcgen05 + TMA), head_dim <= 128, M <= 256.
 laq_status score_tc_launch(const laq_params& p, const Dims& d, const Workspace& w, const void* q,
                            const void* k, char* ws, cudaStream_t stream, int* launches);
+// The same steps in one pass over K, for units whose logits fit the tensor memory of a cluster
+// (*done says whether it was launched; if not, nothing was enqueued).
+laq_status score_cluster_launch(const laq_params& p, const Dims& d, const Workspace& w, const void* q,
+                                const void* k, char* ws, cudaStream_t stream, int* launches, bool* done);
 // Unit whose statistics a test build withholds (-1 in the library).
 int64_t test_withhold_unit();
 // Raw-logit mode (Eq. 4 read literally): one streaming pass over K on CUDA cores.

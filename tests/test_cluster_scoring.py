@@ -1,0 +1,64 @@
+"""Scoring with the logits of a unit kept in the tensor memory of a thread-block cluster (up to 64
+softmax rows): the sizes at which tiles, row groups, clusters and head dims end, against the fp64
+oracle with the tolerances of the other parity tests."""
+import numpy as np
+import pytest
+import torch
+
+from parity_util import SCORE_RTOL
+from test_gpu_parity import compare_all_units, laq, rand_inputs  # noqa: F401 (laq is a fixture)
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # NL Bt Hq Hkv D    L     W  W_local k  B   lens
+    (1, 1, 1, 1, 128, 129, 1, 0, 1, 10, None),           # one row; a tile and one key
+    (1, 1, 1, 1, 128, 128, 9, 3, 3, 20, None),           # nine rows (two groups), exactly one tile
+    (1, 2, 5, 1, 128, 2049, 8, 8, 7, 100, None),         # 40 rows; 17 tiles, every CTA but one short
+    (1, 1, 7, 1, 128, 1000, 8, 0, 5, 60, None),          # 56 rows run as 64
+    (1, 1, 3, 1, 128, 3000, 19, 19, 7, 100, None),       # 57 rows, heads straddle the groups, all local
+    (1, 1, 8, 2, 128, 16384, 16, 0, 5, 64, None),        # the longest unit that fits at 64 rows
+    (1, 1, 8, 2, 128, 16385, 16, 16, 5, 64, None),       # and the first that does not
+    (1, 3, 8, 2, 128, 4100, 16, 16, 7, 50, (4100, 51, 130)),  # CTAs without a tile of the short prompts
+    (3, 7, 8, 2, 128, 700, 4, 2, 3, 40, None),           # more units than clusters: several rounds
+    (1, 1, 4, 1, 8, 300, 4, 0, 3, 40, None),             # head dims 8 .. 256
+    (1, 1, 4, 1, 80, 900, 8, 4, 7, 60, None),
+    (1, 2, 4, 1, 96, 500, 16, 0, 7, 60, (500, 257)),
+    (1, 1, 8, 2, 192, 1100, 8, 0, 7, 60, None),
+    (1, 1, 8, 2, 256, 2000, 16, 16, 7, 60, None),
+]
+
+
+@pytest.mark.parametrize("case", CASES, ids=[f"L{c[5]}-M{c[2] // c[3] * c[6]}-D{c[4]}" for c in CASES])
+def test_cluster_scoring_edges(laq, case):
+    NL, Bt, Hq, Hkv, D, L, W, Wl, kernel, B, lens = case
+    q, k, v = rand_inputs(NL, Bt, Hq, Hkv, D, L, W, seed=L + D + W, kscale=1.5)
+    if lens is not None:
+        for b, Lb in enumerate(lens):
+            k[:, b, :, Lb:] = float("nan")
+    compare_all_units(laq, q, k, v, W, kernel, B, local_window=Wl, seq_lens=lens)
+
+
+@pytest.mark.parametrize("W", [1, 3, 6, 16])
+def test_cluster_scoring_per_head(laq, W):
+    # heads of any length; W = 16 ends inside a group of eight rows only at its end
+    q, k, v = rand_inputs(1, 1, 8, 2, 128, 1300, W, seed=W, kscale=1.5)
+    for mode in (1, 2):
+        compare_all_units(laq, q, k, v, W, 7, 80, group_mode=mode)
+
+
+def test_cluster_scoring_sums_that_overflow(laq):
+    # Every warp takes the logits of its first key as reference. Here those lie 120 nats below the
+    # largest key, so the sums of a warp overflow and are taken again from the true maximum.
+    NL, Bt, Hq, Hkv, D, L, W, kernel, B = 1, 1, 4, 1, 128, 1100, 4, 7, 90
+    q, k, v = rand_inputs(NL, Bt, Hq, Hkv, D, L, W, seed=17)
+    q[..., 0] = 12.0
+    k[..., 0] = 0.0
+    k[:, :, :, ::32, 0] = -56.0                    # logit -59
+    for j in (5, 300, 700):
+        k[:, :, :, j, 0] = 56.0                    # logit +59
+    err, _ = compare_all_units(laq, q, k, v, W, kernel, B)
+    assert err < SCORE_RTOL
+    out = laq.evict(q.cuda(), k.cuda(), v.cuda(), B, pool_kernel=kernel)
+    assert {5, 300, 700} <= set(out["idx"][0, 0, 0].tolist())
+    assert np.isfinite(out["k_out"].float().cpu().numpy()).all()
