@@ -1,6 +1,8 @@
 // Step 4 (average or maximum pooling of the column sums) and step 5 (Eq. 4's ArgSort(...)[:B]: per-unit
 // top-k by radix select on the fp32 bit patterns, ties to the lower position, ascending output
 // followed by the retained tail).
+#include <atomic>
+
 #include "laq_internal.cuh"
 
 namespace laq {
@@ -11,19 +13,28 @@ constexpr int kSelWarps = kSelThreads / 32;
 
 // Geometry shared by the kernels below. Ls_full = L - R is the row length of the score tensor;
 // a unit whose prompt is shorter (per-prompt lengths) scores only its first Lb - R positions.
+// The tables are 5 KB of kernel parameters, which every launch has to carry: calls with neither
+// per-prompt lengths nor per-layer budgets take the kernels without them.
 struct SelGeom {
   int Ls_full, R, B, Bt, Hkv;
+};
+struct SelGeomTables : SelGeom {
   SeqLens sl;
   LayerBudgets lb;
 };
-__device__ __forceinline__ int unit_scored(const SelGeom& g, int64_t u) {
+__device__ __forceinline__ int unit_scored(const SelGeom& g, int64_t u) { return g.Ls_full; }
+__device__ __forceinline__ int unit_scored(const SelGeomTables& g, int64_t u) {
   return unit_len(g.sl, (int)((u / g.Hkv) % g.Bt), g.Ls_full + g.R) - g.R;
 }
 // Slots unit u selects (its budget without the tail) and where its row of kept positions starts.
-__device__ __forceinline__ int unit_kb(const SelGeom& g, int64_t u) {
+__device__ __forceinline__ int unit_kb(const SelGeom& g, int64_t u) { return g.B - g.R; }
+__device__ __forceinline__ int unit_kb(const SelGeomTables& g, int64_t u) {
   return unit_budget(g.lb, u, g.Bt * g.Hkv, g.B) - g.R;
 }
 __device__ __forceinline__ int32_t* unit_out(const SelGeom& g, int32_t* idx, int64_t u) {
+  return idx + u * (int64_t)g.B;
+}
+__device__ __forceinline__ int32_t* unit_out(const SelGeomTables& g, int32_t* idx, int64_t u) {
   return idx + unit_out_row(g.lb, u, g.Bt * g.Hkv, g.B);
 }
 
@@ -48,15 +59,54 @@ __device__ __forceinline__ float pool_at(const float* c, int j, int h, int Ls, f
   return acc * inv_k;
 }
 
-__global__ void pool_kernel(const float* __restrict__ colsum, int L_pad, float* __restrict__ pooled,
-                            int kpool, float inv_k, int pool_max, int64_t u0,
-                            const __grid_constant__ SelGeom g) {
+// Four consecutive positions per thread: three 16-byte loads (rows of column sums are 512-byte aligned)
+// hold every tap of a pooling kernel of up to nine. kPool: pooling kernel at compile time, 0 = kpool,
+// one load per tap. kVec: the score rows allow 16-byte stores.
+// Bound: HBM. 256 units of 32736 scores: 68 us with one position and a load per tap and thread.
+template <int kPool, bool kVec, class Geom>
+__global__ void __launch_bounds__(256)
+pool_kernel(const float* __restrict__ colsum, int L_pad, float* __restrict__ pooled, int kpool, float inv_k,
+            int pool_max, int64_t u0, const __grid_constant__ Geom g) {
   const int64_t u = u0 + blockIdx.y;
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
   if (j >= g.Ls_full) return;
   const int Ls = unit_scored(g, u);
-  pooled[u * g.Ls_full + j] =
-      j < Ls ? pool_at(colsum + u * L_pad, j, kpool / 2, Ls, inv_k, pool_max) : 0.f;
+  const float* c = colsum + u * L_pad;
+  float r[4];
+  if constexpr (kPool == 0) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) r[i] = j + i < Ls ? pool_at(c, j + i, kpool / 2, Ls, inv_k, pool_max) : 0.f;
+  } else {
+    constexpr int h = kPool / 2;
+    static_assert(h <= 4, "one vector of halo");
+    const float fill = pool_max ? __int_as_float(0xff800000) : 0.f;
+    float x[12];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int p = j - 4 + 4 * k;
+      float4 v = make_float4(fill, fill, fill, fill);
+      if (p >= 0 && p < Ls) v = *reinterpret_cast<const float4*>(c + p);  // (rows are padded to 128)
+      x[4 * k] = v.x;
+      x[4 * k + 1] = p + 1 < Ls ? v.y : fill;
+      x[4 * k + 2] = p + 2 < Ls ? v.z : fill;
+      x[4 * k + 3] = p + 3 < Ls ? v.w : fill;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float acc = pool_max ? x[4 + i] : 0.f;
+#pragma unroll
+      for (int t = -h; t <= h; ++t) acc = pool_max ? fmaxf(acc, x[4 + i + t]) : acc + x[4 + i + t];
+      r[i] = j + i < Ls ? (pool_max ? acc : acc * inv_k) : 0.f;
+    }
+  }
+  float* dst = pooled + u * (int64_t)g.Ls_full + j;
+  if (kVec) {
+    *reinterpret_cast<float4*>(dst) = make_float4(r[0], r[1], r[2], r[3]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (j + i < g.Ls_full) dst[i] = r[i];
+  }
 }
 
 // Order-preserving map from fp32 bits to uint32 (larger float <=> larger key).
@@ -165,48 +215,32 @@ __device__ __forceinline__ void select_unit(const float* p, int32_t* out, int Ls
   for (int t = tid; t < R; t += kSelThreads) out[Kb + t] = Ls + t;
 }
 
-// Step 5 alone: scores of unit blockIdx.x in global memory.
+// Step 5 alone, for units too long for the registers of two CTAs: scores of unit blockIdx.x in global
+// memory.
 __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* __restrict__ pooled,
                                                              int32_t* __restrict__ idx,
-                                                             const __grid_constant__ SelGeom g) {
+                                                             const __grid_constant__ SelGeomTables g) {
   const int64_t u = blockIdx.x;
   select_unit(pooled + u * (int64_t)g.Ls_full, unit_out(g, idx, u), unit_scored(g, u), unit_kb(g, u), g.R);
 }
 
-// Steps 4 and 5 in one pass over the column sums: the block pools its unit's scores into shared
-// memory (and into `pooled_out` if the caller wants them), then selects from there, so that the
-// radix passes never go back to global memory. The pooling arithmetic is that of pool_kernel.
-__global__ void __launch_bounds__(kSelThreads) pool_select_kernel(const float* __restrict__ colsum,
-                                                                  int L_pad, float* pooled_out,
-                                                                  int32_t* __restrict__ idx, int kpool,
-                                                                  float inv_k, int pool_max,
-                                                                  const __grid_constant__ SelGeom g) {
-  extern __shared__ float s_pooled[];
-  const int64_t u = blockIdx.x;
-  const float* c = colsum + u * (int64_t)L_pad;
-  const int h = kpool / 2;
-  const int Ls = unit_scored(g, u);
-  for (int j = threadIdx.x; j < g.Ls_full; j += kSelThreads) {
-    const float pj = j < Ls ? pool_at(c, j, h, Ls, inv_k, pool_max) : 0.f;
-    if (j < Ls) s_pooled[j] = pj;
-    if (pooled_out) pooled_out[u * (int64_t)g.Ls_full + j] = pj;
-  }
-  __syncthreads();
-  select_unit(s_pooled, unit_out(g, idx, u), Ls, unit_kb(g, u), g.R);
-}
-
-// Steps 4 and 5 for units of at most kRegItems * 1024 scored positions, with the unit's pooled
-// scores held in registers (kRegItems = 32 per thread) instead of memory. Warp w owns the
-// contiguous positions [1024 w, 1024 w + 1024), lane-strided, which is also the order the kept
-// positions are written in.
-// The key of the Kb-th largest score is found bit by bit from the top, on bit planes: each thread
-// transposes its 32 keys into 32 words (word b holds bit b of every key), so that one step is an
-// AND and a population count per thread plus one block-wide sum -- no atomics, no memory passes.
-// `alive` marks the keys that agree with the threshold's bits so far; if the alive keys with the
-// current bit set, together with the keys already known to lie above, reach Kb, the bit is 1 and
-// only those stay alive; otherwise the bit is 0 and they join the keys above.
+// Steps 4 and 5 with the unit's scores held in registers. Thread t owns the consecutive positions
+// [kItems t, kItems t + kItems), so kept positions leave in ascending order after one block-wide scan.
+// The key of the Kb-th largest score is found from the top, two bits per step: `alive` marks a
+// thread's keys that agree with the threshold's bits so far, and three block-wide counts (alive keys
+// whose next bits are 11, 10, 01) tell which of the four go on and which lie above. The search ends
+// as soon as the alive keys are exactly as many as are still wanted (for scores without ties, after
+// about two thirds of the bits).
+// kItems = 32: the keys are transposed into bit planes (word b holds bit b of all 32), so that a step
+// is a handful of ANDs and population counts. kItems = 8, for a few short units, where nothing but the
+// length of the dependent chain counts: four times the threads, bits taken from the keys one by one.
+// Bound: issue slots (B200, 1024 units of 32736 scores: about 40 instructions per score; the layout
+// with lane-strided positions, 7 shared-memory reads per pooled score, 32 one-bit steps and a ballot
+// per position took 70).
 // The pooling arithmetic is that of pool_kernel, so the scores are bit-identical to laq_score's.
 constexpr int kRegItems = 32;
+constexpr int kMaxSelWarps = 32;
+constexpr int kCopy = -1;  // kPool: the scores are given, no pooling
 
 // In-register transpose of a 32 x 32 bit matrix: on return bit i of a[b] is bit b of the old a[i].
 __device__ __forceinline__ void transpose32(uint32_t (&a)[32]) {
@@ -225,16 +259,13 @@ __device__ __forceinline__ void transpose32(uint32_t (&a)[32]) {
   }
 }
 
-// kPoolStatic > 0 fixes the pooling kernel at compile time (unrolled taps); 0 takes it from `kpool`.
-// kThreads: block size (128 .. 1024); a unit of up to 32 * kThreads scored positions takes the
-// smallest one, so that several blocks of short units share an SM.
 // kPair: a unit of up to 65536 scored positions is taken by a cluster of two 1024-thread CTAs,
 // CTA r holding positions [32768 r, 32768 r + 32768) in registers as before. What the threshold
-// search needs from the other half is one count per bit step, read from the peer's shared memory
+// search needs from the other half is its counts of each step, read from the peer's shared memory
 // after a cluster barrier; the kept positions of the second half are written behind those of the
 // first. Both CTAs execute the same barriers whatever their data, so neither can be left waiting.
 constexpr int kPairHalf = kRegItems * 1024;  // positions per CTA of a pair
-constexpr int kPairHalo = 4;                 // staged positions on either side of a half (>= kpool / 2)
+constexpr int kHalo = 32;                    // staged positions on either side of a CTA's own
 
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -248,147 +279,234 @@ __device__ __forceinline__ uint32_t ld_peer_u32(const uint32_t* p, uint32_t rank
   return v;
 }
 
-template <int kPoolStatic, int kThreads, bool kPair>
-__global__ void __launch_bounds__(kThreads, 1024 / kThreads) pool_select_reg_kernel(
-    const float* __restrict__ colsum, int L_pad, float* pooled_out, int32_t* __restrict__ idx,
-    int kpool, float inv_k, int pool_max, const __grid_constant__ SelGeom g) {
-  constexpr int kWarps = kThreads / 32;
-  __shared__ uint32_t s_cnt[2][kWarps];
-  __shared__ uint32_t s_gt[kWarps], s_eq[kWarps];
-  __shared__ uint32_t s_x[2], s_tot[2];  // pair: this CTA's count of the current bit step; its totals
-  extern __shared__ __align__(16) float s_c[];  // the unit's column sums, [0, Ls) rounded up to 4
+struct SelArgs {
+  const float* src;   // column sums, or the scores themselves (kCopy)
+  int64_t src_row;    // floats per unit in src
+  float* pooled_out;  // may be NULL
+  int32_t* idx;
+  int kpool, pool_max;
+  float inv_k;
+};
+
+// Shared memory holds the source from kHalo positions before the CTA's first to kHalo behind its last,
+// every 32 floats followed by 4 unused ones: a thread's 16-byte reads of its own 32 floats then hit
+// the banks of its neighbours' once.
+__device__ __forceinline__ int staged_at(int i) { return i + ((i >> 5) << 2); }
+inline size_t staged_floats(int n) { return (size_t)(n + 2 * kHalo + 31) / 32 * 36; }
+
+// kPool: pooling kernel at compile time (1, 3, 5, 7), 0 = args.kpool, kCopy.
+template <int kPool, int kItems, bool kPair, class Geom>
+__global__ void __launch_bounds__(1024, 1)
+pool_select_reg_kernel(const __grid_constant__ SelArgs args, const __grid_constant__ Geom g) {
+  __shared__ uint32_t s_cnt[2][2][kMaxSelWarps];
+  __shared__ uint32_t s_scan[kMaxSelWarps];
+  __shared__ uint32_t s_x[2][2], s_tot;  // pair: this CTA's counts of the current step; its totals
+  extern __shared__ __align__(16) float s_c[];
+  const int n_threads = blockDim.x, n_warps = n_threads >> 5;
   const uint32_t rank = kPair ? (blockIdx.x & 1u) : 0u;  // cluster of (2, 1, 1): rank = blockIdx.x % 2
   const int64_t u = kPair ? (int64_t)(blockIdx.x >> 1) : (int64_t)blockIdx.x;
   const int Ls = unit_scored(g, u), Kb = unit_kb(g, u), R = g.R;
-  int32_t* out = unit_out(g, idx, u);
+  int32_t* out = unit_out(g, args.idx, u);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int pos0 = kPair ? (int)rank * kPairHalf : 0;  // first position this CTA holds
-  // One coalesced pass brings the column sums on chip (rows are 512-byte aligned and padded to
-  // a multiple of 128 floats); the pooling taps then read shared memory instead of L1/L2.
-  // A CTA of a pair stages its half and a halo of kPairHalo positions on either side.
-  const int c_lo = kPair ? max(0, pos0 - kPairHalo) : 0;
-  const int c_hi = kPair ? min(Ls, pos0 + kPairHalf + kPairHalo) : Ls;
+  const int n_own = n_threads * kItems;
+
+  // ---- stage: positions that do not exist count nothing in a sum and lose every maximum
+  const float fill = kPool != kCopy && args.pool_max ? __int_as_float(0xff800000) : 0.f;
+  const float* src = args.src + u * args.src_row;
   {
-    const float4* src = reinterpret_cast<const float4*>(colsum + u * (int64_t)L_pad + c_lo);
-    float4* dst = reinterpret_cast<float4*>(s_c);
-    const int n4 = (max(0, c_hi - c_lo) + 3) >> 2;
-#pragma unroll 8
-    for (int k = tid; k < n4; k += kThreads) dst[k] = __ldcs(src + k);
+    const int n4 = (min(n_own, max(0, Ls - pos0)) + 2 * kHalo + 3) >> 2;  // what any thread reads
+    const float* from = src + pos0 - kHalo;
+    const bool aligned = kPool != kCopy;  // rows of column sums are 512-byte aligned
+#pragma unroll 4
+    for (int i = tid; i < n4; i += n_threads) {
+      const int p = pos0 - kHalo + 4 * i;
+      float4 v = make_float4(fill, fill, fill, fill);
+      if (aligned && p >= 0 && p + 4 <= Ls) {
+        v = __ldcs(reinterpret_cast<const float4*>(from) + i);
+      } else if (p >= 0) {
+        if (p < Ls) v.x = __ldcs(from + 4 * i);
+        if (p + 1 < Ls) v.y = __ldcs(from + 4 * i + 1);
+        if (p + 2 < Ls) v.z = __ldcs(from + 4 * i + 2);
+        if (p + 3 < Ls) v.w = __ldcs(from + 4 * i + 3);
+      }
+      *reinterpret_cast<float4*>(s_c + staged_at(4 * i)) = v;
+    }
   }
   __syncthreads();
-  const float* c = s_c - c_lo;  // indexed by position
-  const int base = pos0 + warp * (kRegItems * 32) + lane;
-  const int h = (kPoolStatic > 0 ? kPoolStatic : kpool) / 2;
 
-  uint32_t w[kRegItems];  // first the keys, then their bit planes
-  uint32_t alive = 0u;    // bit `it` set: item `it` of this thread is a real position
+  // ---- pool: keys of this thread's positions
+  const int own = tid * kItems, base = pos0 + own;
+  const int n_real = min(kItems, max(0, Ls - base));
+  uint32_t w[kItems];
+  if (kPool == 0 || kPool == kCopy) {
+    const int h = args.kpool / 2;
 #pragma unroll
-  for (int it = 0; it < kRegItems; ++it) {
-    const int j = base + it * 32;
-    uint32_t key = 0u;
-    if (j < Ls) {
-      float pj;
-      if (kPoolStatic > 0 && j >= h && j + h < Ls) {
-        // interior position, window unrolled
-        if (pool_max) {
-          pj = c[j];
-#pragma unroll
-          for (int t = -(kPoolStatic / 2); t <= kPoolStatic / 2; ++t) pj = fmaxf(pj, c[j + t]);
+    for (int k = 0; k < kItems; ++k) {
+      const int i = kHalo + own + k;
+      float pj = s_c[staged_at(i)];
+      if (kPool == 0 && k < n_real) {
+        if (h <= kHalo) {
+          if (args.pool_max) {
+            for (int t = -h; t <= h; ++t) pj = fmaxf(pj, s_c[staged_at(i + t)]);
+          } else {
+            float acc = 0.f;
+            for (int t = -h; t <= h; ++t) acc += s_c[staged_at(i + t)];
+            pj = acc * args.inv_k;
+          }
         } else {
-          float acc = 0.f;
-#pragma unroll
-          for (int t = -(kPoolStatic / 2); t <= kPoolStatic / 2; ++t) acc += c[j + t];
-          pj = acc * inv_k;
+          pj = pool_at(src, base + k, h, Ls, args.inv_k, args.pool_max);
         }
-      } else {
-        pj = pool_at(c, j, h, Ls, inv_k, pool_max);
       }
-      if (pooled_out) pooled_out[u * (int64_t)g.Ls_full + j] = pj;
-      key = order_key(pj);
-      alive |= 1u << it;
-    } else if (pooled_out && j < g.Ls_full) {
-      pooled_out[u * (int64_t)g.Ls_full + j] = 0.f;  // beyond a shorter prompt's scored positions
+      w[k] = __float_as_uint(pj);
     }
-    w[it] = key;
-  }
-  // w[i] bit b = bit b of key i  ->  w[b] bit i = bit b of key i
-  transpose32(w);
-
-  uint32_t above_mask = 0u;  // items known to lie above the threshold
-  uint32_t above = 0u;       // their number in the whole block
-  uint32_t theta = 0u;
+  } else {
+    constexpr int h = kPool > 0 ? kPool / 2 : 0;
+    static_assert(h <= 4, "one vector of halo");
+    const float4* row = reinterpret_cast<const float4*>(s_c);
+    float x[kItems + 8];  // [own - 4, own + kItems + 4)
 #pragma unroll
-  for (int bit = 31; bit >= 0; --bit) {
-    const uint32_t ones = w[bit] & alive;
-    const uint32_t n_warp = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(ones));
-    uint32_t* slot = s_cnt[bit & 1];
-    if (lane == 0) slot[warp] = n_warp;
-    __syncthreads();
-    uint32_t n = __reduce_add_sync(0xffffffffu, lane < kWarps ? slot[lane] : 0u);
-    if (kPair) {
-      // add the other half's count of this step (the two slots alternate: a slot is rewritten
-      // only after the peer has passed the next barrier, i.e. after it has read it)
-      if (tid == 0) s_x[bit & 1] = n;
-      cluster_sync_all();
-      n += ld_peer_u32(&s_x[bit & 1], rank ^ 1u);
+    for (int k = 0; k < kItems / 4 + 2; ++k) {
+      const float4 v = row[staged_at(kHalo + own - 4 + 4 * k) >> 2];
+      x[4 * k] = v.x; x[4 * k + 1] = v.y; x[4 * k + 2] = v.z; x[4 * k + 3] = v.w;
     }
-    if (above + n >= (uint32_t)Kb) {
-      theta |= 1u << bit;
-      alive = ones;
+    if (args.pool_max) {
+#pragma unroll
+      for (int k = 0; k < kItems; ++k) {
+        float m = x[4 + k];
+#pragma unroll
+        for (int t = -h; t <= h; ++t) m = fmaxf(m, x[4 + k + t]);
+        w[k] = __float_as_uint(m);
+      }
     } else {
-      above += n;
-      above_mask |= ones;
-      alive ^= ones;
+#pragma unroll
+      for (int k = 0; k < kItems; ++k) {
+        float acc = 0.f;
+#pragma unroll
+        for (int t = -h; t <= h; ++t) acc += x[4 + k + t];
+        w[k] = __float_as_uint(acc * args.inv_k);
+      }
     }
   }
-  // `alive` now marks the items whose key equals theta, the key of the Kb-th largest score;
-  // `need` of them are kept (the lowest positions first), with all `above` items
+  if (args.pooled_out) {  // through shared memory, so that the stores are coalesced
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) s_c[staged_at(kHalo + own + k)] = k < n_real ? __uint_as_float(w[k]) : 0.f;
+    __syncthreads();
+    float* dst = args.pooled_out + u * (int64_t)g.Ls_full + pos0;
+    for (int i = tid; i < min(n_own, g.Ls_full - pos0); i += n_threads) dst[i] = s_c[staged_at(kHalo + i)];
+  }
+#pragma unroll
+  for (int k = 0; k < kItems; ++k) w[k] = order_key(__uint_as_float(w[k]));
+  if constexpr (kItems == 32) transpose32(w);  // w[i] bit b -> w[b] bit i
+
+  // ---- threshold
+  uint32_t alive = n_real >= 32 ? 0xffffffffu : (1u << n_real) - 1u;
+  uint32_t above_mask = 0u;  // items known to lie above the threshold
+  uint32_t above = 0u;       // their number in the whole unit
+  uint32_t n_alive = (uint32_t)Ls;
+#pragma unroll
+  for (int bit = 30; bit >= 0; bit -= 2) {
+    if (above + n_alive == (uint32_t)Kb) break;  // uniform: every alive item is wanted
+    uint32_t hi, lo;
+    if constexpr (kItems == 32) {
+      hi = w[bit + 1];
+      lo = w[bit];
+    } else {
+      hi = lo = 0u;
+#pragma unroll
+      for (int k = 0; k < kItems; ++k) {
+        hi |= ((w[k] >> (bit + 1)) & 1u) << k;
+        lo |= ((w[k] >> bit) & 1u) << k;
+      }
+    }
+    const uint32_t m3 = alive & hi & lo, m2 = alive & hi & ~lo, m1 = alive & ~hi & lo;
+    // per warp at most 1024 of each, per CTA 32768: two counts share a word
+    uint32_t n32 = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(m3) | ((uint32_t)__popc(m2) << 16));
+    uint32_t n1 = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(m1));
+    const int buf = (bit >> 1) & 1;
+    if (lane == 0) {
+      s_cnt[buf][0][warp] = n32;
+      s_cnt[buf][1][warp] = n1;
+    }
+    __syncthreads();
+    n32 = __reduce_add_sync(0xffffffffu, lane < n_warps ? s_cnt[buf][0][lane] : 0u);
+    n1 = __reduce_add_sync(0xffffffffu, lane < n_warps ? s_cnt[buf][1][lane] : 0u);
+    uint32_t n3 = n32 & 0xffffu, n2 = n32 >> 16;
+    if (kPair) {
+      // add the other half's counts of this step (the two slots alternate: a slot is rewritten
+      // only after the peer has passed the next barrier, i.e. after it has read it)
+      if (tid == 0) {
+        s_x[buf][0] = n32;
+        s_x[buf][1] = n1;
+      }
+      cluster_sync_all();
+      const uint32_t p32 = ld_peer_u32(&s_x[buf][0], rank ^ 1u);
+      n3 += p32 & 0xffffu;
+      n2 += p32 >> 16;
+      n1 += ld_peer_u32(&s_x[buf][1], rank ^ 1u);
+    }
+    const uint32_t want = (uint32_t)Kb - above;
+    if (n3 >= want) {
+      alive = m3;
+      n_alive = n3;
+    } else if (n3 + n2 >= want) {
+      above += n3;
+      above_mask |= m3;
+      alive = m2;
+      n_alive = n2;
+    } else if (n3 + n2 + n1 >= want) {
+      above += n3 + n2;
+      above_mask |= m3 | m2;
+      alive = m1;
+      n_alive = n1;
+    } else {
+      above += n3 + n2 + n1;
+      above_mask |= m3 | m2 | m1;
+      alive &= ~(hi | lo);
+      n_alive -= n3 + n2 + n1;
+    }
+  }
+  // `alive` now marks the items whose keys agree as far as they were looked at; `need` of them are
+  // kept (the lowest positions first), with all `above` items
   const uint32_t need = (uint32_t)Kb - above;
 
-  const uint32_t n_gt = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(above_mask));
-  const uint32_t n_eq = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(alive));
-  if (lane == 0) {
-    s_gt[warp] = n_gt;
-    s_eq[warp] = n_eq;
+  // ---- write the kept positions in ascending order: one scan of (above, alive) counts, 16 bits each
+  const uint32_t mine = (uint32_t)__popc(above_mask) | ((uint32_t)__popc(alive) << 16);
+  uint32_t scan = mine;
+#pragma unroll
+  for (int s = 1; s < 32; s <<= 1) {
+    const uint32_t v = __shfl_up_sync(0xffffffffu, scan, s);
+    if (lane >= s) scan += v;
   }
+  if (lane == 31) s_scan[warp] = scan;
   __syncthreads();
-  uint32_t gt_run = 0, eq_run = 0;
-  for (int ww = 0; ww < warp; ++ww) {
-    gt_run += s_gt[ww];
-    eq_run += s_eq[ww];
-  }
+  const uint32_t of_warp = lane < n_warps ? s_scan[lane] : 0u;
+  const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? of_warp : 0u) + scan - mine;
+  uint32_t gt = before & 0xffffu, eq = before >> 16;
   if (kPair) {
     // the second half writes behind the first: its running counts start from the first half's totals
-    if (tid == 0) {
-      uint32_t tg = 0, te = 0;
-      for (int ww = 0; ww < kWarps; ++ww) {
-        tg += s_gt[ww];
-        te += s_eq[ww];
-      }
-      s_tot[0] = tg;
-      s_tot[1] = te;
-    }
+    const uint32_t total = __reduce_add_sync(0xffffffffu, of_warp);
+    if (tid == 0) s_tot = total;
     cluster_sync_all();
     if (rank == 1u) {
-      gt_run += ld_peer_u32(&s_tot[0], 0u);
-      eq_run += ld_peer_u32(&s_tot[1], 0u);
+      const uint32_t t = ld_peer_u32(&s_tot, 0u);
+      gt += t & 0xffffu;
+      eq += t >> 16;
     }
   }
-  const uint32_t lt_mask = (1u << lane) - 1u;
-#pragma unroll
-  for (int it = 0; it < kRegItems; ++it) {
-    const bool gt = (above_mask >> it) & 1u;
-    const bool eq = (alive >> it) & 1u;
-    const uint32_t bg = __ballot_sync(0xffffffffu, gt);
-    const uint32_t be = __ballot_sync(0xffffffffu, eq);
-    const uint32_t gt_before = gt_run + __popc(bg & lt_mask);
-    const uint32_t eq_before = eq_run + __popc(be & lt_mask);
-    if (gt || (eq && eq_before < need)) out[gt_before + min(eq_before, need)] = base + it * 32;
-    gt_run += __popc(bg);
-    eq_run += __popc(be);
+  for (uint32_t m = above_mask | alive; m != 0u; m &= m - 1u) {
+    const int k = __ffs(m) - 1;
+    if ((above_mask >> k) & 1u) {
+      out[gt + min(eq, need)] = base + k;
+      ++gt;
+    } else {
+      if (eq < need) out[gt + eq] = base + k;
+      ++eq;
+    }
   }
   if (rank == 0u)
-    for (int t = tid; t < R; t += kThreads) out[Kb + t] = Ls + t;
+    for (int t = tid; t < R; t += n_threads) out[Kb + t] = Ls + t;
   if (kPair) cluster_sync_all();  // no CTA leaves while its peer may still read its shared memory
 }
 
@@ -423,31 +541,148 @@ laq_status group_max_launch(const Dims& d, const float* colsum_h, int L_pad, flo
   return cudaGetLastError() == cudaSuccess ? LAQ_OK : LAQ_ERR_CUDA;
 }
 
-static SelGeom sel_geom(const Dims& d) {
-  SelGeom g;
-  g.Ls_full = d.Ls; g.R = d.R; g.B = d.B; g.Bt = d.Bt; g.Hkv = d.Hkv;
+static void fill_geom(const Dims& d, SelGeom* g) {
+  g->Ls_full = d.Ls; g->R = d.R; g->B = d.B; g->Bt = d.Bt; g->Hkv = d.Hkv;
+}
+static SelGeomTables geom_tables(const Dims& d) {
+  SelGeomTables g;
+  fill_geom(d, &g);
   g.sl = d.sl;
   g.lb = d.lb;
   return g;
 }
+static SelGeom geom_plain(const Dims& d) {
+  SelGeom g;
+  fill_geom(d, &g);
+  return g;
+}
+static bool has_tables(const Dims& d) { return d.sl.n > 0 || d.lb.n > 0; }
+
+namespace {
+
+template <bool kVec, class Geom>
+void launch_pool(dim3 grid, cudaStream_t stream, const Dims& d, const float* colsum, int L_pad, float* pooled,
+                 int64_t u0, const Geom& g) {
+  const float inv_k = 1.0f / (float)d.kpool;
+#define LAQ_POOL(K) \
+  pool_kernel<K, kVec, Geom><<<grid, 256, 0, stream>>>(colsum, L_pad, pooled, d.kpool, inv_k, d.pool_max, u0, g)
+  switch (d.kpool) {
+    case 1: LAQ_POOL(1); break;
+    case 3: LAQ_POOL(3); break;
+    case 5: LAQ_POOL(5); break;
+    case 7: LAQ_POOL(7); break;
+    default: LAQ_POOL(0); break;
+  }
+#undef LAQ_POOL
+}
+
+// Shared memory opt-in of a kernel: a per-device attribute, set once per device and kernel.
+template <class K>
+bool opt_in(K kernel, std::atomic<uint64_t>& devices) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  if (dev < 64 && ((devices.load(std::memory_order_acquire) >> dev) & 1u)) return true;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(staged_floats(kPairHalf) * sizeof(float))) != cudaSuccess)
+    return false;
+  if (dev < 64) devices.fetch_or(1ull << dev, std::memory_order_release);
+  return true;
+}
+
+template <int kPool, int kItems, bool kPair, class Geom>
+bool launch_select(unsigned units, int threads, cudaStream_t stream, const SelArgs& args, const Geom& g) {
+  static std::atomic<uint64_t> devices{0};
+  if (!opt_in(pool_select_reg_kernel<kPool, kItems, kPair, Geom>, devices)) return false;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kPair ? 2 * units : units);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = staged_floats(threads * kItems) * sizeof(float);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = 2;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  if (kPair) {
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+  }
+  return cudaLaunchKernelEx(&cfg, pool_select_reg_kernel<kPool, kItems, kPair, Geom>, args, g) == cudaSuccess;
+}
+
+// Which of the kernels takes units of Ls scores: up to 32768 one CTA with 32 scores per thread, up to
+// 65536 a pair of CTAs. Where the units are so few and short that every one has an SM to itself and
+// waits for its own chain of steps only, 8 scores per thread (one unit of 1016: 14.4 us with 128
+// threads).
+template <int kPool, class Geom>
+bool launch_select_sized(const Dims& d, cudaStream_t stream, const SelArgs& args, const Geom& g) {
+  const unsigned units = (unsigned)d.U;
+  if (d.Ls > kPairHalf) return launch_select<kPool, 32, true, Geom>(units, 1024, stream, args, g);
+  if (d.U <= 148 && d.Ls <= 8 * 1024)
+    return launch_select<kPool, 8, false, Geom>(units, ((d.Ls + 7) / 8 + 31) / 32 * 32, stream, args, g);
+  return launch_select<kPool, 32, false, Geom>(units, ((d.Ls + 31) / 32 + 31) / 32 * 32, stream, args, g);
+}
+
+// pool: 0 the scores are given, 1 pool them first.
+template <class Geom>
+bool launch_select_pooled(const Dims& d, bool pool, cudaStream_t stream, const SelArgs& args, const Geom& g) {
+  if (!pool) return launch_select_sized<kCopy, Geom>(d, stream, args, g);
+  switch (d.kpool) {
+    case 1: return launch_select_sized<1, Geom>(d, stream, args, g);
+    case 3: return launch_select_sized<3, Geom>(d, stream, args, g);
+    case 5: return launch_select_sized<5, Geom>(d, stream, args, g);
+    case 7: return launch_select_sized<7, Geom>(d, stream, args, g);
+    default: return launch_select_sized<0, Geom>(d, stream, args, g);
+  }
+}
+
+}  // namespace
 
 laq_status pool_launch(const Dims& d, const float* colsum, int L_pad, float* pooled,
                        cudaStream_t stream, int* launches) {
-  const SelGeom g = sel_geom(d);
+  const bool vec = d.Ls % 4 == 0 && (reinterpret_cast<uintptr_t>(pooled) & 15u) == 0;
   // grid.y limit: launch in slabs of units
   for (int64_t u0 = 0; u0 < d.U; u0 += 65535) {
     const unsigned nu = (unsigned)((d.U - u0 < 65535) ? d.U - u0 : 65535);
-    pool_kernel<<<dim3((d.Ls + 255) / 256, nu), 256, 0, stream>>>(
-        colsum, L_pad, pooled, d.kpool, 1.0f / (float)d.kpool, d.pool_max, u0, g);
+    const dim3 grid((d.Ls + 1023) / 1024, nu);
+    if (has_tables(d)) {
+      const SelGeomTables g = geom_tables(d);
+      if (vec) launch_pool<true>(grid, stream, d, colsum, L_pad, pooled, u0, g);
+      else launch_pool<false>(grid, stream, d, colsum, L_pad, pooled, u0, g);
+    } else {
+      const SelGeom g = geom_plain(d);
+      if (vec) launch_pool<true>(grid, stream, d, colsum, L_pad, pooled, u0, g);
+      else launch_pool<false>(grid, stream, d, colsum, L_pad, pooled, u0, g);
+    }
     *launches += 1;
   }
   return cudaGetLastError() == cudaSuccess ? LAQ_OK : LAQ_ERR_CUDA;
 }
 
+// Units that the register kernels take.
+static bool fits_registers(const Dims& d) { return d.Ls <= 2 * kPairHalf && d.U <= 0x3fffffff; }
+
+static laq_status select_reg_launch(const Dims& d, bool pool, const float* src, int64_t src_row, float* pooled_out,
+                                    int32_t* idx, cudaStream_t stream, int* launches) {
+  SelArgs args;
+  args.src = src;
+  args.src_row = src_row;
+  args.pooled_out = pooled_out;
+  args.idx = idx;
+  args.kpool = pool ? d.kpool : 1;
+  args.pool_max = pool ? d.pool_max : 0;
+  args.inv_k = 1.0f / (float)args.kpool;
+  const bool ok = has_tables(d) ? launch_select_pooled(d, pool, stream, args, geom_tables(d))
+                                : launch_select_pooled(d, pool, stream, args, geom_plain(d));
+  if (!ok) return LAQ_ERR_CUDA;
+  *launches += 1;
+  return LAQ_OK;
+}
+
 laq_status select_launch(const Dims& d, const float* pooled, int32_t* idx, cudaStream_t stream,
                          int* launches) {
   if (d.U > 0x7fffffff) return LAQ_ERR_UNSUPPORTED;
-  select_kernel<<<(unsigned)d.U, kSelThreads, 0, stream>>>(pooled, idx, sel_geom(d));
+  if (fits_registers(d)) return select_reg_launch(d, false, pooled, d.Ls, nullptr, idx, stream, launches);
+  select_kernel<<<(unsigned)d.U, kSelThreads, 0, stream>>>(pooled, idx, geom_tables(d));
   *launches += 1;
   return cudaGetLastError() == cudaSuccess ? LAQ_OK : LAQ_ERR_CUDA;
 }
@@ -455,89 +690,10 @@ laq_status select_launch(const Dims& d, const float* pooled, int32_t* idx, cudaS
 laq_status pool_select_launch(const Dims& d, const float* colsum, int L_pad, float* pooled_out,
                               int32_t* idx, cudaStream_t stream, int* launches, bool* done) {
   *done = false;
-  if (d.U > 0x7fffffff) return LAQ_OK;
-  const SelGeom g = sel_geom(d);
-  if (d.Ls <= kRegItems * kSelThreads) {
-    const float inv_k = 1.0f / (float)d.kpool;
-    const unsigned grid = (unsigned)d.U;
-    const size_t smem_c = (size_t)((d.Ls + 3) / 4 * 4) * sizeof(float);
-    // the smallest block whose 32 positions per thread cover the unit
-    const int threads = d.Ls <= 32 * 128 ? 128 : (d.Ls <= 32 * 256 ? 256 : (d.Ls <= 32 * 512 ? 512 : 1024));
-#define LAQ_LAUNCH_POOL_SELECT_T(KP, T)                                                               \
-  {                                                                                                   \
-    if (cudaFuncSetAttribute(pool_select_reg_kernel<KP, T, false>,                                    \
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_c) != cudaSuccess) \
-      return LAQ_ERR_CUDA;                                                                            \
-    pool_select_reg_kernel<KP, T, false><<<grid, T, smem_c, stream>>>(colsum, L_pad, pooled_out, idx, \
-                                                                      d.kpool, inv_k, d.pool_max, g); \
-  }
-#define LAQ_LAUNCH_POOL_SELECT(KP)                     \
-  switch (threads) {                                   \
-    case 128: LAQ_LAUNCH_POOL_SELECT_T(KP, 128) break; \
-    case 256: LAQ_LAUNCH_POOL_SELECT_T(KP, 256) break; \
-    case 512: LAQ_LAUNCH_POOL_SELECT_T(KP, 512) break; \
-    default: LAQ_LAUNCH_POOL_SELECT_T(KP, 1024) break; \
-  }
-    switch (d.kpool) {
-      case 1: LAQ_LAUNCH_POOL_SELECT(1); break;
-      case 3: LAQ_LAUNCH_POOL_SELECT(3); break;
-      case 5: LAQ_LAUNCH_POOL_SELECT(5); break;
-      case 7: LAQ_LAUNCH_POOL_SELECT(7); break;
-      default: LAQ_LAUNCH_POOL_SELECT(0); break;
-    }
-#undef LAQ_LAUNCH_POOL_SELECT
-#undef LAQ_LAUNCH_POOL_SELECT_T
-    *launches += 1;
-    *done = true;
-    return cudaGetLastError() == cudaSuccess ? LAQ_OK : LAQ_ERR_CUDA;
-  }
-  if (d.Ls <= 2 * kPairHalf && d.kpool / 2 <= kPairHalo && d.U <= 0x3fffffff) {
-    // two CTAs per unit, as a cluster: each holds half of the positions in registers
-    const float inv_k = 1.0f / (float)d.kpool;
-    const size_t smem_c = (size_t)(kPairHalf + 2 * kPairHalo) * sizeof(float);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(2 * d.U));
-    cfg.blockDim = dim3(1024);
-    cfg.dynamicSmemBytes = smem_c;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = 2;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    int kpool = d.kpool, pool_max = d.pool_max;
-#define LAQ_LAUNCH_POOL_SELECT_PAIR(KP)                                                              \
-  {                                                                                                  \
-    if (cudaFuncSetAttribute(pool_select_reg_kernel<KP, 1024, true>,                                 \
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_c) != cudaSuccess || \
-        cudaLaunchKernelEx(&cfg, pool_select_reg_kernel<KP, 1024, true>, colsum, L_pad, pooled_out,  \
-                           idx, kpool, inv_k, pool_max, g) != cudaSuccess)                           \
-      return LAQ_ERR_CUDA;                                                                           \
-  }
-    switch (d.kpool) {
-      case 1: LAQ_LAUNCH_POOL_SELECT_PAIR(1); break;
-      case 3: LAQ_LAUNCH_POOL_SELECT_PAIR(3); break;
-      case 5: LAQ_LAUNCH_POOL_SELECT_PAIR(5); break;
-      case 7: LAQ_LAUNCH_POOL_SELECT_PAIR(7); break;
-      default: LAQ_LAUNCH_POOL_SELECT_PAIR(0); break;
-    }
-#undef LAQ_LAUNCH_POOL_SELECT_PAIR
-    *launches += 1;
-    *done = true;
-    return LAQ_OK;
-  }
-  const size_t smem = (size_t)d.Ls * sizeof(float);
-  if (smem > 200u * 1024u || d.U > 0x7fffffff) return LAQ_OK;  // the caller uses the two-kernel path
-  if (cudaFuncSetAttribute(pool_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem) != cudaSuccess)
-    return LAQ_ERR_CUDA;
-  pool_select_kernel<<<(unsigned)d.U, kSelThreads, smem, stream>>>(
-      colsum, L_pad, pooled_out, idx, d.kpool, 1.0f / (float)d.kpool, d.pool_max, g);
-  *launches += 1;
-  *done = true;
-  return cudaGetLastError() == cudaSuccess ? LAQ_OK : LAQ_ERR_CUDA;
+  if (!fits_registers(d)) return LAQ_OK;  // the caller uses the two-kernel path
+  const laq_status st = select_reg_launch(d, true, colsum, L_pad, pooled_out, idx, stream, launches);
+  *done = st == LAQ_OK;
+  return st;
 }
 
 }  // namespace laq
