@@ -1,6 +1,8 @@
 // Step 6: gathers the kept key/value rows into the dense compressed cache ("cache re-eviction
 // based on the given budget", Section 4.3). Pure 128-bit copies; each 16-byte vector of each
 // output row is one work item of a half-warp.
+#include <type_traits>
+
 #include "laq_internal.cuh"
 
 namespace laq {
@@ -19,7 +21,11 @@ struct CompactArgs {
   int Bt, Hkv, B, dv, L;
   int kv_div;  // unit head h reads KV head h / kv_div (1 unless every query head is a unit)
   int64_t u0;  // first unit of this launch (units are launched in slabs of at most 65535)
-  LayerBudgets lb;  // per-layer budgets: B is then the largest, and the outputs are one dense ragged pool
+};
+// With per-layer budgets B is the largest, and the outputs are one dense ragged pool. (The table is
+// 3 KB of kernel parameters; calls without it take the kernel without it.)
+struct CompactLayersArgs : CompactArgs {
+  LayerBudgets lb;
 };
 
 // grid (row groups, units), block 256 threads = 16 half-warps. A half-warp copies one 256-byte
@@ -29,23 +35,34 @@ struct CompactArgs {
 constexpr int kRowsInFlight = 4;
 constexpr int kRowsPerBlock = 16 * kRowsInFlight;
 
-__global__ void __launch_bounds__(256) compact_kernel(const __grid_constant__ CompactArgs a) {
+__device__ __forceinline__ int unit_rows(const CompactArgs& a, int64_t u) { return a.B; }
+__device__ __forceinline__ int unit_rows(const CompactLayersArgs& a, int64_t u) {
+  return unit_budget(a.lb, u, a.Bt * a.Hkv, a.B);
+}
+__device__ __forceinline__ int64_t first_row(const CompactArgs& a, int64_t u) { return u * (int64_t)a.B; }
+__device__ __forceinline__ int64_t first_row(const CompactLayersArgs& a, int64_t u) {
+  return unit_out_row(a.lb, u, a.Bt * a.Hkv, a.B);
+}
+
+template <class Args>
+__global__ void __launch_bounds__(256) compact_kernel(const __grid_constant__ Args a) {
+  constexpr bool kLayers = !std::is_same<Args, CompactArgs>::value;
   const int64_t u = a.u0 + blockIdx.y;
   const int h = (int)(u % a.Hkv);
   const int b = (int)((u / a.Hkv) % a.Bt);
   const int64_t layer = u / ((int64_t)a.Hkv * a.Bt);
   const int half_warp = threadIdx.x >> 4, c0 = threadIdx.x & 15;
   const int slot0 = blockIdx.x * kRowsPerBlock + half_warp;
-  const int B = unit_budget(a.lb, u, a.Bt * a.Hkv, a.B);
+  const int B = unit_rows(a, u);
   if (blockIdx.x * kRowsPerBlock >= B) return;  // a layer with a smaller budget (block-uniform)
-  const int64_t row = unit_out_row(a.lb, u, a.Bt * a.Hkv, a.B);
+  const int64_t row = first_row(a, u);
   const int32_t* idx = a.idx + row;
   const int h_src = h / a.kv_div;
   const uint4* kbase = a.k + layer * a.ks_layer + b * a.ks_batch + h_src * a.ks_head;
   const uint4* vbase = a.v + layer * a.vs_layer + b * a.vs_batch + h_src * a.vs_head;
-  const int64_t obase =
-      a.lb.n > 0 ? row * a.dv : layer * a.os_layer + b * a.os_batch + h * a.os_head;
-  const int64_t os_pos = a.lb.n > 0 ? a.dv : a.os_pos;
+  const int64_t obase = kLayers ? row * a.dv : layer * a.os_layer + b * a.os_batch + h * a.os_head;
+  const int64_t os_pos = kLayers ? a.dv : a.os_pos;
+  wait_for_predecessor();  // the positions, and whoever still reads what is overwritten here
   int32_t pos[kRowsInFlight];
 #pragma unroll
   for (int r = 0; r < kRowsInFlight; ++r) {
@@ -101,7 +118,7 @@ laq_status compact_launch(const laq_params& p, const Dims& d, const void* k, con
                           const int32_t* idx, void* k_out, void* v_out, cudaStream_t stream,
                           int* launches) {
   if (!k_out && !v_out) return LAQ_OK;
-  CompactArgs a;
+  CompactLayersArgs a;
   a.k = (const uint4*)k;
   a.v = (const uint4*)v;
   a.k_out = (uint4*)k_out;
@@ -116,14 +133,23 @@ laq_status compact_launch(const laq_params& p, const Dims& d, const void* k, con
   a.Bt = d.Bt; a.Hkv = d.Hkv; a.B = d.B; a.dv = d.D / 8; a.L = d.L;
   a.lb = d.lb;
   a.kv_div = d.kv_div > 0 ? d.kv_div : 1;
+  cudaLaunchAttribute attr;
+  programmatic_launch(&attr);
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(256);
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
   // units sit on grid.y, which holds at most 65535 blocks
   for (int64_t u0 = 0; u0 < d.U; u0 += 65535) {
     a.u0 = u0;
     const int64_t nu = d.U - u0 < 65535 ? d.U - u0 : 65535;
-    compact_kernel<<<dim3((unsigned)((d.B + kRowsPerBlock - 1) / kRowsPerBlock), (unsigned)nu), 256, 0,
-                     stream>>>(a);
+    cfg.gridDim = dim3((unsigned)((d.B + kRowsPerBlock - 1) / kRowsPerBlock), (unsigned)nu);
+    const CompactArgs& plain = a;
+    if ((d.lb.n > 0 ? cudaLaunchKernelEx(&cfg, compact_kernel<CompactLayersArgs>, a)
+                    : cudaLaunchKernelEx(&cfg, compact_kernel<CompactArgs>, plain)) != cudaSuccess)
+      return LAQ_ERR_CUDA;
     *launches += 1;
-    if (cudaGetLastError() != cudaSuccess) return LAQ_ERR_CUDA;
   }
   return LAQ_OK;
 }

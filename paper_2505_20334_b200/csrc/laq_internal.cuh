@@ -141,6 +141,18 @@ laq_status compact_launch(const laq_params& p, const Dims& d, const void* k, con
 laq_status streaming_launch(const Dims& d, int n_sink, int32_t* idx, cudaStream_t stream,
                             int* launches);
 
+// Programmatic dependent launch: a kernel launched with `attr` may start while the kernel before it in
+// the stream still runs; it has to call wait_for_predecessor() before it touches memory that one
+// writes (or reads, where it overwrites it). allow_successor() lets such a kernel start from here on.
+inline void programmatic_launch(cudaLaunchAttribute* attr) {
+  attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr->val.programmaticStreamSerializationAllowed = 1;
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void allow_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
+
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 }  // namespace laq

@@ -521,10 +521,19 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
                      const __grid_constant__ ClArgs a) {
   long long clk0 = 0;
   unsigned long long ns0 = 0;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    clk0 = clock64();
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(ns0));
+  if (threadIdx.x == 0) {
+    prefetch_tensor_map(&tmap_q);
+    prefetch_tensor_map(&tmap_k);
+    if (blockIdx.x == 0) {
+      clk0 = clock64();
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(ns0));
+      // The status word starts at OK. CTAs start in order and a wait runs out long after that, so
+      // no record of this launch is lost.
+      a.hdr[HDR_STATUS] = 0;
+      a.hdr[HDR_WHERE] = 0;
+    }
   }
+  allow_successor();
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // stages first: the swizzled layout needs 1024-byte aligned addresses
   const uint32_t smem_base = smem_u32(smem_raw);
@@ -848,7 +857,7 @@ laq_status score_cluster_launch(const laq_params& p, const Dims& d, const Worksp
   const int n_tiles = w.L_pad / TILE_KEYS, slots = 1 << a.slots_log2;
   // The cluster size: ceil(U / clusters) rounds of T tiles per CTA. Cycles as measured on B200: a tile
   // takes the arithmetic of both passes or the CTA's share of the HBM stream (3600 bytes per cycle, at
-  // most 30 per SM); a unit about 1000 more, and 2500 if its tiles leave no room for the next unit's. Large clusters
+  // most 30 per SM); a unit about 1600 more, and 2500 if its tiles leave no room for the next unit's. Large clusters
   // leave SMs idle (15 of 8 CTAs and 7 of 16 fit the 148), small ones fit fewer keys.
   // L 6007, 64 rows, 256 units: 102 us with 8 CTAs, 131 with 16; 64-dim heads, 32 rows, L 4096, 128
   // units: 26.1 / 24.6 / 27.0 us with 2 / 4 / 8.
@@ -859,7 +868,7 @@ laq_status score_cluster_launch(const laq_params& p, const Dims& d, const Worksp
     if (n < 1 || T > slots || C > n_tiles) continue;
     const double rounds = (double)((d.U + n - 1) / n);
     const double tile = fmax(200.0 + 20.0 * d.M, (double)(a.boxes * kBoxBytes) * fmax(n * C, 120.0) / 3600.0);
-    const double cost = rounds * (T * tile + (2 * T <= slots ? 1000.0 : 2500.0));
+    const double cost = rounds * (T * tile + (2 * T <= slots ? 1600.0 : 2500.0));
     if (best < 0 || cost < best_cost) {
       best = i;
       best_cost = cost;

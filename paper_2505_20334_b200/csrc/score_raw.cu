@@ -49,6 +49,7 @@ __global__ void __launch_bounds__(kRawThreads) score_raw_d128_kernel(
     const __nv_bfloat16* __restrict__ k, const float* __restrict__ qsum, float* __restrict__ colsum,
     int Bt, int Hkv, int L_alloc, int L_pad, float scale, int64_t s_layer, int64_t s_batch,
     int64_t s_head, int64_t s_pos, const __grid_constant__ SeqLens sl) {
+  allow_successor();
   const int64_t u = blockIdx.x;
   const int h = (int)(u % Hkv);
   const int64_t lb = u / Hkv;

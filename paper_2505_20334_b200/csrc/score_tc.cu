@@ -329,6 +329,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
     clk0 = clock64();
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(ns0));
   }
+  allow_successor();
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   Ctl* ctl = reinterpret_cast<Ctl*>(smem_raw);
   const uint32_t smem_base = smem_u32(smem_raw);

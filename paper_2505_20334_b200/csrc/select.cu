@@ -310,6 +310,8 @@ pool_select_reg_kernel(const __grid_constant__ SelArgs args, const __grid_consta
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int pos0 = kPair ? (int)rank * kPairHalf : 0;  // first position this CTA holds
   const int n_own = n_threads * kItems;
+  allow_successor();
+  wait_for_predecessor();
 
   // ---- stage: positions that do not exist count nothing in a sum and lose every maximum
   const float fill = kPool != kCopy && args.pool_max ? __int_as_float(0xff800000) : 0.f;
@@ -598,14 +600,13 @@ bool launch_select(unsigned units, int threads, cudaStream_t stream, const SelAr
   cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = staged_floats(threads * kItems) * sizeof(float);
   cfg.stream = stream;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = 2;
-  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-  if (kPair) {
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-  }
+  cudaLaunchAttribute attr[2];
+  programmatic_launch(&attr[0]);
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 2;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = kPair ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, pool_select_reg_kernel<kPool, kItems, kPair, Geom>, args, g) == cudaSuccess;
 }
 
