@@ -147,17 +147,15 @@ laq_status run_scoring(const laq_params* p, const Dims& d, const Workspace& w,
                               const void* q, const void* k, char* ws, cudaStream_t stream,
                               int* launches) {
   if (g_ev_begin && cudaEventRecord(g_ev_begin, stream) != cudaSuccess) return LAQ_ERR_CUDA;
-  bool done = false;
-  laq_status st = LAQ_OK;
-  if (!d.score_raw) st = score_cluster_launch(*p, d, w, q, k, ws, stream, launches, &done);
+  bool done = d.score_raw;
+  laq_status st = d.score_raw ? score_raw_launch(*p, d, w, q, k, ws, stream, launches)
+                              : score_cluster_launch(*p, d, w, q, k, ws, stream, launches, &done);
   if (st == LAQ_OK && !done) {
-    // header and unit counters are contiguous: one clear (the cluster kernel has none of the counters
-    // and sets its status word itself)
+    // header and unit counters are contiguous: one clear (the other kernels have no counters and set
+    // the header themselves)
     if (cudaMemsetAsync(ws + w.off_hdr, 0, w.off_part - w.off_hdr, stream) != cudaSuccess) return LAQ_ERR_CUDA;
-    st = d.score_raw ? score_raw_launch(*p, d, w, q, k, ws, stream, launches)
-         : use_tensor_core_path(d)
-             ? score_tc_launch(*p, d, w, q, k, ws, stream, launches)
-             : score_simt_launch(*p, d, w, q, k, ws, stream, launches);
+    st = use_tensor_core_path(d) ? score_tc_launch(*p, d, w, q, k, ws, stream, launches)
+                                 : score_simt_launch(*p, d, w, q, k, ws, stream, launches);
   }
   if (g_ev_end && cudaEventRecord(g_ev_end, stream) != cudaSuccess) return LAQ_ERR_CUDA;
   return st;

@@ -857,10 +857,11 @@ laq_status score_cluster_launch(const laq_params& p, const Dims& d, const Worksp
   const int n_tiles = w.L_pad / TILE_KEYS, slots = 1 << a.slots_log2;
   // The cluster size: ceil(U / clusters) rounds of T tiles per CTA. Cycles as measured on B200: a tile
   // takes the arithmetic of both passes or the CTA's share of the HBM stream (3600 bytes per cycle, at
-  // most 30 per SM); a unit about 1600 more, and 2500 if its tiles leave no room for the next unit's. Large clusters
-  // leave SMs idle (15 of 8 CTAs and 7 of 16 fit the 148), small ones fit fewer keys.
-  // L 6007, 64 rows, 256 units: 102 us with 8 CTAs, 131 with 16; 64-dim heads, 32 rows, L 4096, 128
-  // units: 26.1 / 24.6 / 27.0 us with 2 / 4 / 8.
+  // most 30 per SM). The exchange of a unit is hidden where its tiles leave room for as many of the next
+  // unit's, costs about 1000 where they leave some, and 3000 where they leave none. Large clusters leave
+  // SMs idle (15 of 8 CTAs and 7 of 16 fit the 148), small ones fit fewer keys.
+  // L 6007, 64 rows, 256 units: 102 us with 8 CTAs, 121 with 16; L 4096: 67 / 63 us with 4 / 8; 64-dim
+  // heads, 32 rows, L 4096, 128 units: 26.1 / 24.6 / 27.0 us with 2 / 4 / 8.
   int best = -1;
   double best_cost = 0.0;
   for (int i = 0; i < 5; ++i) {
@@ -868,7 +869,8 @@ laq_status score_cluster_launch(const laq_params& p, const Dims& d, const Worksp
     if (n < 1 || T > slots || C > n_tiles) continue;
     const double rounds = (double)((d.U + n - 1) / n);
     const double tile = fmax(200.0 + 20.0 * d.M, (double)(a.boxes * kBoxBytes) * fmax(n * C, 120.0) / 3600.0);
-    const double cost = rounds * (T * tile + (2 * T <= slots ? 1600.0 : 2500.0));
+    const double exchange = 2 * T <= slots ? 60.0 * C : (T < slots ? 1000.0 : 3000.0);
+    const double cost = rounds * (T * tile + exchange);
     if (best < 0 || cost < best_cost) {
       best = i;
       best_cost = cost;

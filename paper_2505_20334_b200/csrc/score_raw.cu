@@ -11,23 +11,48 @@
 namespace laq {
 namespace {
 
-// qsum[u][d] = sum over the unit's G*W query rows of q[r][d], in row order, fp32.
-__global__ void qsum_kernel(const __nv_bfloat16* __restrict__ q, float* __restrict__ qsum, int Bt,
-                            int Hkv, int G, int W, int D, int64_t s_layer, int64_t s_batch,
-                            int64_t s_head, int64_t s_pos) {
+constexpr int kQsumThreads = 256;
+
+// qsum[u][d] = sum over the unit's G*W query rows of q[r][d], fp32. One block per unit: a thread takes
+// eight dims (16 bytes) of every n-th row, and the n partial sums are added in order, so the result
+// does not depend on the launch. Bound: latency (512 units of 128 rows: 22 us with one dim per thread
+// and all rows in turn). Block 0 also clears the workspace header.
+__global__ void __launch_bounds__(kQsumThreads)
+qsum_kernel(const __nv_bfloat16* __restrict__ q, float* __restrict__ qsum, int32_t* __restrict__ hdr, int Bt,
+            int Hkv, int G, int W, int D, int64_t s_layer, int64_t s_batch, int64_t s_head, int64_t s_pos) {
+  __shared__ float s_part[kQsumThreads * 8];
+  allow_successor();
   const int64_t u = blockIdx.x;
+  if (u == 0 && threadIdx.x < HDR_WORDS) hdr[threadIdx.x] = 0;
   const int h = (int)(u % Hkv);
   const int64_t lb = u / Hkv;
   const int b = (int)(lb % Bt);
   const int64_t layer = lb / Bt;
-  const int d = threadIdx.x;
-  if (d >= D) return;
-  const __nv_bfloat16* base = q + layer * s_layer + b * s_batch;
-  float acc = 0.f;
-  for (int g = 0; g < G; ++g)
-    for (int i = 0; i < W; ++i)
-      acc += __bfloat162float(base[(int64_t)(h * G + g) * s_head + (int64_t)i * s_pos + d]);
-  qsum[u * D + d] = acc;
+  const int dv = D / 8, n_groups = kQsumThreads / dv;
+  const int c = threadIdx.x % dv, group = threadIdx.x / dv;
+  if (group < n_groups) {
+    const __nv_bfloat16* base = q + layer * s_layer + b * s_batch + (int64_t)h * G * s_head + 8 * c;
+    float acc[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] = 0.f;
+    for (int r = group; r < G * W; r += n_groups) {
+      const uint4 v = *reinterpret_cast<const uint4*>(base + (r / W) * s_head + (r % W) * s_pos);
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        acc[2 * i] += __uint_as_float(w[i] << 16);
+        acc[2 * i + 1] += __uint_as_float(w[i] & 0xffff0000u);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s_part[group * D + 8 * c + i] = acc[i];
+  }
+  __syncthreads();
+  for (int d = threadIdx.x; d < D; d += kQsumThreads) {
+    float sum = 0.f;
+    for (int g = 0; g < n_groups; ++g) sum += s_part[g * D + d];
+    qsum[u * D + d] = sum;
+  }
 }
 
 constexpr int kRawThreads = 256;
@@ -50,6 +75,7 @@ __global__ void __launch_bounds__(kRawThreads) score_raw_d128_kernel(
     int Bt, int Hkv, int L_alloc, int L_pad, float scale, int64_t s_layer, int64_t s_batch,
     int64_t s_head, int64_t s_pos, const __grid_constant__ SeqLens sl) {
   allow_successor();
+  wait_for_predecessor();  // the query sums
   const int64_t u = blockIdx.x;
   const int h = (int)(u % Hkv);
   const int64_t lb = u / Hkv;
@@ -118,6 +144,8 @@ __global__ void score_raw_any_kernel(const __nv_bfloat16* __restrict__ k,
                                      int64_t s_layer, int64_t s_batch, int64_t s_head,
                                      int64_t s_pos, const __grid_constant__ SeqLens sl) {
   __shared__ float s_q[256];
+  allow_successor();
+  wait_for_predecessor();  // the query sums
   const int64_t u = blockIdx.x;
   const int h = (int)(u % Hkv);
   const int64_t lb = u / Hkv;
@@ -151,26 +179,32 @@ laq_status score_raw_launch(const laq_params& p, const Dims& d, const Workspace&
   float* colsum = reinterpret_cast<float*>(ws + w.off_colsum);
   const __nv_bfloat16* qb = static_cast<const __nv_bfloat16*>(q);
   const __nv_bfloat16* kb = static_cast<const __nv_bfloat16*>(k);
-  qsum_kernel<<<(unsigned)d.U, (d.D + 31) / 32 * 32, 0, stream>>>(
-      qb, qsum, d.Bt, d.Hkv, d.G, d.W, d.D, p.q_stride_layer, p.q_stride_batch, p.q_stride_head,
-      p.q_stride_pos);
+  qsum_kernel<<<(unsigned)d.U, kQsumThreads, 0, stream>>>(
+      qb, qsum, reinterpret_cast<int32_t*>(ws + w.off_hdr), d.Bt, d.Hkv, d.G, d.W, d.D, p.q_stride_layer,
+      p.q_stride_batch, p.q_stride_head, p.q_stride_pos);
+  if (cudaGetLastError() != cudaSuccess) return LAQ_ERR_CUDA;
   *launches += 1;
+  cudaLaunchAttribute attr;
+  programmatic_launch(&attr);
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(kRawThreads);
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
   // grid.x = units, grid.y = chunks of keys
-  if (d.D == 128) {
-    const unsigned chunks = (unsigned)((d.L + kRawKeysPerBlock - 1) / kRawKeysPerBlock);
-    if (chunks > 65535) return LAQ_ERR_UNSUPPORTED;
-    score_raw_d128_kernel<<<dim3((unsigned)d.U, chunks), kRawThreads, 0, stream>>>(
-        kb, qsum, colsum, d.Bt, d.Hkv, d.L, w.L_pad, d.scale, p.k_stride_layer, p.k_stride_batch,
-        p.k_stride_head, p.k_stride_pos, d.sl);
-  } else {
-    const unsigned chunks = (unsigned)((d.L + 255) / 256);
-    if (chunks > 65535) return LAQ_ERR_UNSUPPORTED;
-    score_raw_any_kernel<<<dim3((unsigned)d.U, chunks), 256, 0, stream>>>(
-        kb, qsum, colsum, d.Bt, d.Hkv, d.D, d.L, w.L_pad, d.scale, p.k_stride_layer,
-        p.k_stride_batch, p.k_stride_head, p.k_stride_pos, d.sl);
-  }
+  const int per_block = d.D == 128 ? kRawKeysPerBlock : kRawThreads;
+  const unsigned chunks = (unsigned)((d.L + per_block - 1) / per_block);
+  if (chunks > 65535) return LAQ_ERR_UNSUPPORTED;
+  cfg.gridDim = dim3((unsigned)d.U, chunks);
+  const cudaError_t e =
+      d.D == 128
+          ? cudaLaunchKernelEx(&cfg, score_raw_d128_kernel, kb, (const float*)qsum, colsum, d.Bt, d.Hkv, d.L, w.L_pad,
+                               d.scale, p.k_stride_layer, p.k_stride_batch, p.k_stride_head, p.k_stride_pos, d.sl)
+          : cudaLaunchKernelEx(&cfg, score_raw_any_kernel, kb, (const float*)qsum, colsum, d.Bt, d.Hkv, d.D, d.L,
+                               w.L_pad, d.scale, p.k_stride_layer, p.k_stride_batch, p.k_stride_head, p.k_stride_pos,
+                               d.sl);
   *launches += 1;
-  return cudaGetLastError() == cudaSuccess ? LAQ_OK : LAQ_ERR_CUDA;
+  return e == cudaSuccess ? LAQ_OK : LAQ_ERR_CUDA;
 }
 
 }  // namespace laq

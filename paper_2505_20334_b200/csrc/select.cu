@@ -366,27 +366,32 @@ pool_select_reg_kernel(const __grid_constant__ SelArgs args, const __grid_consta
     constexpr int h = kPool > 0 ? kPool / 2 : 0;
     static_assert(h <= 4, "one vector of halo");
     const float4* row = reinterpret_cast<const float4*>(s_c);
-    float x[kItems + 8];  // [own - 4, own + kItems + 4)
+    // eight positions at a time from a window of sixteen: with all 40 words in registers at once next
+    // to the keys the block of 1024 threads spills
 #pragma unroll
-    for (int k = 0; k < kItems / 4 + 2; ++k) {
-      const float4 v = row[staged_at(kHalo + own - 4 + 4 * k) >> 2];
-      x[4 * k] = v.x; x[4 * k + 1] = v.y; x[4 * k + 2] = v.z; x[4 * k + 3] = v.w;
-    }
-    if (args.pool_max) {
+    for (int k0 = 0; k0 < kItems; k0 += 8) {
+      float x[16];  // [own + k0 - 4, own + k0 + 12)
 #pragma unroll
-      for (int k = 0; k < kItems; ++k) {
-        float m = x[4 + k];
-#pragma unroll
-        for (int t = -h; t <= h; ++t) m = fmaxf(m, x[4 + k + t]);
-        w[k] = __float_as_uint(m);
+      for (int k = 0; k < 4; ++k) {
+        const float4 v = row[staged_at(kHalo + own + k0 - 4 + 4 * k) >> 2];
+        x[4 * k] = v.x; x[4 * k + 1] = v.y; x[4 * k + 2] = v.z; x[4 * k + 3] = v.w;
       }
-    } else {
+      if (args.pool_max) {
 #pragma unroll
-      for (int k = 0; k < kItems; ++k) {
-        float acc = 0.f;
+        for (int k = 0; k < 8; ++k) {
+          float m = x[4 + k];
 #pragma unroll
-        for (int t = -h; t <= h; ++t) acc += x[4 + k + t];
-        w[k] = __float_as_uint(acc * args.inv_k);
+          for (int t = -h; t <= h; ++t) m = fmaxf(m, x[4 + k + t]);
+          w[k0 + k] = __float_as_uint(m);
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          float acc = 0.f;
+#pragma unroll
+          for (int t = -h; t <= h; ++t) acc += x[4 + k + t];
+          w[k0 + k] = __float_as_uint(acc * args.inv_k);
+        }
       }
     }
   }
