@@ -97,9 +97,22 @@ static laq_status check_strides_vo(const laq_params* p, bool need_v) {
 
 int choose_tiles_per_task(const Dims& d) {
   const int n_tiles = (d.L + TILE_KEYS - 1) / TILE_KEYS;
-  // default, measured on B200: 16 tiles (2048 keys) per task; 8 for short prompts, so that a unit
-  // still splits into several tasks
-  int t = d.tiles_per_task > 0 ? d.tiles_per_task : (n_tiles >= 64 ? 16 : 8);
+  int t = d.tiles_per_task;
+  if (t <= 0) {
+    // Measured on B200: 16 tiles (2048 keys) per task where there is much to do. With little, 8: the end
+    // of the launch, when SMs wait for the last tasks, weighs less (128 rows, 16 x 8 units of 12001 to
+    // 2311 keys: 475 -> 434 us; 256 units of 8192 keys 333 -> 320 us), at the price of more hand-offs
+    // (1024 units of 32768 keys: 3.79 -> 3.82 ms). Very long prompts stay with 16: sweep 2 has to trail
+    // by a unit, and twice the tasks would put it out of L2's reach (65536 keys: 770 -> 910 us).
+    int64_t tiles = d.U * (int64_t)n_tiles;
+    if (d.sl.n > 0) {
+      int64_t per_layer = 0;
+      for (int b = 0; b < d.Bt; ++b) per_layer += (d.sl.len[b] + TILE_KEYS - 1) / TILE_KEYS;
+      tiles = per_layer * d.Hkv * d.NL;
+    }
+    const int64_t much = d.sl.n > 0 ? 40000 : 24000;
+    t = n_tiles >= 400 || (n_tiles >= 64 && tiles >= much) ? 16 : 8;
+  }
   if (t > n_tiles) t = n_tiles;
   return t;
 }

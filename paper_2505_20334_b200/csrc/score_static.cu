@@ -55,6 +55,8 @@ extern "C" laq_status laq_score_static(const laq_params* p, const void* q, const
   if ((st = check_strides_qk(p)) != LAQ_OK) return st;
   Workspace w;
   plan_workspace(d, choose_tiles_per_task(d), &w);
+  // longer tasks leave fewer partial statistics: what does not fit otherwise may fit with them
+  if (w.off_pooled > kStaticScratchBytes && d.tiles_per_task <= 0) plan_workspace(d, 16, &w);
   // everything up to and including the column sums is needed; the caller supplies the scores
   if (w.off_pooled > kStaticScratchBytes) return LAQ_ERR_WORKSPACE;
   void* base = nullptr;
