@@ -453,6 +453,55 @@ static void* device_view_of_pinned(const void* host) {
   return nullptr;
 }
 
+}  // extern "C"
+
+// A stream for the copies of laq_evict_host and the events that order them with the caller's stream.
+// Every host thread has its own per device, made at its first call there and given back when the thread
+// ends; calls of one thread share it in order.
+constexpr int kMaxPieces = 16;
+struct CopyStream {
+  cudaStream_t stream = nullptr;
+  cudaEvent_t ready[kMaxPieces] = {};
+  bool usable = false;
+  bool create() {
+    usable = cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking) == cudaSuccess;
+    for (int i = 0; i < kMaxPieces && usable; ++i)
+      usable = cudaEventCreateWithFlags(&ready[i], cudaEventDisableTiming) == cudaSuccess;
+    if (!usable) {
+      destroy();
+      (void)cudaGetLastError();
+    }
+    return usable;
+  }
+  void destroy() {
+    for (cudaEvent_t& e : ready)
+      if (e) {
+        cudaEventDestroy(e);
+        e = nullptr;
+      }
+    if (stream) cudaStreamDestroy(stream);
+    stream = nullptr;
+    usable = false;
+  }
+};
+struct ThreadCopyStreams {
+  static constexpr int kDevices = 16;
+  CopyStream of_device[kDevices];
+  ~ThreadCopyStreams() {
+    for (CopyStream& c : of_device)
+      if (c.usable) c.destroy();
+  }
+};
+static CopyStream* copy_stream() {
+  static thread_local ThreadCopyStreams mine;
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= ThreadCopyStreams::kDevices) return nullptr;
+  CopyStream& c = mine.of_device[dev];
+  return c.usable || c.create() ? &c : nullptr;
+}
+
+extern "C" {
+
 size_t laq_host_staging_bytes(const laq_params* p) {
   Dims d;
   if (derive_dims(p, &d) != LAQ_OK) return 0;
@@ -490,25 +539,52 @@ laq_status laq_evict_host(const laq_params* p, const void* q_host, const void* k
   // host-to-device traffic) is skipped; pageable memory is staged on the device like Q and K.
   // The same holds for the outputs: pinned K_out / V_out are written by the gather directly, in
   // the same kernel that reads the V rows, so both directions of the bus work at once.
-  const void* v_dev = device_view_of_pinned(v_host);
-  void* ko_dev = device_view_of_pinned(k_out_host);
-  void* vo_dev = device_view_of_pinned(v_out_host);
-  if (cudaMemcpyAsync(sb + h.off_q, q_host, h.q_bytes, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
-      cudaMemcpyAsync(sb + h.off_k, k_host, h.kv_bytes, cudaMemcpyHostToDevice, stream) != cudaSuccess)
+  const char* v_pinned = (const char*)device_view_of_pinned(v_host);
+  char* ko_pinned = (char*)device_view_of_pinned(k_out_host);
+  char* vo_pinned = (char*)device_view_of_pinned(v_out_host);
+  // The bus is what bounds the call, so the copies of later layers run on a stream of their own while
+  // earlier ones are scored and gathered (8 layers x 8 heads x 8192 keys: 2.96 ms in one piece, of
+  // which 2.44 are the copy of K). Not worth it below a few MB per piece.
+  constexpr size_t kPieceBytes = 4u << 20;
+  int pieces = (int)(h.kv_bytes / kPieceBytes);
+  if (pieces > d.NL) pieces = d.NL;
+  if (pieces > kMaxPieces) pieces = kMaxPieces;
+  CopyStream* copy = pieces > 1 ? copy_stream() : nullptr;
+  if (!copy) pieces = 1;
+  cudaStream_t from_host = copy ? copy->stream : stream;
+  if (copy && (cudaEventRecord(copy->ready[0], stream) != cudaSuccess ||
+               cudaStreamWaitEvent(from_host, copy->ready[0], 0) != cudaSuccess))
     return LAQ_ERR_CUDA;
-  if (!v_dev) {
-    if (cudaMemcpyAsync(sb + h.off_v, v_host, h.kv_bytes, cudaMemcpyHostToDevice, stream) != cudaSuccess)
+  if (cudaMemcpyAsync(sb + h.off_q, q_host, h.q_bytes, cudaMemcpyHostToDevice, from_host) != cudaSuccess)
+    return LAQ_ERR_CUDA;
+  const size_t q_layer = h.q_bytes / d.NL, kv_layer = h.kv_bytes / d.NL, out_layer = h.out_bytes / d.NL,
+               idx_layer = h.idx_bytes / d.NL;
+  int launches = 0;
+  for (int i = 0; i < pieces; ++i) {
+    const size_t n0 = (size_t)d.NL * i / pieces, nl = (size_t)d.NL * (i + 1) / pieces - n0;
+    if (cudaMemcpyAsync(sb + h.off_k + n0 * kv_layer, (const char*)k_host + n0 * kv_layer, nl * kv_layer,
+                        cudaMemcpyHostToDevice, from_host) != cudaSuccess)
       return LAQ_ERR_CUDA;
-    v_dev = sb + h.off_v;
+    if (!v_pinned && cudaMemcpyAsync(sb + h.off_v + n0 * kv_layer, (const char*)v_host + n0 * kv_layer,
+                                     nl * kv_layer, cudaMemcpyHostToDevice, from_host) != cudaSuccess)
+      return LAQ_ERR_CUDA;
+    if (copy && (cudaEventRecord(copy->ready[i], from_host) != cudaSuccess ||
+                 cudaStreamWaitEvent(stream, copy->ready[i], 0) != cudaSuccess))
+      return LAQ_ERR_CUDA;
+    dp.n_layers = (int32_t)nl;
+    st = laq_evict(&dp, sb + h.off_q + n0 * q_layer, sb + h.off_k + n0 * kv_layer,
+                   (v_pinned ? v_pinned : sb + h.off_v) + n0 * kv_layer,
+                   (ko_pinned ? ko_pinned : sb + h.off_ko) + n0 * out_layer,
+                   (vo_pinned ? vo_pinned : sb + h.off_vo) + n0 * out_layer,
+                   (int32_t*)(sb + h.off_idx + n0 * idx_layer), nullptr, ws, ws_bytes, cuda_stream);
+    launches += g_last_launches;
+    if (st != LAQ_OK) return st;
   }
-  st = laq_evict(&dp, sb + h.off_q, sb + h.off_k, v_dev, ko_dev ? ko_dev : sb + h.off_ko,
-                 vo_dev ? vo_dev : sb + h.off_vo, (int32_t*)(sb + h.off_idx), nullptr, ws, ws_bytes,
-                 cuda_stream);
-  if (st != LAQ_OK) return st;
-  if ((!ko_dev && cudaMemcpyAsync(k_out_host, sb + h.off_ko, h.out_bytes, cudaMemcpyDeviceToHost,
-                                  stream) != cudaSuccess) ||
-      (!vo_dev && cudaMemcpyAsync(v_out_host, sb + h.off_vo, h.out_bytes, cudaMemcpyDeviceToHost,
-                                  stream) != cudaSuccess) ||
+  g_last_launches = launches;
+  if ((!ko_pinned && cudaMemcpyAsync(k_out_host, sb + h.off_ko, h.out_bytes, cudaMemcpyDeviceToHost,
+                                     stream) != cudaSuccess) ||
+      (!vo_pinned && cudaMemcpyAsync(v_out_host, sb + h.off_vo, h.out_bytes, cudaMemcpyDeviceToHost,
+                                     stream) != cudaSuccess) ||
       (idx_host && cudaMemcpyAsync(idx_host, sb + h.off_idx, h.idx_bytes, cudaMemcpyDeviceToHost,
                                    stream) != cudaSuccess))
     return LAQ_ERR_CUDA;
