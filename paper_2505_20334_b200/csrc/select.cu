@@ -341,13 +341,13 @@ pool_select_reg_kernel(const __grid_constant__ SelArgs args, const __grid_consta
   const int own = tid * kItems, base = pos0 + own;
   const int n_real = min(kItems, max(0, Ls - base));
   uint32_t w[kItems];
-  if (kPool == 0 || kPool == kCopy) {
+  if (kPool == 0) {
     const int h = args.kpool / 2;
 #pragma unroll
     for (int k = 0; k < kItems; ++k) {
       const int i = kHalo + own + k;
       float pj = s_c[staged_at(i)];
-      if (kPool == 0 && k < n_real) {
+      if (k < n_real) {
         if (h <= kHalo) {
           if (args.pool_max) {
             for (int t = -h; t <= h; ++t) pj = fmaxf(pj, s_c[staged_at(i + t)]);
@@ -376,7 +376,10 @@ pool_select_reg_kernel(const __grid_constant__ SelArgs args, const __grid_consta
         const float4 v = row[staged_at(kHalo + own + k0 - 4 + 4 * k) >> 2];
         x[4 * k] = v.x; x[4 * k + 1] = v.y; x[4 * k + 2] = v.z; x[4 * k + 3] = v.w;
       }
-      if (args.pool_max) {
+      if (kPool == kCopy) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) w[k0 + k] = __float_as_uint(x[4 + k]);
+      } else if (args.pool_max) {
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           float m = x[4 + k];
