@@ -294,7 +294,8 @@ struct SelArgs {
 __device__ __forceinline__ int staged_at(int i) { return i + ((i >> 5) << 2); }
 inline size_t staged_floats(int n) { return (size_t)(n + 2 * kHalo + 31) / 32 * 36; }
 
-// kPool: pooling kernel at compile time (1, 3, 5, 7), 0 = args.kpool, kCopy.
+// kPool: pooling kernel at compile time (1, 3, 5, 7, 9: the window fits the vectors of halo), 0 =
+// args.kpool, kCopy.
 template <int kPool, int kItems, bool kPair, class Geom>
 __global__ void __launch_bounds__(1024, 1)
 pool_select_reg_kernel(const __grid_constant__ SelArgs args, const __grid_constant__ Geom g) {
@@ -581,6 +582,7 @@ void launch_pool(dim3 grid, cudaStream_t stream, const Dims& d, const float* col
     case 3: LAQ_POOL(3); break;
     case 5: LAQ_POOL(5); break;
     case 7: LAQ_POOL(7); break;
+    case 9: LAQ_POOL(9); break;
     default: LAQ_POOL(0); break;
   }
 #undef LAQ_POOL
@@ -640,6 +642,7 @@ bool launch_select_pooled(const Dims& d, bool pool, cudaStream_t stream, const S
     case 3: return launch_select_sized<3, Geom>(d, stream, args, g);
     case 5: return launch_select_sized<5, Geom>(d, stream, args, g);
     case 7: return launch_select_sized<7, Geom>(d, stream, args, g);
+    case 9: return launch_select_sized<9, Geom>(d, stream, args, g);
     default: return launch_select_sized<0, Geom>(d, stream, args, g);
   }
 }
