@@ -51,8 +51,10 @@
  *     finishes; laq_last_device_status() reads that record back (it synchronises the stream).
  *   - No exceptions cross the boundary. Mutable state kept inside the library: cached per-device
  *     attributes; two per-host-thread instrumentation values (the stage events of
- *     laq_set_stage_events and the counter behind laq_last_launch_count); the cached address and
- *     the contents of laq_score_static's scratch array.
+ *     laq_set_stage_events and the counter behind laq_last_launch_count); one stream and its events
+ *     per host thread and device for the copies of laq_evict_host (made at the first call that
+ *     uses them, given back when the thread ends); the cached address and the contents of
+ *     laq_score_static's scratch array.
  */
 #ifndef LAQ_H_
 #define LAQ_H_
@@ -106,7 +108,7 @@ typedef struct {
   int32_t batch;       /* Bt >= 1 */
   int32_t n_q_heads;   /* Hq, a multiple of n_kv_heads */
   int32_t n_kv_heads;  /* Hkv >= 1; query head h reads KV head h / G */
-  int32_t head_dim;    /* D, a multiple of 8 up to 256; 128 takes the tensor-core path */
+  int32_t head_dim;    /* D, a multiple of 8 up to 256 (up to 128 on tensor cores) */
   int32_t prompt_len;  /* L */
   int32_t window_len;  /* W >= 1 lookahead queries per query head; G*W <= 256 */
   int32_t keep_tail;   /* R, 0 <= R < B: last R positions always kept and never scored */
@@ -301,6 +303,9 @@ LAQ_API laq_status laq_recall(int64_t n_units, const int32_t* idx_pred, int32_t 
  * device at all, which halves the host-to-device traffic; pageable v_host is staged like Q and K.
  * Pinned k_out_host / v_out_host are likewise written by the gather directly instead of being
  * staged and copied back.
+ * Caches of 8 MB of keys or more are taken in pieces of layers: the copies run on a second stream,
+ * ordered before and after `cuda_stream` by events, so that those of later layers overlap the scoring
+ * and gather of earlier ones.
  */
 LAQ_API size_t laq_host_staging_bytes(const laq_params* p);
 LAQ_API laq_status laq_evict_host(const laq_params* p, const void* q_host, const void* k_host,

@@ -57,7 +57,7 @@ struct Dims {
 };
 
 // Workspace layout (all offsets in bytes from the 256-byte aligned base).
-//   header   : int32 words (see HDR_*), zeroed at the start of every scoring call
+//   header   : int32 words (see HDR_*); every scoring call starts its status word at OK
 //   unit_cnt : int32 [U]   partial row statistics delivered so far, zeroed per call
 //   part     : float2 [U][n_part][M_pad]  partial (max, sum) in the log2 domain, one per task
 //   row_off  : float [U][M_pad]  b_r = log2e*scale*m_r + log2(l_r) (CUDA-core path only)
