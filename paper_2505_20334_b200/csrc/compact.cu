@@ -47,6 +47,7 @@ __device__ __forceinline__ int64_t first_row(const CompactLayersArgs& a, int64_t
 template <class Args>
 __global__ void __launch_bounds__(256) compact_kernel(const __grid_constant__ Args a) {
   constexpr bool kLayers = !std::is_same<Args, CompactArgs>::value;
+  allow_successor();  // the next call's scoring kernel sets itself up while this one drains
   const int64_t u = a.u0 + blockIdx.y;
   const int h = (int)(u % a.Hkv);
   const int b = (int)((u / a.Hkv) % a.Bt);

@@ -516,16 +516,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
   if (threadIdx.x == 0) {
     prefetch_tensor_map(&tmap_q);
     prefetch_tensor_map(&tmap_k);
-    if (blockIdx.x == 0) {
-      clk0 = clock64();
-      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(ns0));
-      // The status word starts at OK. CTAs start in order and a wait runs out long after that, so
-      // no record of this launch is lost.
-      a.hdr[HDR_STATUS] = 0;
-      a.hdr[HDR_WHERE] = 0;
-    }
   }
-  allow_successor();
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // stages first: the swizzled layout needs 1024-byte aligned addresses
   const uint32_t smem_base = smem_u32(smem_raw);
@@ -586,6 +577,17 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // Up to here nothing outside the SM was touched: the set-up overlaps the predecessor's end.
+  wait_for_predecessor();
+  allow_successor();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    clk0 = clock64();
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(ns0));
+    // The status word starts at OK. CTAs start in order and a wait runs out long after that, so
+    // no record of this launch is lost.
+    a.hdr[HDR_STATUS] = 0;
+    a.hdr[HDR_WHERE] = 0;
+  }
   cluster_sync();  // the cluster's barriers are initialised before anything is sent to them
   const uint32_t tmem_base = ctl->tmem_base;
   const uint32_t slot_mask = (1u << a.slots_log2) - 1u;
@@ -912,17 +914,18 @@ laq_status score_cluster_launch(const laq_params& p, const Dims& d, const Worksp
   if (!make_tensor_map(&tmap_q, q, qdims, qstr, qbox) || !make_tensor_map(&tmap_k, k, kdims, kstr, kbox))
     return LAQ_OK;  // layout TMA cannot describe
 
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = (unsigned)C;
-  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cudaLaunchAttribute attr[2];
+  programmatic_launch(&attr[0]);
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)C;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(clusters * C));
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = kSmemBytes;
   cfg.stream = stream;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
   if (cudaLaunchKernelEx(&cfg, kKernels[per_head ? 1 : 0][variant], tmap_q, tmap_k, a) != cudaSuccess)
     return LAQ_ERR_CUDA;
   *launches += 1;

@@ -21,6 +21,7 @@ __global__ void __launch_bounds__(kQsumThreads)
 qsum_kernel(const __nv_bfloat16* __restrict__ q, float* __restrict__ qsum, int32_t* __restrict__ hdr, int Bt,
             int Hkv, int G, int W, int D, int64_t s_layer, int64_t s_batch, int64_t s_head, int64_t s_pos) {
   __shared__ float s_part[kQsumThreads * 8];
+  wait_for_predecessor();
   allow_successor();
   const int64_t u = blockIdx.x;
   if (u == 0 && threadIdx.x < HDR_WORDS) hdr[threadIdx.x] = 0;
@@ -179,18 +180,20 @@ laq_status score_raw_launch(const laq_params& p, const Dims& d, const Workspace&
   float* colsum = reinterpret_cast<float*>(ws + w.off_colsum);
   const __nv_bfloat16* qb = static_cast<const __nv_bfloat16*>(q);
   const __nv_bfloat16* kb = static_cast<const __nv_bfloat16*>(k);
-  qsum_kernel<<<(unsigned)d.U, kQsumThreads, 0, stream>>>(
-      qb, qsum, reinterpret_cast<int32_t*>(ws + w.off_hdr), d.Bt, d.Hkv, d.G, d.W, d.D, p.q_stride_layer,
-      p.q_stride_batch, p.q_stride_head, p.q_stride_pos);
-  if (cudaGetLastError() != cudaSuccess) return LAQ_ERR_CUDA;
-  *launches += 1;
   cudaLaunchAttribute attr;
   programmatic_launch(&attr);
   cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(kRawThreads);
+  cfg.gridDim = dim3((unsigned)d.U);
+  cfg.blockDim = dim3(kQsumThreads);
   cfg.stream = stream;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, qsum_kernel, qb, qsum, reinterpret_cast<int32_t*>(ws + w.off_hdr), d.Bt, d.Hkv, d.G,
+                         d.W, d.D, p.q_stride_layer, p.q_stride_batch, p.q_stride_head, p.q_stride_pos) !=
+      cudaSuccess)
+    return LAQ_ERR_CUDA;
+  *launches += 1;
+  cfg.blockDim = dim3(kRawThreads);
   // grid.x = units, grid.y = chunks of keys
   const int per_block = d.D == 128 ? kRawKeysPerBlock : kRawThreads;
   const unsigned chunks = (unsigned)((d.L + per_block - 1) / per_block);
