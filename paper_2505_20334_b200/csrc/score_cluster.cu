@@ -97,7 +97,8 @@ struct Ctl {
   uint64_t k_full[kMaxStages], k_empty[kMaxStages];
   uint64_t slot_full[kMaxSlots], slot_empty[kMaxSlots];
   uint64_t stat_full[2], stat_empty[2];  // the pass-1 warps' pairs of a unit: delivered / read
-  uint64_t lse_full[2];                  // every CTA of the cluster has sent its pairs of a unit
+  uint64_t lse_full[2];  // every CTA of the cluster has sent its pairs of a unit; both exchange warps
+                         // arrive, so that neither can be two phases behind (a parity wait would miss one)
   uint64_t boff_full[2], boff_empty[2];  // -b_r of a unit: written / no longer needed
   uint64_t drain;
   uint32_t tmem_base;
@@ -544,7 +545,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
       mbar_init(smem_u32(&ctl->q_empty[i]), 1);
       mbar_init(smem_u32(&ctl->stat_full[i]), kPass1Warps);
       mbar_init(smem_u32(&ctl->stat_empty[i]), kExchangeWarps);
-      mbar_init(smem_u32(&ctl->lse_full[i]), 1);
+      mbar_init(smem_u32(&ctl->lse_full[i]), kExchangeWarps);
       mbar_init(smem_u32(&ctl->boff_full[i]), kExchangeWarps);
       mbar_init(smem_u32(&ctl->boff_empty[i]), kPass2Warps);
     }
@@ -702,6 +703,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
       if (!bounded_wait(a, ctl, &ctl->stat_full[buf], parity, 31)) break;
       const uint32_t bar = smem_u32(&ctl->lse_full[buf]);
       if (tid == 0) mbar_expect_tx(bar, (uint32_t)(C * a.M) * 8u);
+      else if (lane == 0) mbar_arrive(bar);
       float2* in = lse_in + (size_t)buf * C * rows8;
       if (u != a.withhold_unit) {
         for (int r = tid; r < a.M; r += 32 * kExchangeWarps) {

@@ -62,3 +62,18 @@ def test_cluster_scoring_sums_that_overflow(laq):
     out = laq.evict(q.cuda(), k.cuda(), v.cuda(), B, pool_kernel=kernel)
     assert {5, 300, 700} <= set(out["idx"][0, 0, 0].tolist())
     assert np.isfinite(out["k_out"].float().cpu().numpy()).all()
+
+
+@pytest.mark.parametrize("W,L,lens", [(1, 128, None), (2, 700, None), (4, 500, tuple([500, 131] * 16))])
+def test_cluster_scoring_many_short_units_of_few_rows(laq, W, L, lens):
+    # At most 32 rows: one of the two exchange warps has no row of its own. Three and more units fit the
+    # tensor memory at once, so the other one can be that far ahead; the two must stay in step.
+    NL, Bt, Hq, Hkv, D, kernel, B = 4, 32, 16, 4, 128, 3, 24
+    q, k, v = rand_inputs(NL, Bt, Hq, Hkv, D, L, W, seed=W + L, kscale=1.5)
+    compare_all_units(laq, q, k, v, W, kernel, B, seq_lens=lens)
+    qc, kc, vc = q.cuda(), k.cuda(), v.cuda()
+    first = laq.evict(qc, kc, vc, B, pool_kernel=kernel, want_scores=True, seq_lens=lens)
+    for _ in range(50):
+        out = laq.evict(qc, kc, vc, B, pool_kernel=kernel, want_scores=True, seq_lens=lens, ws=first["ws"])
+    assert laq.laq_last_device_status(out["params"], out["ws"]) == laq.LAQ_OK
+    assert torch.equal(out["scores"], first["scores"]) and torch.equal(out["idx"], first["idx"])
