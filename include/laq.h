@@ -314,8 +314,8 @@ LAQ_API laq_status laq_evict_host(const laq_params* p, const void* q_host, const
                                   size_t ws_bytes, void* cuda_stream);
 
 /*
- * Synchronises `cuda_stream` and reports what the last laq_score / laq_evict call that used
- * `ws` recorded on the device: LAQ_OK, LAQ_ERR_TIMEOUT (a bounded wait ran out; outputs are
+ * Synchronises `cuda_stream` and reports what the last laq_score / laq_evict / laq_evict_layers /
+ * laq_evict_host call that used `ws` recorded on the device: LAQ_OK, LAQ_ERR_TIMEOUT (a bounded wait ran out; outputs are
  * not valid) or LAQ_ERR_CUDA (the synchronise or the read-back failed).
  */
 LAQ_API laq_status laq_last_device_status(const laq_params* p, const void* ws, size_t ws_bytes,

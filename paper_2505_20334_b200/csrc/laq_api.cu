@@ -68,6 +68,7 @@ laq_status derive_dims(const laq_params* p, Dims* d) {
   d->tiles_per_task = p->tiles_per_task;
   d->sched_lag_tasks = p->sched_lag_tasks;
   d->scale = p->softmax_scale > 0.0f ? p->softmax_scale : 1.0f / sqrtf((float)d->D);
+  d->keep_status = false;
   d->lb.n = 0;
   return derive_seq_lens(p, &d->sl);
 }
@@ -166,7 +167,8 @@ laq_status run_scoring(const laq_params* p, const Dims& d, const Workspace& w,
   if (st == LAQ_OK && !done) {
     // header and unit counters are contiguous: one clear (the other kernels have no counters and set
     // the header themselves)
-    if (cudaMemsetAsync(ws + w.off_hdr, 0, w.off_part - w.off_hdr, stream) != cudaSuccess) return LAQ_ERR_CUDA;
+    const size_t from = w.off_hdr + (d.keep_status ? HDR_TICKET * sizeof(int32_t) : 0);
+    if (cudaMemsetAsync(ws + from, 0, w.off_part - from, stream) != cudaSuccess) return LAQ_ERR_CUDA;
     st = use_tensor_core_path(d) ? score_tc_launch(*p, d, w, q, k, ws, stream, launches)
                                  : score_simt_launch(*p, d, w, q, k, ws, stream, launches);
   }
@@ -572,11 +574,14 @@ laq_status laq_evict_host(const laq_params* p, const void* q_host, const void* k
                  cudaStreamWaitEvent(stream, copy->ready[i], 0) != cudaSuccess))
       return LAQ_ERR_CUDA;
     dp.n_layers = (int32_t)nl;
-    st = laq_evict(&dp, sb + h.off_q + n0 * q_layer, sb + h.off_k + n0 * kv_layer,
-                   (v_pinned ? v_pinned : sb + h.off_v) + n0 * kv_layer,
-                   (ko_pinned ? ko_pinned : sb + h.off_ko) + n0 * out_layer,
-                   (vo_pinned ? vo_pinned : sb + h.off_vo) + n0 * out_layer,
-                   (int32_t*)(sb + h.off_idx + n0 * idx_layer), nullptr, ws, ws_bytes, cuda_stream);
+    Dims di;
+    if ((st = derive_dims(&dp, &di)) != LAQ_OK) return st;
+    di.keep_status = i > 0;  // one call, one status: a wait that ran out in an earlier piece stays on record
+    st = evict_impl(&dp, di, sb + h.off_q + n0 * q_layer, sb + h.off_k + n0 * kv_layer,
+                    (v_pinned ? v_pinned : sb + h.off_v) + n0 * kv_layer,
+                    (ko_pinned ? ko_pinned : sb + h.off_ko) + n0 * out_layer,
+                    (vo_pinned ? vo_pinned : sb + h.off_vo) + n0 * out_layer,
+                    (int32_t*)(sb + h.off_idx + n0 * idx_layer), nullptr, ws, ws_bytes, cuda_stream);
     launches += g_last_launches;
     if (st != LAQ_OK) return st;
   }

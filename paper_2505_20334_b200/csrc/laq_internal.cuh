@@ -52,12 +52,13 @@ struct Dims {
   int64_t U;    // units
   float scale;  // softmax scale
   int tiles_per_task, sched_lag_tasks;  // caller's scheduling knobs (0 = automatic)
+  bool keep_status;  // a later piece of one call: the workspace's status word keeps what is recorded there
   SeqLens sl;   // per-prompt lengths (n = 0: uniform)
   LayerBudgets lb;  // per-layer budgets (n = 0: B for every layer; otherwise B = the largest)
 };
 
 // Workspace layout (all offsets in bytes from the 256-byte aligned base).
-//   header   : int32 words (see HDR_*); every scoring call starts its status word at OK
+//   header   : int32 words (see HDR_*); every call starts its status words at OK
 //   unit_cnt : int32 [U]   partial row statistics delivered so far, zeroed per call
 //   part     : float2 [U][n_part][M_pad]  partial (max, sum) in the log2 domain, one per task
 //   row_off  : float [U][M_pad]  b_r = log2e*scale*m_r + log2(l_r) (CUDA-core path only)
@@ -74,10 +75,11 @@ struct Workspace {
   int L_pad;   // L padded to a multiple of 128
 };
 
+// HDR_STATUS / HDR_WHERE: the first bounded wait that ran out in the call.
 // HDR_CYCLES / HDR_NANOS (two words each): SM clock cycles and wall-clock nanoseconds the first CTA
 // of the last tensor-core scoring launch ran for (instrumentation: their ratio is the SM clock the
 // kernel actually ran at, which the board's power management lowers under load).
-enum { HDR_STATUS = 0, HDR_TICKET = 1, HDR_WHERE = 2, HDR_CYCLES = 4, HDR_NANOS = 6, HDR_WORDS = 64 };
+enum { HDR_STATUS = 0, HDR_WHERE = 1, HDR_TICKET = 2, HDR_CYCLES = 4, HDR_NANOS = 6, HDR_WORDS = 64 };
 
 // Keys per scoring task (a task = one sweep over KEYS_PER_TASK consecutive keys of one unit).
 constexpr int TILE_KEYS = 128;
@@ -88,8 +90,9 @@ int choose_tiles_per_task(const Dims& d);
 
 // Host-side checks and the scoring dispatch shared by every entry point that scores.
 laq_status check_strides_qk(const laq_params* p);
-// Steps 1-3 into the workspace's colsum array: clears the header and the unit counters, records
-// the caller's stage events around the scoring kernel and picks the back end.
+// Steps 1-3 into the workspace's colsum array: picks the back end, clears the header and the unit
+// counters for those that need it (the others set the header themselves) and records the caller's
+// stage events around the scoring kernel.
 laq_status run_scoring(const laq_params* p, const Dims& d, const Workspace& w, const void* q,
                        const void* k, char* ws, cudaStream_t stream, int* launches);
 void set_last_launch_count(int n);

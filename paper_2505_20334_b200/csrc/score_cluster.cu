@@ -85,6 +85,7 @@ struct ClArgs {
   int stride_log2;   // TMEM columns per tile
   int c_log2;        // log2 of the cluster size
   float scale_log2;
+  int keep_status;    // the status words keep what an earlier piece of the call recorded
   int withhold_unit;  // test hook: this unit's statistics are never sent (-1: none)
   int32_t* hdr;
   float* colsum;
@@ -584,10 +585,9 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     clk0 = clock64();
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(ns0));
-    // The status word starts at OK. CTAs start in order and a wait runs out long after that, so
+    // The status words start at OK. CTAs start in order and a wait runs out long after that, so
     // no record of this launch is lost.
-    a.hdr[HDR_STATUS] = 0;
-    a.hdr[HDR_WHERE] = 0;
+    if (!a.keep_status) a.hdr[HDR_STATUS] = a.hdr[HDR_WHERE] = 0;
   }
   cluster_sync();  // the cluster's barriers are initialised before anything is sent to them
   const uint32_t tmem_base = ctl->tmem_base;
@@ -900,6 +900,7 @@ laq_status score_cluster_launch(const laq_params& p, const Dims& d, const Worksp
   a.Bt = d.Bt; a.Hkv = d.Hkv; a.G = d.G; a.W = d.W; a.W_local = d.W_local; a.L = d.L; a.M = d.M;
   a.L_pad = w.L_pad;
   a.scale_log2 = d.scale * kLog2e;
+  a.keep_status = d.keep_status;
   a.withhold_unit = (int)test_withhold_unit();
   a.hdr = (int32_t*)(ws + w.off_hdr);
   const bool per_head = d.group_mode != LAQ_GROUP_SUM;

@@ -16,15 +16,16 @@ constexpr int kQsumThreads = 256;
 // qsum[u][d] = sum over the unit's G*W query rows of q[r][d], fp32. One block per unit: a thread takes
 // eight dims (16 bytes) of every n-th row, and the n partial sums are added in order, so the result
 // does not depend on the launch. Bound: latency (512 units of 128 rows: 22 us with one dim per thread
-// and all rows in turn). Block 0 also clears the workspace header.
+// and all rows in turn). Block 0 also clears the workspace header
+// from word hdr_from on.
 __global__ void __launch_bounds__(kQsumThreads)
-qsum_kernel(const __nv_bfloat16* __restrict__ q, float* __restrict__ qsum, int32_t* __restrict__ hdr, int Bt,
-            int Hkv, int G, int W, int D, int64_t s_layer, int64_t s_batch, int64_t s_head, int64_t s_pos) {
+qsum_kernel(const __nv_bfloat16* __restrict__ q, float* __restrict__ qsum, int32_t* __restrict__ hdr, int hdr_from,
+            int Bt, int Hkv, int G, int W, int D, int64_t s_layer, int64_t s_batch, int64_t s_head, int64_t s_pos) {
   __shared__ float s_part[kQsumThreads * 8];
   wait_for_predecessor();
   allow_successor();
   const int64_t u = blockIdx.x;
-  if (u == 0 && threadIdx.x < HDR_WORDS) hdr[threadIdx.x] = 0;
+  if (u == 0 && (int)threadIdx.x >= hdr_from && threadIdx.x < HDR_WORDS) hdr[threadIdx.x] = 0;
   const int h = (int)(u % Hkv);
   const int64_t lb = u / Hkv;
   const int b = (int)(lb % Bt);
@@ -188,9 +189,9 @@ laq_status score_raw_launch(const laq_params& p, const Dims& d, const Workspace&
   cfg.stream = stream;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, qsum_kernel, qb, qsum, reinterpret_cast<int32_t*>(ws + w.off_hdr), d.Bt, d.Hkv, d.G,
-                         d.W, d.D, p.q_stride_layer, p.q_stride_batch, p.q_stride_head, p.q_stride_pos) !=
-      cudaSuccess)
+  if (cudaLaunchKernelEx(&cfg, qsum_kernel, qb, qsum, reinterpret_cast<int32_t*>(ws + w.off_hdr),
+                         d.keep_status ? (int)HDR_TICKET : 0, d.Bt, d.Hkv, d.G, d.W, d.D, p.q_stride_layer,
+                         p.q_stride_batch, p.q_stride_head, p.q_stride_pos) != cudaSuccess)
     return LAQ_ERR_CUDA;
   *launches += 1;
   cfg.blockDim = dim3(kRawThreads);

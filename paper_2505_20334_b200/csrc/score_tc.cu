@@ -869,9 +869,13 @@ bool make_tensor_map(CUtensorMap* map, const void* base, const uint64_t dims[5],
 namespace {
 
 #ifdef LAQ_TEST_HOOKS
-std::atomic<long long> g_withhold_unit{-1};
+std::atomic<long long> g_withhold_unit{-1}, g_withhold_launches{-1};
 }  // namespace
-int64_t test_withhold_unit() { return g_withhold_unit.load(); }
+int64_t test_withhold_unit() {
+  if (g_withhold_launches.load() == 0) return -1;
+  if (g_withhold_launches.load() > 0) g_withhold_launches.fetch_sub(1);
+  return g_withhold_unit.load();
+}
 #else
 }  // namespace
 int64_t test_withhold_unit() { return -1; }
@@ -882,8 +886,12 @@ int64_t test_withhold_unit() { return -1; }
 #ifdef LAQ_TEST_HOOKS
 // Test builds only (never part of liblaq.so): the scoring kernel withholds the statistics of one
 // unit, so that the bounded wait of that unit's second sweep runs out. -1 switches it off.
+// laq_test_withhold_launches(n): in the next n scoring launches only (-1: in all of them).
 extern "C" __attribute__((visibility("default"))) void laq_test_withhold_unit(long long unit) {
   laq::g_withhold_unit.store(unit);
+}
+extern "C" __attribute__((visibility("default"))) void laq_test_withhold_launches(long long n) {
+  laq::g_withhold_launches.store(n);
 }
 #endif
 

@@ -14,6 +14,19 @@ from parity_util import SCORE_RTOL, score_rel_err
 pytestmark = pytest.mark.gpu
 
 
+def hooked_library():
+    """A copy of the library with the test hooks and a ~1.5 ms limit on every wait."""
+    from paper_2505_20334_b200 import binding as laq
+    from paper_2505_20334_b200 import build
+
+    build.build_liblaq()
+    hooked = laq.load_library(build.build_liblaq(
+        defines=["-DLAQ_TEST_HOOKS", "-DLAQ_TIMEOUT_CYCLES=3000000LL"], variant="hooks"))
+    for f in (hooked.laq_test_withhold_unit, hooked.laq_test_withhold_launches):
+        f.argtypes, f.restype = [ctypes.c_longlong], None
+    return hooked
+
+
 def test_wait_that_runs_out_is_reported_and_the_context_stays_usable():
     from paper_2505_20334_b200 import binding as laq
     from paper_2505_20334_b200 import build
@@ -60,3 +73,35 @@ def test_wait_that_runs_out_is_reported_and_the_context_stays_usable():
     assert torch.equal(again, scores)
     ref = orc.evict(q.cpu(), k.cpu(), None, R, kernel, B, want_idx=False)["scores"]
     assert score_rel_err(scores.cpu().numpy(), ref) <= SCORE_RTOL
+
+
+@pytest.mark.parametrize("W", [16, 32])     # 64 rows: one sweep in a cluster; 128 rows: two sweeps
+def test_wait_that_runs_out_in_one_piece_of_a_host_call_is_reported(W):
+    # a host cache large enough to be taken in two pieces of layers; only the first one's scoring gives up
+    from paper_2505_20334_b200 import binding as laq
+
+    hooked = hooked_library()
+    NL, Bt, Hq, Hkv, D, L, kernel, B = 2, 1, 8, 2, 128, 8192, 7, 100     # 8.4 MB of keys
+    g = torch.Generator().manual_seed(W)
+    q = torch.randn((NL, Bt, Hq, W, D), generator=g).to(torch.bfloat16).pin_memory()
+    k, v = (torch.randn((NL, Bt, Hkv, L, D), generator=g).to(torch.bfloat16).pin_memory() for _ in range(2))
+    he = laq.HostEvictor(tuple(q.shape), tuple(k.shape), B, kernel, W, "cuda")
+    p = ctypes.byref(he.params)
+    stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+
+    def run():
+        assert hooked.laq_evict_host(p, q.data_ptr(), k.data_ptr(), v.data_ptr(), he.h_k_out.data_ptr(),
+                                     he.h_v_out.data_ptr(), he.h_idx.data_ptr(), he.staging.data_ptr(),
+                                     he.staging.numel(), he.ws.data_ptr(), he.ws.numel(), stream) == laq.LAQ_OK
+        return hooked.laq_last_device_status(p, he.ws.data_ptr(), he.ws.numel(), stream)
+
+    assert run() == laq.LAQ_OK and hooked.laq_last_launch_count() > 3      # two pieces
+    want = he.h_idx.clone()
+    hooked.laq_test_withhold_unit(1)
+    hooked.laq_test_withhold_launches(1)
+    try:
+        assert run() == laq.LAQ_ERR_TIMEOUT
+    finally:
+        hooked.laq_test_withhold_unit(-1)
+        hooked.laq_test_withhold_launches(-1)
+    assert run() == laq.LAQ_OK and torch.equal(he.h_idx, want)             # the next call starts afresh
