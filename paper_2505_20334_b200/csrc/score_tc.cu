@@ -313,12 +313,15 @@ __device__ __forceinline__ void stats_cols64(uint32_t taddr, float c, float& m, 
 // kPerHead: sweep 2 keeps one column sum per query head (colsum is [U*G][L_pad]); the launcher
 // only picks it when a head's rows never straddle a group of four rows or a 32-row chunk unevenly
 // (W a multiple of 4 that divides 32, or 32 or 64).
-template <bool kDup, bool kWide, bool kPerHead>
+// kPolyS1: share of sweep 1's exponentials on the FMA pipe (of every 8 pairs), measured to pay only for
+// 64 < M <= 128. Its polynomial has a relative error of 7.5e-5, which leaves the scores within 1e-6 of the
+// exact ones in the 2-norm; on the MUFU alone they are within 2e-7. Head dims other than 128 take none, so
+// that their scores are as precise as on CUDA cores, where they used to be formed (64 dims, 128 rows, 128
+// units of 32768 keys: 324 us, with the polynomial 310; 256 units of 4096: 95.4 and 93.9).
+template <bool kDup, bool kWide, bool kPerHead, int kPolyS1>
 __global__ void __launch_bounds__(kThreads, 1)
 score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
                 const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ TcArgs a) {
-  // share of sweep 1's exponentials on the FMA pipe: measured to pay only for 64 < M <= 128
-  constexpr int kPolyS1 = (kDup || kWide) ? 0 : LAQ_POLY_PAIRS_S1;
   constexpr uint32_t kQRows = kWide ? 256u : 128u;   // rows per 64-dim half of a Q stage
   constexpr uint32_t kSlotShift = kWide ? 1u : 2u;   // log2 of the K stages = accumulator buffers
   constexpr uint32_t kTbCols = kWide ? 256u : 128u;  // TMEM columns per accumulator buffer
@@ -976,15 +979,18 @@ laq_status score_tc_launch(const laq_params& p, const Dims& d, const Workspace& 
 
   const size_t smem = kCtlBytes + 2u * (size_t)q_rows * 256u + (size_t)n_slots * kKStageBytes;
   const bool per_head = d.group_mode != LAQ_GROUP_SUM;
-  auto kernel = per_head ? (dup ? score_tc_kernel<true, false, true>
-                                : (wide ? score_tc_kernel<false, true, true>
-                                        : score_tc_kernel<false, false, true>))
-                         : (dup ? score_tc_kernel<true, false, false>
-                                : (wide ? score_tc_kernel<false, true, false>
-                                        : score_tc_kernel<false, false, false>));
+  typedef void (*Kernel)(const CUtensorMap, const CUtensorMap, const TcArgs);
+  // [per head][dup, wide, neither, neither with other head dims]
+  static const Kernel kernels[2][4] = {
+      {score_tc_kernel<true, false, false, 0>, score_tc_kernel<false, true, false, 0>,
+       score_tc_kernel<false, false, false, LAQ_POLY_PAIRS_S1>, score_tc_kernel<false, false, false, 0>},
+      {score_tc_kernel<true, false, true, 0>, score_tc_kernel<false, true, true, 0>,
+       score_tc_kernel<false, false, true, LAQ_POLY_PAIRS_S1>, score_tc_kernel<false, false, true, 0>}};
+  const int variant = dup ? 0 : (wide ? 1 : (d.D == 128 ? 2 : 3));
+  const Kernel kernel = kernels[per_head][variant];
   // the shared-memory opt-in is a per-device attribute of each kernel variant: set once
   static std::atomic<uint32_t> smem_opted_in[kMaxDevices];
-  const uint32_t variant_bit = 1u << ((dup ? 0 : (wide ? 1 : 2)) + (per_head ? 3 : 0));
+  const uint32_t variant_bit = 1u << (variant + (per_head ? 4 : 0));
   if (dev >= kMaxDevices || !(smem_opted_in[dev].load(std::memory_order_acquire) & variant_bit)) {
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
         cudaSuccess)
