@@ -9,12 +9,16 @@
 namespace laq {
 namespace {
 
+constexpr int kRecallWarps = 8;
+// What a launch may have in shared memory without an opt-in, less the kernel's own static array.
+constexpr int kMaxStaged = (48 * 1024 - kRecallWarps * (int)sizeof(int)) / (int)sizeof(int32_t);
+
 __global__ void __launch_bounds__(256) recall_kernel(const int32_t* __restrict__ pred, int n_pred,
                                                      const int32_t* __restrict__ gold, int n_gold,
                                                      int32_t* __restrict__ n_common,
                                                      float* __restrict__ recall, int staged) {
   extern __shared__ int32_t s_gold[];
-  __shared__ int s_hits[8];
+  __shared__ int s_hits[kRecallWarps];
   wait_for_predecessor();
   const int64_t u = blockIdx.x;
   const int32_t* a = pred + u * n_pred;
@@ -40,7 +44,7 @@ __global__ void __launch_bounds__(256) recall_kernel(const int32_t* __restrict__
   __syncthreads();
   if (threadIdx.x == 0) {
     hits = 0;
-    for (int w = 0; w < 8; ++w) hits += s_hits[w];
+    for (int w = 0; w < kRecallWarps; ++w) hits += s_hits[w];
     if (n_common) n_common[u] = hits;
     if (recall) recall[u] = n_gold > 0 ? (float)hits / (float)n_gold : 0.f;
   }
@@ -60,7 +64,7 @@ extern "C" laq_status laq_recall(int64_t n_units, const int32_t* idx_pred, int32
        reinterpret_cast<uintptr_t>(n_common) | reinterpret_cast<uintptr_t>(recall)) & 3u)
     return LAQ_ERR_INVALID_ARG;
   if (n_units > (1ll << 34)) return LAQ_ERR_UNSUPPORTED;
-  const bool staged = n_gold <= 12288;
+  const bool staged = n_gold <= kMaxStaged;
   cudaLaunchAttribute attr;
   programmatic_launch(&attr);
   cudaLaunchConfig_t cfg = {};
