@@ -147,8 +147,8 @@ laq_status compact_launch(const laq_params& p, const Dims& d, const void* k, con
     const int64_t nu = d.U - u0 < 65535 ? d.U - u0 : 65535;
     cfg.gridDim = dim3((unsigned)((d.B + kRowsPerBlock - 1) / kRowsPerBlock), (unsigned)nu);
     const CompactArgs& plain = a;
-    if ((d.lb.n > 0 ? cudaLaunchKernelEx(&cfg, compact_kernel<CompactLayersArgs>, a)
-                    : cudaLaunchKernelEx(&cfg, compact_kernel<CompactArgs>, plain)) != cudaSuccess)
+    if (!cuda_ok(d.lb.n > 0 ? cudaLaunchKernelEx(&cfg, compact_kernel<CompactLayersArgs>, a)
+                            : cudaLaunchKernelEx(&cfg, compact_kernel<CompactArgs>, plain)))
       return LAQ_ERR_CUDA;
     *launches += 1;
   }

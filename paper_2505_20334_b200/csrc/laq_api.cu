@@ -160,7 +160,7 @@ void set_last_launch_count(int n) { g_last_launches = n; }
 laq_status run_scoring(const laq_params* p, const Dims& d, const Workspace& w,
                               const void* q, const void* k, char* ws, cudaStream_t stream,
                               int* launches) {
-  if (g_ev_begin && cudaEventRecord(g_ev_begin, stream) != cudaSuccess) return LAQ_ERR_CUDA;
+  if (g_ev_begin && !cuda_ok(cudaEventRecord(g_ev_begin, stream))) return LAQ_ERR_CUDA;
   bool done = d.score_raw;
   laq_status st = d.score_raw ? score_raw_launch(*p, d, w, q, k, ws, stream, launches)
                               : score_cluster_launch(*p, d, w, q, k, ws, stream, launches, &done);
@@ -168,11 +168,11 @@ laq_status run_scoring(const laq_params* p, const Dims& d, const Workspace& w,
     // header and unit counters are contiguous: one clear (the other kernels have no counters and set
     // the header themselves)
     const size_t from = w.off_hdr + (d.keep_status ? HDR_TICKET * sizeof(int32_t) : 0);
-    if (cudaMemsetAsync(ws + from, 0, w.off_part - from, stream) != cudaSuccess) return LAQ_ERR_CUDA;
+    if (!cuda_ok(cudaMemsetAsync(ws + from, 0, w.off_part - from, stream))) return LAQ_ERR_CUDA;
     st = use_tensor_core_path(d) ? score_tc_launch(*p, d, w, q, k, ws, stream, launches)
                                  : score_simt_launch(*p, d, w, q, k, ws, stream, launches);
   }
-  if (g_ev_end && cudaEventRecord(g_ev_end, stream) != cudaSuccess) return LAQ_ERR_CUDA;
+  if (g_ev_end && !cuda_ok(cudaEventRecord(g_ev_end, stream))) return LAQ_ERR_CUDA;
   return st;
 }
 
@@ -448,11 +448,10 @@ static void plan_staging(const Dims& d, HostStaging* h) {
 // aligned; NULL for pageable memory.
 static void* device_view_of_pinned(const void* host) {
   cudaPointerAttributes attr;
-  if (cudaPointerGetAttributes(&attr, host) == cudaSuccess && attr.type == cudaMemoryTypeHost &&
+  if (cuda_ok(cudaPointerGetAttributes(&attr, host)) && attr.type == cudaMemoryTypeHost &&
       attr.devicePointer != nullptr && (reinterpret_cast<uintptr_t>(attr.devicePointer) & 15u) == 0)
     return attr.devicePointer;
-  (void)cudaGetLastError();  // an unregistered pointer is not an error here
-  return nullptr;
+  return nullptr;  // an unregistered pointer is not an error here
 }
 
 }  // extern "C"
@@ -466,13 +465,10 @@ struct CopyStream {
   cudaEvent_t ready[kMaxPieces] = {};
   bool usable = false;
   bool create() {
-    usable = cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking) == cudaSuccess;
+    usable = cuda_ok(cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking));
     for (int i = 0; i < kMaxPieces && usable; ++i)
-      usable = cudaEventCreateWithFlags(&ready[i], cudaEventDisableTiming) == cudaSuccess;
-    if (!usable) {
-      destroy();
-      (void)cudaGetLastError();
-    }
+      usable = cuda_ok(cudaEventCreateWithFlags(&ready[i], cudaEventDisableTiming));
+    if (!usable) destroy();
     return usable;
   }
   void destroy() {
@@ -497,7 +493,7 @@ struct ThreadCopyStreams {
 static CopyStream* copy_stream() {
   static thread_local ThreadCopyStreams mine;
   int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= ThreadCopyStreams::kDevices) return nullptr;
+  if (!cuda_ok(cudaGetDevice(&dev)) || dev < 0 || dev >= ThreadCopyStreams::kDevices) return nullptr;
   CopyStream& c = mine.of_device[dev];
   return c.usable || c.create() ? &c : nullptr;
 }
@@ -554,24 +550,24 @@ laq_status laq_evict_host(const laq_params* p, const void* q_host, const void* k
   CopyStream* copy = pieces > 1 ? copy_stream() : nullptr;
   if (!copy) pieces = 1;
   cudaStream_t from_host = copy ? copy->stream : stream;
-  if (copy && (cudaEventRecord(copy->ready[0], stream) != cudaSuccess ||
-               cudaStreamWaitEvent(from_host, copy->ready[0], 0) != cudaSuccess))
+  if (copy && (!cuda_ok(cudaEventRecord(copy->ready[0], stream)) ||
+               !cuda_ok(cudaStreamWaitEvent(from_host, copy->ready[0], 0))))
     return LAQ_ERR_CUDA;
-  if (cudaMemcpyAsync(sb + h.off_q, q_host, h.q_bytes, cudaMemcpyHostToDevice, from_host) != cudaSuccess)
+  if (!cuda_ok(cudaMemcpyAsync(sb + h.off_q, q_host, h.q_bytes, cudaMemcpyHostToDevice, from_host)))
     return LAQ_ERR_CUDA;
   const size_t q_layer = h.q_bytes / d.NL, kv_layer = h.kv_bytes / d.NL, out_layer = h.out_bytes / d.NL,
                idx_layer = h.idx_bytes / d.NL;
   int launches = 0;
   for (int i = 0; i < pieces; ++i) {
     const size_t n0 = (size_t)d.NL * i / pieces, nl = (size_t)d.NL * (i + 1) / pieces - n0;
-    if (cudaMemcpyAsync(sb + h.off_k + n0 * kv_layer, (const char*)k_host + n0 * kv_layer, nl * kv_layer,
-                        cudaMemcpyHostToDevice, from_host) != cudaSuccess)
+    if (!cuda_ok(cudaMemcpyAsync(sb + h.off_k + n0 * kv_layer, (const char*)k_host + n0 * kv_layer, nl * kv_layer,
+                                 cudaMemcpyHostToDevice, from_host)))
       return LAQ_ERR_CUDA;
-    if (!v_pinned && cudaMemcpyAsync(sb + h.off_v + n0 * kv_layer, (const char*)v_host + n0 * kv_layer,
-                                     nl * kv_layer, cudaMemcpyHostToDevice, from_host) != cudaSuccess)
+    if (!v_pinned && !cuda_ok(cudaMemcpyAsync(sb + h.off_v + n0 * kv_layer, (const char*)v_host + n0 * kv_layer,
+                                              nl * kv_layer, cudaMemcpyHostToDevice, from_host)))
       return LAQ_ERR_CUDA;
-    if (copy && (cudaEventRecord(copy->ready[i], from_host) != cudaSuccess ||
-                 cudaStreamWaitEvent(stream, copy->ready[i], 0) != cudaSuccess))
+    if (copy && (!cuda_ok(cudaEventRecord(copy->ready[i], from_host)) ||
+                 !cuda_ok(cudaStreamWaitEvent(stream, copy->ready[i], 0))))
       return LAQ_ERR_CUDA;
     dp.n_layers = (int32_t)nl;
     Dims di;
@@ -586,12 +582,12 @@ laq_status laq_evict_host(const laq_params* p, const void* q_host, const void* k
     if (st != LAQ_OK) return st;
   }
   g_last_launches = launches;
-  if ((!ko_pinned && cudaMemcpyAsync(k_out_host, sb + h.off_ko, h.out_bytes, cudaMemcpyDeviceToHost,
-                                     stream) != cudaSuccess) ||
-      (!vo_pinned && cudaMemcpyAsync(v_out_host, sb + h.off_vo, h.out_bytes, cudaMemcpyDeviceToHost,
-                                     stream) != cudaSuccess) ||
-      (idx_host && cudaMemcpyAsync(idx_host, sb + h.off_idx, h.idx_bytes, cudaMemcpyDeviceToHost,
-                                   stream) != cudaSuccess))
+  if ((!ko_pinned &&
+       !cuda_ok(cudaMemcpyAsync(k_out_host, sb + h.off_ko, h.out_bytes, cudaMemcpyDeviceToHost, stream))) ||
+      (!vo_pinned &&
+       !cuda_ok(cudaMemcpyAsync(v_out_host, sb + h.off_vo, h.out_bytes, cudaMemcpyDeviceToHost, stream))) ||
+      (idx_host &&
+       !cuda_ok(cudaMemcpyAsync(idx_host, sb + h.off_idx, h.idx_bytes, cudaMemcpyDeviceToHost, stream))))
     return LAQ_ERR_CUDA;
   return LAQ_OK;
 }
@@ -602,9 +598,9 @@ laq_status laq_last_device_status(const laq_params* p, const void* ws, size_t ws
   laq_status st = derive_dims(p, &d);
   if (st != LAQ_OK) return st;
   if (!ws || ws_bytes < HDR_WORDS * sizeof(int32_t)) return LAQ_ERR_WORKSPACE;
-  if (cudaStreamSynchronize((cudaStream_t)cuda_stream) != cudaSuccess) return LAQ_ERR_CUDA;
+  if (!cuda_ok(cudaStreamSynchronize((cudaStream_t)cuda_stream))) return LAQ_ERR_CUDA;
   int32_t hdr[HDR_WORDS];
-  if (cudaMemcpy(hdr, ws, sizeof hdr, cudaMemcpyDeviceToHost) != cudaSuccess) return LAQ_ERR_CUDA;
+  if (!cuda_ok(cudaMemcpy(hdr, ws, sizeof hdr, cudaMemcpyDeviceToHost))) return LAQ_ERR_CUDA;
   if (hdr[HDR_STATUS] == 0) return LAQ_OK;
   return hdr[HDR_STATUS] == LAQ_ERR_TIMEOUT ? LAQ_ERR_TIMEOUT : LAQ_ERR_INTERNAL;
 }
@@ -613,9 +609,9 @@ laq_status laq_last_kernel_clock(const void* ws, size_t ws_bytes, void* cuda_str
                                  int64_t* sm_cycles, int64_t* nanoseconds) {
   if (!ws || ws_bytes < HDR_WORDS * sizeof(int32_t) || !sm_cycles || !nanoseconds)
     return LAQ_ERR_INVALID_ARG;
-  if (cudaStreamSynchronize((cudaStream_t)cuda_stream) != cudaSuccess) return LAQ_ERR_CUDA;
+  if (!cuda_ok(cudaStreamSynchronize((cudaStream_t)cuda_stream))) return LAQ_ERR_CUDA;
   int32_t hdr[HDR_WORDS];
-  if (cudaMemcpy(hdr, ws, sizeof hdr, cudaMemcpyDeviceToHost) != cudaSuccess) return LAQ_ERR_CUDA;
+  if (!cuda_ok(cudaMemcpy(hdr, ws, sizeof hdr, cudaMemcpyDeviceToHost))) return LAQ_ERR_CUDA;
   memcpy(sm_cycles, &hdr[HDR_CYCLES], sizeof(int64_t));
   memcpy(nanoseconds, &hdr[HDR_NANOS], sizeof(int64_t));
   return LAQ_OK;

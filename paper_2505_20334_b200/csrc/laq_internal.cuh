@@ -156,6 +156,14 @@ __device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepco
 __device__ __forceinline__ void allow_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 #endif
 
+// Whether a runtime call succeeded. A failure is reported by the call that meets it: the runtime's own
+// record of it is taken back, so that no later call finds it when it checks a launch of its own.
+inline bool cuda_ok(cudaError_t e) {
+  if (e == cudaSuccess) return true;
+  (void)cudaGetLastError();
+  return false;
+}
+
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 }  // namespace laq

@@ -76,9 +76,9 @@ extern "C" laq_status laq_recall(int64_t n_units, const int32_t* idx_pred, int32
   constexpr int64_t kSlab = 1ll << 30;  // units per launch (one block each)
   for (int64_t u0 = 0; u0 < n_units; u0 += kSlab) {
     cfg.gridDim = dim3((unsigned)(n_units - u0 < kSlab ? n_units - u0 : kSlab));
-    if (cudaLaunchKernelEx(&cfg, recall_kernel, idx_pred + u0 * n_pred, (int)n_pred, idx_gold + u0 * n_gold,
-                           (int)n_gold, n_common ? n_common + u0 : nullptr, recall ? recall + u0 : nullptr,
-                           staged ? 1 : 0) != cudaSuccess)
+    if (!cuda_ok(cudaLaunchKernelEx(&cfg, recall_kernel, idx_pred + u0 * n_pred, (int)n_pred,
+                                    idx_gold + u0 * n_gold, (int)n_gold, n_common ? n_common + u0 : nullptr,
+                                    recall ? recall + u0 : nullptr, staged ? 1 : 0)))
       return LAQ_ERR_CUDA;
   }
   return LAQ_OK;

@@ -807,13 +807,11 @@ bool cluster_counts(int dev, ClusterCounts* out) {
     std::lock_guard<std::mutex> lock(mutex);
     if (!known[dev].load(std::memory_order_relaxed)) {
       for (int i = 0; i < 2 * kVariants; ++i)
-        if (cudaFuncSetAttribute(kKernels[i / kVariants][i % kVariants], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kSmemBytes) != cudaSuccess ||
-            cudaFuncSetAttribute(kKernels[i / kVariants][i % kVariants],
-                                 cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-          (void)cudaGetLastError();
+        if (!cuda_ok(cudaFuncSetAttribute(kKernels[i / kVariants][i % kVariants],
+                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes)) ||
+            !cuda_ok(cudaFuncSetAttribute(kKernels[i / kVariants][i % kVariants],
+                                          cudaFuncAttributeNonPortableClusterSizeAllowed, 1)))
           return false;
-        }
       for (int i = 0; i < 5; ++i) {
         cudaLaunchAttribute attr;
         attr.id = cudaLaunchAttributeClusterDimension;
@@ -826,10 +824,7 @@ bool cluster_counts(int dev, ClusterCounts* out) {
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, kKernels[0][kVariants - 1], &cfg) != cudaSuccess) {
-          (void)cudaGetLastError();
-          n = 0;
-        }
+        if (!cuda_ok(cudaOccupancyMaxActiveClusters(&n, kKernels[0][kVariants - 1], &cfg))) n = 0;
         cached[dev].resident[i] = n;
       }
       known[dev].store(true, std::memory_order_release);
@@ -855,7 +850,7 @@ laq_status score_cluster_launch(const laq_params& p, const Dims& d, const Worksp
     return LAQ_OK;
   int dev = 0;
   ClusterCounts counts;
-  if (cudaGetDevice(&dev) != cudaSuccess) return LAQ_ERR_CUDA;
+  if (!cuda_ok(cudaGetDevice(&dev))) return LAQ_ERR_CUDA;
   if (!cluster_counts(dev, &counts)) return LAQ_OK;
   ClArgs a;
   a.groups = (d.M + 7) / 8;
@@ -929,7 +924,7 @@ laq_status score_cluster_launch(const laq_params& p, const Dims& d, const Worksp
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  if (cudaLaunchKernelEx(&cfg, kKernels[per_head ? 1 : 0][variant], tmap_q, tmap_k, a) != cudaSuccess)
+  if (!cuda_ok(cudaLaunchKernelEx(&cfg, kKernels[per_head ? 1 : 0][variant], tmap_q, tmap_k, a)))
     return LAQ_ERR_CUDA;
   *launches += 1;
   *done = true;

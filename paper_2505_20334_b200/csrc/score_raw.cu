@@ -189,9 +189,9 @@ laq_status score_raw_launch(const laq_params& p, const Dims& d, const Workspace&
   cfg.stream = stream;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, qsum_kernel, qb, qsum, reinterpret_cast<int32_t*>(ws + w.off_hdr),
-                         d.keep_status ? (int)HDR_TICKET : 0, d.Bt, d.Hkv, d.G, d.W, d.D, p.q_stride_layer,
-                         p.q_stride_batch, p.q_stride_head, p.q_stride_pos) != cudaSuccess)
+  if (!cuda_ok(cudaLaunchKernelEx(&cfg, qsum_kernel, qb, qsum, reinterpret_cast<int32_t*>(ws + w.off_hdr),
+                                  d.keep_status ? (int)HDR_TICKET : 0, d.Bt, d.Hkv, d.G, d.W, d.D, p.q_stride_layer,
+                                  p.q_stride_batch, p.q_stride_head, p.q_stride_pos)))
     return LAQ_ERR_CUDA;
   *launches += 1;
   cfg.blockDim = dim3(kRawThreads);
@@ -208,7 +208,7 @@ laq_status score_raw_launch(const laq_params& p, const Dims& d, const Workspace&
                                w.L_pad, d.scale, p.k_stride_layer, p.k_stride_batch, p.k_stride_head, p.k_stride_pos,
                                d.sl);
   *launches += 1;
-  return e == cudaSuccess ? LAQ_OK : LAQ_ERR_CUDA;
+  return cuda_ok(e) ? LAQ_OK : LAQ_ERR_CUDA;
 }
 
 }  // namespace laq

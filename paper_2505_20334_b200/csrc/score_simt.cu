@@ -198,10 +198,10 @@ laq_status score_simt_launch(const laq_params& p, const Dims& d, const Workspace
   const int dv = d.D / 8;
   const size_t smem_stats = ((size_t)w.M_pad * (dv + 1) + (size_t)kStageKeys * dv) * sizeof(uint4);
   const size_t smem_col = ((size_t)(kColTile + kRowBlock) * (dv + 1)) * sizeof(uint4);
-  if (cudaFuncSetAttribute(simt_stats_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem_stats) != cudaSuccess ||
-      cudaFuncSetAttribute(simt_colsum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem_col) != cudaSuccess)
+  if (!cuda_ok(cudaFuncSetAttribute(simt_stats_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)smem_stats)) ||
+      !cuda_ok(cudaFuncSetAttribute(simt_colsum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)smem_col)))
     return LAQ_ERR_CUDA;
   simt_stats_kernel<<<dim3((unsigned)d.U, n_chunks), w.M_pad, smem_stats, stream>>>(a);
   simt_merge_kernel<<<(unsigned)d.U, w.M_pad, 0, stream>>>(a, n_chunks);

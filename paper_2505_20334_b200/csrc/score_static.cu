@@ -27,11 +27,11 @@ void* g_scratch_ptr[kMaxDevices] = {};
 // remembered.
 laq_status static_scratch(void** out) {
   int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return LAQ_ERR_CUDA;
+  if (!cuda_ok(cudaGetDevice(&dev)) || dev < 0 || dev >= kMaxDevices) return LAQ_ERR_CUDA;
   std::lock_guard<std::mutex> lock(g_mutex);
   if (!g_scratch_ptr[dev]) {
     void* ptr = nullptr;
-    if (cudaGetSymbolAddress(&ptr, g_static_scratch) != cudaSuccess || !ptr) return LAQ_ERR_CUDA;
+    if (!cuda_ok(cudaGetSymbolAddress(&ptr, g_static_scratch)) || !ptr) return LAQ_ERR_CUDA;
     g_scratch_ptr[dev] = ptr;
   }
   *out = g_scratch_ptr[dev];

@@ -918,8 +918,8 @@ laq_status score_tc_launch(const laq_params& p, const Dims& d, const Workspace& 
     return score_simt_launch(p, d, w, q, k, ws, stream, launches);
   if (d.U >= 0x7fffffff) return LAQ_ERR_UNSUPPORTED;
   int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+  if (!cuda_ok(cudaGetDevice(&dev)) ||
+      !cuda_ok(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) || sms < 1)
     return LAQ_ERR_CUDA;
   // One ticket per task that holds tiles (with per-prompt lengths a short prompt has fewer).
   int64_t n_stream = (int64_t)d.U * a.tasks_per_unit;
@@ -992,8 +992,7 @@ laq_status score_tc_launch(const laq_params& p, const Dims& d, const Workspace& 
   static std::atomic<uint32_t> smem_opted_in[kMaxDevices];
   const uint32_t variant_bit = 1u << (variant + (per_head ? 4 : 0));
   if (dev >= kMaxDevices || !(smem_opted_in[dev].load(std::memory_order_acquire) & variant_bit)) {
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
+    if (!cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
       return LAQ_ERR_CUDA;
     if (dev < kMaxDevices) smem_opted_in[dev].fetch_or(variant_bit, std::memory_order_release);
   }

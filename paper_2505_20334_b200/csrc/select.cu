@@ -592,10 +592,10 @@ void launch_pool(dim3 grid, cudaStream_t stream, const Dims& d, const float* col
 template <class K>
 bool opt_in(K kernel, std::atomic<uint64_t>& devices) {
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  if (!cuda_ok(cudaGetDevice(&dev))) return false;
   if (dev < 64 && ((devices.load(std::memory_order_acquire) >> dev) & 1u)) return true;
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)(staged_floats(kPairHalf) * sizeof(float))) != cudaSuccess)
+  if (!cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)(staged_floats(kPairHalf) * sizeof(float)))))
     return false;
   if (dev < 64) devices.fetch_or(1ull << dev, std::memory_order_release);
   return true;
@@ -617,7 +617,7 @@ bool launch_select(unsigned units, int threads, cudaStream_t stream, const SelAr
   attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = kPair ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, pool_select_reg_kernel<kPool, kItems, kPair, Geom>, args, g) == cudaSuccess;
+  return cuda_ok(cudaLaunchKernelEx(&cfg, pool_select_reg_kernel<kPool, kItems, kPair, Geom>, args, g));
 }
 
 // Which of the kernels takes units of Ls scores: up to 32768 one CTA with 32 scores per thread, up to
