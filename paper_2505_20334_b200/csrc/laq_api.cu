@@ -118,6 +118,26 @@ int choose_tiles_per_task(const Dims& d) {
   return t;
 }
 
+// The bounds of what choose_tiles_per_task may return for units of d.L positions, whatever the number of
+// units and the lengths of their prompts.
+static int shortest_tiles_per_task(const Dims& d) {
+  const int n_tiles = (d.L + TILE_KEYS - 1) / TILE_KEYS;
+  const int t = d.tiles_per_task > 0 ? d.tiles_per_task : (n_tiles >= 400 ? 16 : 8);
+  return t < n_tiles ? t : n_tiles;
+}
+static int longest_tiles_per_task(const Dims& d) {
+  const int n_tiles = (d.L + TILE_KEYS - 1) / TILE_KEYS;
+  const int t = d.tiles_per_task > 0 ? d.tiles_per_task : (n_tiles >= 64 ? 16 : 8);
+  return t < n_tiles ? t : n_tiles;
+}
+
+bool plan_workspace_within(const Dims& d, size_t bytes, size_t Workspace::*end, Workspace* w) {
+  plan_workspace(d, choose_tiles_per_task(d), w);
+  if (w->*end <= bytes) return true;
+  plan_workspace(d, longest_tiles_per_task(d), w);
+  return w->*end <= bytes;
+}
+
 void plan_workspace(const Dims& d, int tiles_per_task, Workspace* w) {
   const int n_tiles = (d.L + TILE_KEYS - 1) / TILE_KEYS;
   const int n_tasks = (n_tiles + tiles_per_task - 1) / tiles_per_task;
@@ -199,8 +219,10 @@ laq_status selection_source(const Dims& d, const Workspace& w, char* ws, cudaStr
   return LAQ_OK;
 }
 
-static laq_status check_ws(const Workspace& w, const void* ws, size_t ws_bytes) {
-  if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0 || ws_bytes < w.total)
+// Plans the workspace of a call inside the caller's `ws`.
+static laq_status plan_in_ws(const Dims& d, const void* ws, size_t ws_bytes, Workspace* w) {
+  if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0 ||
+      !plan_workspace_within(d, ws_bytes, &Workspace::total, w))
     return LAQ_ERR_WORKSPACE;
   return LAQ_OK;
 }
@@ -236,7 +258,7 @@ size_t laq_workspace_bytes(const laq_params* p) {
   Dims d;
   if (derive_dims(p, &d) != LAQ_OK) return 0;
   Workspace w;
-  plan_workspace(d, choose_tiles_per_task(d), &w);
+  plan_workspace(d, shortest_tiles_per_task(d), &w);
   return w.total;
 }
 
@@ -251,8 +273,7 @@ laq_status laq_score(const laq_params* p, const void* q, const void* k, float* s
     return LAQ_ERR_INVALID_ARG;
   if ((st = check_strides_qk(p)) != LAQ_OK) return st;
   Workspace w;
-  plan_workspace(d, choose_tiles_per_task(d), &w);
-  if ((st = check_ws(w, ws, ws_bytes)) != LAQ_OK) return st;
+  if ((st = plan_in_ws(d, ws, ws_bytes, &w)) != LAQ_OK) return st;
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   char* wsb = (char*)ws;
   int launches = 0;
@@ -327,8 +348,7 @@ static laq_status evict_impl(const laq_params* p, const Dims& d, const void* q, 
   if ((st = check_strides_qk(p)) != LAQ_OK) return st;
   if ((k_out || v_out) && (st = check_strides_vo(p, v_out != nullptr)) != LAQ_OK) return st;
   Workspace w;
-  plan_workspace(d, choose_tiles_per_task(d), &w);
-  if ((st = check_ws(w, ws, ws_bytes)) != LAQ_OK) return st;
+  if ((st = plan_in_ws(d, ws, ws_bytes, &w)) != LAQ_OK) return st;
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   char* wsb = (char*)ws;
   int launches = 0;
@@ -527,8 +547,7 @@ laq_status laq_evict_host(const laq_params* p, const void* q_host, const void* k
   // everything laq_evict would refuse is refused here, before the first copy is enqueued
   {
     Workspace w;
-    plan_workspace(d, choose_tiles_per_task(d), &w);
-    if ((st = check_ws(w, ws, ws_bytes)) != LAQ_OK) return st;
+    if ((st = plan_in_ws(d, ws, ws_bytes, &w)) != LAQ_OK) return st;
   }
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   char* sb = (char*)staging;

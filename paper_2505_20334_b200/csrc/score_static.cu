@@ -53,18 +53,15 @@ extern "C" laq_status laq_score_static(const laq_params* p, const void* q, const
       (reinterpret_cast<uintptr_t>(k) & 15u) || (reinterpret_cast<uintptr_t>(scores) & 3u))
     return LAQ_ERR_INVALID_ARG;
   if ((st = check_strides_qk(p)) != LAQ_OK) return st;
-  Workspace w;
-  plan_workspace(d, choose_tiles_per_task(d), &w);
-  // longer tasks leave fewer partial statistics: what does not fit otherwise may fit with them
-  if (w.off_pooled > kStaticScratchBytes && d.tiles_per_task <= 0) plan_workspace(d, 16, &w);
   // everything up to and including the column sums is needed; the caller supplies the scores
-  if (w.off_pooled > kStaticScratchBytes) return LAQ_ERR_WORKSPACE;
+  Workspace w;
+  if (!plan_workspace_within(d, kStaticScratchBytes, &Workspace::off_pooled, &w)) return LAQ_ERR_WORKSPACE;
   void* base = nullptr;
   if ((st = static_scratch(&base)) != LAQ_OK) return st;
   char* ws = static_cast<char*>(base);
   cudaStream_t stream = (cudaStream_t)cuda_stream;
-  // run_scoring clears the header and the per-unit counters, which must start at zero; the rest
-  // of the scratch is written before it is read
+  // run_scoring has whatever must start at zero cleared (the header, and the unit counters where they
+  // are used); the rest of the scratch is written before it is read
   int launches = 0;
   st = run_scoring(p, d, w, q, k, ws, stream, &launches);
   const float* colsum = nullptr;

@@ -153,3 +153,25 @@ def test_group_mode_and_streaming_arguments_are_checked_on_the_host(binding):
         st = binding.lib.laq_streaming_indices(ctypes.byref(p), n_sink, ctypes.c_void_p(16), None)
         assert st == binding.LAQ_ERR_INVALID_ARG
     assert binding.lib.laq_streaming_indices(ctypes.byref(p), 4, None, None) == binding.LAQ_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("rows", [32, 128, 256])
+@pytest.mark.parametrize("layers,batch,length", [(1, 4, 1000), (12, 4, 12001), (16, 4, 12001), (60, 4, 12001),
+                                                 (3, 2, 8192), (8, 1, 32768), (4, 4, 51000), (4, 4, 65536)])
+def test_workspace_depends_on_allocated_sizes_only(binding, rows, layers, batch, length):
+    # a workspace is sized once and kept for later batches: shorter prompts, fewer layers and shorter
+    # allocations must not need more of it
+    group = 8 if rows == 256 else 4
+    def params(n_layers, n_batch, n_pos):
+        return binding.make_params(n_layers, n_batch, 8 * group, 8, 128, n_pos, rows // group, 32, 7, 64)
+    p = params(layers, batch, length)
+    base = binding.laq_workspace_bytes(p)
+    assert base > 0
+    for lens in ([length] * batch, [length] + [300] * (batch - 1), [65] * batch,
+                 [length - (length - 500) * b // batch for b in range(batch)]):
+        p.set_seq_lens(lens)
+        assert binding.laq_workspace_bytes(p) == base
+    for n in range(1, layers):
+        assert binding.laq_workspace_bytes(params(n, batch, length)) < base
+    for n_pos in range(200, length, 997):
+        assert binding.laq_workspace_bytes(params(layers, batch, n_pos)) < base

@@ -22,3 +22,43 @@ def test_scores_of_other_head_dims_are_as_precise_as_fp32_sums(laq, D, W):  # no
     ref = orc.evict(q, k, v, W, 7, 100)["scores"]
     got = out["scores"].cpu().numpy().astype(np.float64)
     assert np.linalg.norm(got - ref) <= 4.8e-7 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("W", [8, 32])          # 32 and 128 rows
+def test_one_workspace_serves_batches_of_other_lengths(laq, W):  # noqa: F811
+    # sized for the allocated batch, then used for batches of shorter prompts and for fewer layers: the
+    # sizes lie on either side of where tasks of 8 and of 16 tiles are chosen (12032 .. 48128 tiles)
+    NL, Bt, Hkv, D, L, B = 16, 4, 8, 128, 12001, 200
+    g = torch.Generator(device="cuda").manual_seed(W)
+    q = torch.randn((NL, Bt, 4 * Hkv, W, D), generator=g, device="cuda", dtype=torch.bfloat16)
+    k = torch.randn((NL, Bt, Hkv, L, D), generator=g, device="cuda", dtype=torch.bfloat16)
+    ws = laq.alloc_workspace(laq.params_for(q, k, W, 7, B), "cuda")
+    for n, lens in ((NL, None), (NL, (12001, 8771, 5541, 2311)), (NL, (12001,) * 4), (NL, (201,) * 4), (12, None),
+                    (12, (12001,) * 4), (4, None)):
+        p = laq.params_for(q[:n], k[:n], W, 7, B)
+        p.set_seq_lens(lens)
+        scores = torch.empty((n, Bt, Hkv, L - W), dtype=torch.float32, device="cuda")
+        assert laq.laq_score(p, q[:n], k[:n], scores, ws, check=False) == laq.LAQ_OK
+        assert laq.laq_last_device_status(p, ws) == laq.LAQ_OK
+        own = torch.empty_like(scores)
+        laq.laq_score(p, q[:n], k[:n], own, laq.alloc_workspace(p, "cuda"))
+        assert torch.equal(scores, own)
+
+
+def test_static_scratch_takes_longer_tasks_where_shorter_ones_do_not_fit(laq):  # noqa: F811
+    # 256 rows and 16384 keys: 97 KB of scratch a unit with tasks of 8 tiles, 81 KB with tasks of 16, so that
+    # 92 units fit the fixed 8 MB only with the latter, which the caller's workspace would not need
+    NL, Hkv, D, L, W, B = 23, 4, 128, 16384, 32, 100
+    g = torch.Generator(device="cuda").manual_seed(5)
+    q = torch.randn((NL, 1, 8 * Hkv, W, D), generator=g, device="cuda", dtype=torch.bfloat16)
+    k = torch.randn((NL, 1, Hkv, L, D), generator=g, device="cuda", dtype=torch.bfloat16)
+    p = laq.params_for(q, k, W, 7, B)
+    want = torch.empty((NL, 1, Hkv, L - W), dtype=torch.float32, device="cuda")
+    laq.laq_score(p, q, k, want, laq.alloc_workspace(p, "cuda"))
+    got = torch.full_like(want, float("nan"))
+    assert laq.laq_score_static(p, q, k, got, check=False) == laq.LAQ_OK
+    # the same terms, the row sums added in other groups: fp32 rounding only
+    assert float((got - want).norm() / want.norm()) < 5e-7
+    # and what does not fit even so (108 units) is refused
+    p = laq.make_params(27, 1, 8 * Hkv, Hkv, D, L, W, W, 7, B)
+    assert laq.laq_score_static(p, q, k, got, check=False) == laq.LAQ_ERR_WORKSPACE
