@@ -510,12 +510,25 @@ struct ThreadCopyStreams {
       if (c.usable) c.destroy();
   }
 };
-static CopyStream* copy_stream() {
+// The graph capture a stream belongs to (0: none); false if that cannot be told.
+static bool capture_of(cudaStream_t stream, unsigned long long* id) {
+  cudaStreamCaptureStatus status;
+  *id = 0;
+  if (!cuda_ok(cudaStreamGetCaptureInfo(stream, &status, id))) return false;
+  if (status == cudaStreamCaptureStatusNone) *id = 0;
+  return status != cudaStreamCaptureStatusInvalidated;
+}
+// Null also while the thread's copy stream belongs to a graph capture that `caller` is not part of: the
+// capture of a call takes the copy stream in until it ends, and calls outside of it go without.
+static CopyStream* copy_stream(cudaStream_t caller) {
   static thread_local ThreadCopyStreams mine;
   int dev = -1;
   if (!cuda_ok(cudaGetDevice(&dev)) || dev < 0 || dev >= ThreadCopyStreams::kDevices) return nullptr;
   CopyStream& c = mine.of_device[dev];
-  return c.usable || c.create() ? &c : nullptr;
+  if (!c.usable && !c.create()) return nullptr;
+  unsigned long long of_copies = 0, of_caller = 0;
+  if (!capture_of(c.stream, &of_copies) || !capture_of(caller, &of_caller)) return nullptr;
+  return of_copies == 0 || of_copies == of_caller ? &c : nullptr;
 }
 
 extern "C" {
@@ -566,7 +579,7 @@ laq_status laq_evict_host(const laq_params* p, const void* q_host, const void* k
   int pieces = (int)(h.kv_bytes / kPieceBytes);
   if (pieces > d.NL) pieces = d.NL;
   if (pieces > kMaxPieces) pieces = kMaxPieces;
-  CopyStream* copy = pieces > 1 ? copy_stream() : nullptr;
+  CopyStream* copy = pieces > 1 ? copy_stream(stream) : nullptr;
   if (!copy) pieces = 1;
   cudaStream_t from_host = copy ? copy->stream : stream;
   if (copy && (!cuda_ok(cudaEventRecord(copy->ready[0], stream)) ||

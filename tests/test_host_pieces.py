@@ -38,3 +38,35 @@ def test_host_cache_in_pieces_equals_device_run(laq, pinned, lens):
                     assert (np.abs(s[diff] - theta) <= 1e-5 * theta).all()
                     assert (bits(hk[n, b, h]) == bits(k[n, b, h])[a]).all()
                     assert (bits(hv[n, b, h]) == bits(v[n, b, h])[a]).all()
+
+
+def test_host_call_while_another_one_is_being_captured(laq):
+    # The copies of a large host cache run on a second stream, which a capture of the caller's stream takes
+    # in. A call on another stream meanwhile must neither join that capture nor fail.
+    NL, Bt, Hq, Hkv, D, L, W, kernel, B = 4, 1, 4, 2, 128, 4100, 8, 7, 200   # 8.4 MB of keys: two pieces
+    sets = [[t.pin_memory() for t in rand_inputs(NL, Bt, Hq, Hkv, D, L, W, seed=s, kscale=1.5)] for s in (1, 2)]
+    evictors = [laq.HostEvictor(tuple(q.shape), tuple(k.shape), B, kernel, W, "cuda") for q, k, _ in sets]
+    want = []
+    for he, host in zip(evictors, sets):
+        he.run(*host)
+        torch.cuda.synchronize()
+        want.append([t.clone() for t in (he.h_k_out, he.h_v_out, he.h_idx)])
+        for t in (he.h_k_out, he.h_v_out, he.h_idx):
+            t.zero_()
+    capturing, other = torch.cuda.Stream(), torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=capturing, capture_error_mode="relaxed"):
+        evictors[0].run(*sets[0], stream=capturing)
+        evictors[1].run(*sets[1], stream=other)
+        evictors[0].run(*sets[0], stream=capturing)
+    other.synchronize()
+    assert not evictors[0].h_idx.any()                     # captured, not run
+    for _ in range(2):
+        graph.replay()
+        torch.cuda.synchronize()
+        for he, w in zip(evictors, want):
+            for got, ref in zip((he.h_k_out, he.h_v_out, he.h_idx), w):
+                assert torch.equal(got.view(torch.int16), ref.view(torch.int16))
+    evictors[0].run(*sets[0])                              # and the second stream works as before
+    torch.cuda.synchronize()
+    assert torch.equal(evictors[0].h_idx, want[0][2])
