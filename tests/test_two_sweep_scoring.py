@@ -42,7 +42,9 @@ def test_one_workspace_serves_batches_of_other_lengths(laq, W):  # noqa: F811
         assert laq.laq_last_device_status(p, ws) == laq.LAQ_OK
         own = torch.empty_like(scores)
         laq.laq_score(p, q[:n], k[:n], own, laq.alloc_workspace(p, "cuda"))
-        assert torch.equal(scores, own)
+        # (which softmax warps take a tile depends on the tiles their CTA has had before, so the order of a
+        # sum is not fixed where tasks have odd numbers of tiles: fp32 rounding only)
+        assert float((scores - own).norm() / own.norm()) < 5e-7
 
 
 def test_static_scratch_takes_longer_tasks_where_shorter_ones_do_not_fit(laq):  # noqa: F811
