@@ -324,8 +324,9 @@ LAQ_API laq_status laq_last_device_status(const laq_params* p, const void* ws, s
 /*
  * Instrumentation for benchmarks: caller-owned CUDA events (cudaEvent_t passed as void*) that
  * later laq_score / laq_evict calls made by this host thread record on their stream immediately
- * before and after the scoring kernel (steps 1-3). Pass NULL, NULL to stop recording. The events
- * must outlive the calls that record them.
+ * before and after the scoring kernel (steps 1-3); laq_evict_host records them before the first piece's
+ * and after the last piece's. Pass NULL, NULL to stop recording. The events must outlive the calls that
+ * record them.
  */
 LAQ_API void laq_set_stage_events(void* score_begin, void* score_end);
 

@@ -68,7 +68,7 @@ laq_status derive_dims(const laq_params* p, Dims* d) {
   d->tiles_per_task = p->tiles_per_task;
   d->sched_lag_tasks = p->sched_lag_tasks;
   d->scale = p->softmax_scale > 0.0f ? p->softmax_scale : 1.0f / sqrtf((float)d->D);
-  d->keep_status = false;
+  d->keep_status = d->more_pieces = false;
   d->lb.n = 0;
   return derive_seq_lens(p, &d->sl);
 }
@@ -180,7 +180,7 @@ void set_last_launch_count(int n) { g_last_launches = n; }
 laq_status run_scoring(const laq_params* p, const Dims& d, const Workspace& w,
                               const void* q, const void* k, char* ws, cudaStream_t stream,
                               int* launches) {
-  if (g_ev_begin && !cuda_ok(cudaEventRecord(g_ev_begin, stream))) return LAQ_ERR_CUDA;
+  if (g_ev_begin && !d.keep_status && !cuda_ok(cudaEventRecord(g_ev_begin, stream))) return LAQ_ERR_CUDA;
   bool done = d.score_raw;
   laq_status st = d.score_raw ? score_raw_launch(*p, d, w, q, k, ws, stream, launches)
                               : score_cluster_launch(*p, d, w, q, k, ws, stream, launches, &done);
@@ -192,7 +192,7 @@ laq_status run_scoring(const laq_params* p, const Dims& d, const Workspace& w,
     st = use_tensor_core_path(d) ? score_tc_launch(*p, d, w, q, k, ws, stream, launches)
                                  : score_simt_launch(*p, d, w, q, k, ws, stream, launches);
   }
-  if (g_ev_end && !cuda_ok(cudaEventRecord(g_ev_end, stream))) return LAQ_ERR_CUDA;
+  if (g_ev_end && !d.more_pieces && !cuda_ok(cudaEventRecord(g_ev_end, stream))) return LAQ_ERR_CUDA;
   return st;
 }
 
@@ -605,6 +605,7 @@ laq_status laq_evict_host(const laq_params* p, const void* q_host, const void* k
     Dims di;
     if ((st = derive_dims(&dp, &di)) != LAQ_OK) return st;
     di.keep_status = i > 0;  // one call, one status: a wait that ran out in an earlier piece stays on record
+    di.more_pieces = i + 1 < pieces;
     st = evict_impl(&dp, di, sb + h.off_q + n0 * q_layer, sb + h.off_k + n0 * kv_layer,
                     (v_pinned ? v_pinned : sb + h.off_v) + n0 * kv_layer,
                     (ko_pinned ? ko_pinned : sb + h.off_ko) + n0 * out_layer,

@@ -52,7 +52,9 @@ struct Dims {
   int64_t U;    // units
   float scale;  // softmax scale
   int tiles_per_task, sched_lag_tasks;  // caller's scheduling knobs (0 = automatic)
-  bool keep_status;  // a later piece of one call: the workspace's status word keeps what is recorded there
+  // one call in pieces: pieces of it have run before (the workspace's status words keep what those
+  // recorded), pieces of it follow (the end of scoring is yet to come)
+  bool keep_status, more_pieces;
   SeqLens sl;   // per-prompt lengths (n = 0: uniform)
   LayerBudgets lb;  // per-layer budgets (n = 0: B for every layer; otherwise B = the largest)
 };

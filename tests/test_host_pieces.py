@@ -70,3 +70,25 @@ def test_host_call_while_another_one_is_being_captured(laq):
     evictors[0].run(*sets[0])                              # and the second stream works as before
     torch.cuda.synchronize()
     assert torch.equal(evictors[0].h_idx, want[0][2])
+
+
+def test_stage_events_of_a_host_call_span_all_its_pieces(laq):
+    # 32 MB of keys in pieces: the copy of the last pieces lies between the first scoring and the last
+    NL, Bt, Hq, Hkv, D, L, W, kernel, B = 8, 1, 4, 2, 128, 8192, 8, 7, 200
+    host = [t.pin_memory() for t in rand_inputs(NL, Bt, Hq, Hkv, D, L, W, seed=3)]
+    he = laq.HostEvictor(tuple(host[0].shape), tuple(host[1].shape), B, kernel, W, "cuda")
+    events = [torch.cuda.Event(enable_timing=True) for _ in range(4)]
+    for e in events:
+        e.record()
+    he.run(*host)
+    torch.cuda.synchronize()
+    laq.laq_set_stage_events(events[1], events[2])
+    try:
+        events[0].record()
+        he.run(*host)
+        events[3].record()
+    finally:
+        laq.laq_set_stage_events()
+    torch.cuda.synchronize()
+    # eight pieces: from the first one's scoring to the last one's is most of the call
+    assert events[1].elapsed_time(events[2]) > 0.5 * events[0].elapsed_time(events[3])
