@@ -155,6 +155,8 @@ laq_status streaming_launch(const Dims& d, int n_sink, int32_t* idx, cudaStream_
 // Programmatic dependent launch: a kernel launched with `attr` may start while the kernel before it in
 // the stream still runs; it has to call wait_for_predecessor() before it touches memory that one
 // writes (or reads, where it overwrites it). allow_successor() lets such a kernel start from here on.
+// What the predecessor writes must not be declared const __restrict__: that allows loads through the
+// read-only path, for data that nothing writes while the kernel runs, and loads ahead of the wait.
 inline void programmatic_launch(cudaLaunchAttribute* attr) {
   attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr->val.programmaticStreamSerializationAllowed = 1;

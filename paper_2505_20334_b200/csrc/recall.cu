@@ -13,10 +13,9 @@ constexpr int kRecallWarps = 8;
 // What a launch may have in shared memory without an opt-in, less the kernel's own static array.
 constexpr int kMaxStaged = (48 * 1024 - kRecallWarps * (int)sizeof(int)) / (int)sizeof(int32_t);
 
-__global__ void __launch_bounds__(256) recall_kernel(const int32_t* __restrict__ pred, int n_pred,
-                                                     const int32_t* __restrict__ gold, int n_gold,
-                                                     int32_t* __restrict__ n_common,
-                                                     float* __restrict__ recall, int staged) {
+__global__ void __launch_bounds__(256) recall_kernel(const int32_t* pred, int n_pred, const int32_t* gold,
+                                                     int n_gold, int32_t* n_common, float* recall,
+                                                     int staged) {
   extern __shared__ int32_t s_gold[];
   __shared__ int s_hits[kRecallWarps];
   wait_for_predecessor();

@@ -16,11 +16,10 @@ constexpr int kQsumThreads = 256;
 // qsum[u][d] = sum over the unit's G*W query rows of q[r][d], fp32. One block per unit: a thread takes
 // eight dims (16 bytes) of every n-th row, and the n partial sums are added in order, so the result
 // does not depend on the launch. Bound: latency (512 units of 128 rows: 22 us with one dim per thread
-// and all rows in turn). Block 0 also clears the workspace header
-// from word hdr_from on.
+// and all rows in turn). Block 0 also clears the workspace header from word hdr_from on.
 __global__ void __launch_bounds__(kQsumThreads)
-qsum_kernel(const __nv_bfloat16* __restrict__ q, float* __restrict__ qsum, int32_t* __restrict__ hdr, int hdr_from,
-            int Bt, int Hkv, int G, int W, int D, int64_t s_layer, int64_t s_batch, int64_t s_head, int64_t s_pos) {
+qsum_kernel(const __nv_bfloat16* q, float* qsum, int32_t* hdr, int hdr_from, int Bt, int Hkv, int G, int W, int D,
+            int64_t s_layer, int64_t s_batch, int64_t s_head, int64_t s_pos) {
   __shared__ float s_part[kQsumThreads * 8];
   wait_for_predecessor();
   allow_successor();
@@ -60,6 +59,8 @@ qsum_kernel(const __nv_bfloat16* __restrict__ q, float* __restrict__ qsum, int32
 constexpr int kRawThreads = 256;
 constexpr int kRawKeysPerBlock = 1024;  // 8 warps x 4 rounds x 32 keys
 
+// (The read-only path: K is complete before the kernel that uses this can start, because the kernel of the
+// query sums, its predecessor, waits for what was before it before it lets any successor start.)
 __device__ __forceinline__ uint4 ld_stream16(const void* p) {
   uint4 v;
   asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
@@ -73,9 +74,9 @@ __device__ __forceinline__ uint4 ld_stream16(const void* p) {
 // are then added across lanes by recursive halving (15 shuffles instead of 64), which leaves the
 // total of key i in lane i: one coalesced 128-byte store per warp and round.
 __global__ void __launch_bounds__(kRawThreads) score_raw_d128_kernel(
-    const __nv_bfloat16* __restrict__ k, const float* __restrict__ qsum, float* __restrict__ colsum,
-    int Bt, int Hkv, int L_alloc, int L_pad, float scale, int64_t s_layer, int64_t s_batch,
-    int64_t s_head, int64_t s_pos, const __grid_constant__ SeqLens sl) {
+    const __nv_bfloat16* k, const float* qsum, float* colsum, int Bt, int Hkv, int L_alloc, int L_pad,
+    float scale, int64_t s_layer, int64_t s_batch, int64_t s_head, int64_t s_pos,
+    const __grid_constant__ SeqLens sl) {
   allow_successor();
   wait_for_predecessor();  // the query sums
   const int64_t u = blockIdx.x;
@@ -140,11 +141,10 @@ __global__ void __launch_bounds__(kRawThreads) score_raw_d128_kernel(
 }
 
 // Any head_dim that is a multiple of 8 (up to 256): one thread per key, qsum in shared memory.
-__global__ void score_raw_any_kernel(const __nv_bfloat16* __restrict__ k,
-                                     const float* __restrict__ qsum, float* __restrict__ colsum,
-                                     int Bt, int Hkv, int D, int L_alloc, int L_pad, float scale,
-                                     int64_t s_layer, int64_t s_batch, int64_t s_head,
-                                     int64_t s_pos, const __grid_constant__ SeqLens sl) {
+__global__ void score_raw_any_kernel(const __nv_bfloat16* k, const float* qsum, float* colsum, int Bt, int Hkv,
+                                     int D, int L_alloc, int L_pad, float scale, int64_t s_layer,
+                                     int64_t s_batch, int64_t s_head, int64_t s_pos,
+                                     const __grid_constant__ SeqLens sl) {
   __shared__ float s_q[256];
   allow_successor();
   wait_for_predecessor();  // the query sums
