@@ -60,23 +60,24 @@ __device__ __forceinline__ float pool_at(const float* c, int j, int h, int Ls, f
 }
 
 // Four consecutive positions per thread: three 16-byte loads (rows of column sums are 512-byte aligned)
-// hold every tap of a pooling kernel of up to nine. kPool: pooling kernel at compile time, 0 = kpool,
-// one load per tap. kVec: the score rows allow 16-byte stores.
+// hold every tap of a pooling kernel of up to nine. kPool: pooling kernel at compile time, 0 = kpool: one
+// position per thread and a load per tap. kVec: the score rows allow 16-byte stores.
 // Bound: HBM. 256 units of 32736 scores: 68 us with one position and a load per tap and thread.
 template <int kPool, bool kVec, class Geom>
 __global__ void __launch_bounds__(256)
 pool_kernel(const float* __restrict__ colsum, int L_pad, float* __restrict__ pooled, int kpool, float inv_k,
             int pool_max, int64_t u0, const __grid_constant__ Geom g) {
   const int64_t u = u0 + blockIdx.y;
-  const int j = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
-  if (j >= g.Ls_full) return;
   const int Ls = unit_scored(g, u);
   const float* c = colsum + u * L_pad;
-  float r[4];
   if constexpr (kPool == 0) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) r[i] = j + i < Ls ? pool_at(c, j + i, kpool / 2, Ls, inv_k, pool_max) : 0.f;
+    const int j = 256 * blockIdx.x + threadIdx.x;
+    if (j < g.Ls_full)
+      pooled[u * (int64_t)g.Ls_full + j] = j < Ls ? pool_at(c, j, kpool / 2, Ls, inv_k, pool_max) : 0.f;
   } else {
+    const int j = 4 * (blockIdx.x * 256 + threadIdx.x);
+    if (j >= g.Ls_full) return;
+    float r[4];
     constexpr int h = kPool / 2;
     static_assert(h <= 4, "one vector of halo");
     const float fill = pool_max ? __int_as_float(0xff800000) : 0.f;
@@ -98,14 +99,14 @@ pool_kernel(const float* __restrict__ colsum, int L_pad, float* __restrict__ poo
       for (int t = -h; t <= h; ++t) acc = pool_max ? fmaxf(acc, x[4 + i + t]) : acc + x[4 + i + t];
       r[i] = j + i < Ls ? (pool_max ? acc : acc * inv_k) : 0.f;
     }
-  }
-  float* dst = pooled + u * (int64_t)g.Ls_full + j;
-  if (kVec) {
-    *reinterpret_cast<float4*>(dst) = make_float4(r[0], r[1], r[2], r[3]);
-  } else {
+    float* dst = pooled + u * (int64_t)g.Ls_full + j;
+    if (kVec) {
+      *reinterpret_cast<float4*>(dst) = make_float4(r[0], r[1], r[2], r[3]);
+    } else {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (j + i < g.Ls_full) dst[i] = r[i];
+      for (int i = 0; i < 4; ++i)
+        if (j + i < g.Ls_full) dst[i] = r[i];
+    }
   }
 }
 
@@ -286,16 +287,18 @@ struct SelArgs {
   int32_t* idx;
   int kpool, pool_max;
   float inv_k;
+  int halo;  // kPool == 0: staged positions on either side, as many as a window reaches (a multiple of 4)
 };
 
 // Shared memory holds the source from kHalo positions before the CTA's first to kHalo behind its last,
 // every 32 floats followed by 4 unused ones: a thread's 16-byte reads of its own 32 floats then hit
-// the banks of its neighbours' once.
+// the banks of its neighbours' once. (kPool == 0 reads it by neighbouring threads, stages args.halo
+// positions on either side and leaves no gaps until the pooled scores change hands.)
 __device__ __forceinline__ int staged_at(int i) { return i + ((i >> 5) << 2); }
 inline size_t staged_floats(int n) { return (size_t)(n + 2 * kHalo + 31) / 32 * 36; }
 
-// kPool: pooling kernel at compile time (1, 3, 5, 7, 9: the window fits the vectors of halo), 0 =
-// args.kpool, kCopy.
+// kPool: pooling kernel at compile time (1, 3, 5, 7, 9: the window fits the vectors of halo), kCopy, or 0 =
+// args.kpool.
 template <int kPool, int kItems, bool kPair, class Geom>
 __global__ void __launch_bounds__(1024, 1)
 pool_select_reg_kernel(const __grid_constant__ SelArgs args, const __grid_constant__ Geom g) {
@@ -318,12 +321,13 @@ pool_select_reg_kernel(const __grid_constant__ SelArgs args, const __grid_consta
   const float fill = kPool != kCopy && args.pool_max ? __int_as_float(0xff800000) : 0.f;
   const float* src = args.src + u * args.src_row;
   {
-    const int n4 = (min(n_own, max(0, Ls - pos0)) + 2 * kHalo + 3) >> 2;  // what any thread reads
-    const float* from = src + pos0 - kHalo;
+    const int halo = kPool == 0 ? args.halo : kHalo;
+    const int n4 = (min(n_own, max(0, Ls - pos0)) + 2 * halo + 3) >> 2;  // what any thread reads
+    const float* from = src + pos0 - halo;
     const bool aligned = kPool != kCopy;  // rows of column sums are 512-byte aligned
 #pragma unroll 4
     for (int i = tid; i < n4; i += n_threads) {
-      const int p = pos0 - kHalo + 4 * i;
+      const int p = pos0 - halo + 4 * i;
       float4 v = make_float4(fill, fill, fill, fill);
       if (aligned && p >= 0 && p + 4 <= Ls) {
         v = __ldcs(reinterpret_cast<const float4*>(from) + i);
@@ -333,7 +337,7 @@ pool_select_reg_kernel(const __grid_constant__ SelArgs args, const __grid_consta
         if (p + 2 < Ls) v.z = __ldcs(from + 4 * i + 2);
         if (p + 3 < Ls) v.w = __ldcs(from + 4 * i + 3);
       }
-      *reinterpret_cast<float4*>(s_c + staged_at(4 * i)) = v;
+      *reinterpret_cast<float4*>(s_c + (kPool == 0 ? 4 * i : staged_at(4 * i))) = v;
     }
   }
   __syncthreads();
@@ -342,27 +346,43 @@ pool_select_reg_kernel(const __grid_constant__ SelArgs args, const __grid_consta
   const int own = tid * kItems, base = pos0 + own;
   const int n_real = min(kItems, max(0, Ls - base));
   uint32_t w[kItems];
-  if (kPool == 0) {
-    const int h = args.kpool / 2;
+  if constexpr (kPool == 0) {
+    // One load per tap. Item k of a thread is position k * n_threads + tid here: neighbouring threads load
+    // neighbouring words, and the pooled scores change hands through shared memory. Positions that do not
+    // exist hold `fill`; a window that reaches beyond the halo finds none there either. Four positions at a
+    // time share the loop over the taps. (256 units of 4088 scores, kernel 31: the whole call 150 us with a
+    // thread's consecutive positions one after the other, 96 so; kernel 65: 221 and 114.)
+    const int h = min(args.kpool / 2, args.halo);
 #pragma unroll
-    for (int k = 0; k < kItems; ++k) {
-      const int i = kHalo + own + k;
-      float pj = s_c[staged_at(i)];
-      if (k < n_real) {
-        if (h <= kHalo) {
-          if (args.pool_max) {
-            for (int t = -h; t <= h; ++t) pj = fmaxf(pj, s_c[staged_at(i + t)]);
-          } else {
-            float acc = 0.f;
-            for (int t = -h; t <= h; ++t) acc += s_c[staged_at(i + t)];
-            pj = acc * args.inv_k;
-          }
-        } else {
-          pj = pool_at(src, base + k, h, Ls, args.inv_k, args.pool_max);
-        }
+    for (int k0 = 0; k0 < kItems; k0 += 4) {
+      const float* c[4];
+      float acc[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        // (beyond the last position: anything)
+        c[k] = s_c + args.halo + min((k0 + k) * n_threads + tid, max(0, Ls - 1 - pos0));
+        acc[k] = args.pool_max ? *c[k] : 0.f;
       }
-      w[k] = __float_as_uint(pj);
+      if (args.pool_max) {
+#pragma unroll 4
+        for (int t = -h; t <= h; ++t)
+#pragma unroll
+          for (int k = 0; k < 4; ++k) acc[k] = fmaxf(acc[k], c[k][t]);
+      } else {
+#pragma unroll 4
+        for (int t = -h; t <= h; ++t)
+#pragma unroll
+          for (int k = 0; k < 4; ++k) acc[k] += c[k][t];
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) w[k0 + k] = __float_as_uint(args.pool_max ? acc[k] : acc[k] * args.inv_k);
     }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) s_c[staged_at(kHalo + k * n_threads + tid)] = __uint_as_float(w[k]);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) w[k] = __float_as_uint(s_c[staged_at(kHalo + own + k)]);
   } else {
     constexpr int h = kPool > 0 ? kPool / 2 : 0;
     static_assert(h <= 4, "one vector of halo");
@@ -588,15 +608,21 @@ void launch_pool(dim3 grid, cudaStream_t stream, const Dims& d, const float* col
 #undef LAQ_POOL
 }
 
+// Floats of shared memory that the kernel for any pooling window (kPool == 0) may take.
+constexpr size_t kMaxWindowed = 56 * 1024;
+// Positions it stages on either side of a CTA's own: what a window reaches of the Ls there are.
+int window_halo(const Dims& d) {
+  const int h = d.kpool / 2 < d.Ls ? d.kpool / 2 : d.Ls;
+  return (h + 3) / 4 * 4;
+}
+
 // Shared memory opt-in of a kernel: a per-device attribute, set once per device and kernel.
 template <class K>
-bool opt_in(K kernel, std::atomic<uint64_t>& devices) {
+bool opt_in(K kernel, size_t bytes, std::atomic<uint64_t>& devices) {
   int dev = 0;
   if (!cuda_ok(cudaGetDevice(&dev))) return false;
   if (dev < 64 && ((devices.load(std::memory_order_acquire) >> dev) & 1u)) return true;
-  if (!cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)(staged_floats(kPairHalf) * sizeof(float)))))
-    return false;
+  if (!cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes))) return false;
   if (dev < 64) devices.fetch_or(1ull << dev, std::memory_order_release);
   return true;
 }
@@ -604,11 +630,16 @@ bool opt_in(K kernel, std::atomic<uint64_t>& devices) {
 template <int kPool, int kItems, bool kPair, class Geom>
 bool launch_select(unsigned units, int threads, cudaStream_t stream, const SelArgs& args, const Geom& g) {
   static std::atomic<uint64_t> devices{0};
-  if (!opt_in(pool_select_reg_kernel<kPool, kItems, kPair, Geom>, devices)) return false;
+  if (!opt_in(pool_select_reg_kernel<kPool, kItems, kPair, Geom>,
+              (kPool == 0 ? kMaxWindowed : staged_floats(kPairHalf)) * sizeof(float), devices))
+    return false;
+  size_t floats = staged_floats(threads * kItems);
+  if (kPool == 0 && floats < (size_t)threads * kItems + 2 * args.halo)
+    floats = (size_t)threads * kItems + 2 * args.halo;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kPair ? 2 * units : units);
   cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = staged_floats(threads * kItems) * sizeof(float);
+  cfg.dynamicSmemBytes = floats * sizeof(float);
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   programmatic_launch(&attr[0]);
@@ -623,12 +654,14 @@ bool launch_select(unsigned units, int threads, cudaStream_t stream, const SelAr
 // Which of the kernels takes units of Ls scores: up to 32768 one CTA with 32 scores per thread, up to
 // 65536 a pair of CTAs. Where the units are so few and short that every one has an SM to itself and
 // waits for its own chain of steps only, 8 scores per thread (one unit of 1016: 14.4 us with 128
-// threads).
+// threads); and where a wide window makes the taps most of the work, which wants more threads to a unit
+// (256 units of 4088, kernel 1001: the whole call 618 us with 32 scores per thread, 208 with 8; kernel
+// 129: 94; kernel 101, still with 32: 134).
 template <int kPool, class Geom>
 bool launch_select_sized(const Dims& d, cudaStream_t stream, const SelArgs& args, const Geom& g) {
   const unsigned units = (unsigned)d.U;
   if (d.Ls > kPairHalf) return launch_select<kPool, 32, true, Geom>(units, 1024, stream, args, g);
-  if (d.U <= 148 && d.Ls <= 8 * 1024)
+  if (d.Ls <= 8 * 1024 && (d.U <= 148 || (kPool == 0 && d.kpool > 128)))
     return launch_select<kPool, 8, false, Geom>(units, ((d.Ls + 7) / 8 + 31) / 32 * 32, stream, args, g);
   return launch_select<kPool, 32, false, Geom>(units, ((d.Ls + 31) / 32 + 31) / 32 * 32, stream, args, g);
 }
@@ -655,7 +688,8 @@ laq_status pool_launch(const Dims& d, const float* colsum, int L_pad, float* poo
   // grid.y limit: launch in slabs of units
   for (int64_t u0 = 0; u0 < d.U; u0 += 65535) {
     const unsigned nu = (unsigned)((d.U - u0 < 65535) ? d.U - u0 : 65535);
-    const dim3 grid((d.Ls + 1023) / 1024, nu);
+    const int per_block = d.kpool > 9 ? 256 : 1024;  // a position per thread, or four
+    const dim3 grid((d.Ls + per_block - 1) / per_block, nu);
     if (has_tables(d)) {
       const SelGeomTables g = geom_tables(d);
       if (vec) launch_pool<true>(grid, stream, d, colsum, L_pad, pooled, u0, g);
@@ -683,6 +717,7 @@ static laq_status select_reg_launch(const Dims& d, bool pool, const float* src, 
   args.kpool = pool ? d.kpool : 1;
   args.pool_max = pool ? d.pool_max : 0;
   args.inv_k = 1.0f / (float)args.kpool;
+  args.halo = pool ? window_halo(d) : 0;
   const bool ok = has_tables(d) ? launch_select_pooled(d, pool, stream, args, geom_tables(d))
                                 : launch_select_pooled(d, pool, stream, args, geom_plain(d));
   if (!ok) return LAQ_ERR_CUDA;
@@ -702,7 +737,10 @@ laq_status select_launch(const Dims& d, const float* pooled, int32_t* idx, cudaS
 laq_status pool_select_launch(const Dims& d, const float* colsum, int L_pad, float* pooled_out,
                               int32_t* idx, cudaStream_t stream, int* launches, bool* done) {
   *done = false;
-  if (!fits_registers(d)) return LAQ_OK;  // the caller uses the two-kernel path
+  // else the caller uses the two-kernel path: units too long, or windows that do not fit next to them
+  if (!fits_registers(d)) return LAQ_OK;
+  const int own = d.Ls < kPairHalf ? (d.Ls + 1023) / 1024 * 1024 : kPairHalf;
+  if (d.kpool > 9 && own + 2 * (size_t)window_halo(d) > kMaxWindowed) return LAQ_OK;
   const laq_status st = select_reg_launch(d, true, colsum, L_pad, pooled_out, idx, stream, launches);
   *done = st == LAQ_OK;
   return st;

@@ -54,3 +54,13 @@ def test_pooling_inside_the_selection_equals_pooling_alone(laq, kernel, mode):
         idx = torch.empty_like(out["idx"])
         laq.laq_select(out["params"], alone, idx)
         assert torch.equal(alone, out["scores"]) and torch.equal(idx, out["idx"])
+
+
+@pytest.mark.parametrize("kernel", [11, 63, 101, 1999])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_wide_pooling_windows(laq, kernel, mode):
+    # one load per tap: windows inside what is staged around a CTA's positions, beyond it, and wider than
+    # the short units themselves; ragged too, where a unit ends inside the row
+    test_pooling_inside_the_selection_equals_pooling_alone(laq, kernel, mode)
+    q, k, v = rand_inputs(1, 3, 8, 2, 128, 1500, 8, seed=kernel, kscale=1.5)
+    compare_all_units(laq, q, k, v, 8, kernel, 50, pool_mode=mode, seq_lens=(1500, 1497, 61))
