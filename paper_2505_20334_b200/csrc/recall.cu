@@ -57,15 +57,16 @@ recall_kernel(const int32_t* pred, int n_pred, const int32_t* gold, int n_gold, 
   }
 }
 
-// Whether a warp per unit is the faster one. Measured on B200: a block adds 1.05 ns to the launch,
-// 0.8 ns more for every 1000 staged positions and 2.9 for every 1000 lookups; a warp 0.15 and 6.5 for every
-// 1000 lookups, but its chain of lookups takes 4 us + 33 ns a lookup however few the units are. us with a
-// warp / with a block, n_pred = n_gold unless given: 64: 10000 units 8.3 / 12.9, 40000 16.5 / 46.2, 2500
-// 4.7 / 4.6; 256: 40000 57.7 / 69.4, 5000 12.4 / 9.9; 1024: 40000 289 / 221, 256 37.0 / 4.6; 128 against
-// 12000: 2500 10.5 / 33.4, 256 8.9 / 4.2.
+// Whether a warp per unit is the faster one. Measured on B200: a block adds 1.05 ns to the launch, 0.8 ns
+// more for every 1000 staged positions (1.6 where M_gold is too long to be staged) and 2.9 for every 1000
+// lookups; a warp 0.15 and 6.5 for every 1000 lookups, but its chain of lookups takes 3 us + 33 ns a lookup
+// however few the units are. us with a warp / with a block, n_pred = n_gold unless given: 64: 10000 units
+// 8.3 / 12.9, 5000 6.2 / 7.2, 2500 5.3 / 4.6; 256: 40000 57.7 / 69.4, 5000 12.4 / 9.9; 1024: 40000 289 / 221,
+// 256 37.0 / 4.6; 128 against 12000: 2500 10.5 / 33.4, 256 8.9 / 4.2; 64 against 20000: 2500 7.3 / 9.2, 1184
+// 7.3 / 4.1; 512 against 20000: 10000 57.5 / 45.2.
 bool recall_by_warps(int64_t n_units, int n_pred, int n_gold, bool staged) {
-  const double stage = staged ? n_gold / 1200.0 : 0.0;
-  return n_pred < 250 + (staged ? n_gold / 5 : 0) && n_units * (1.05 + stage) > 4000.0 + 33.0 * n_pred;
+  const double stage = staged ? n_gold / 1200.0 : 1.6;
+  return n_pred < 250 + (staged ? n_gold / 5 : 0) && n_units * (1.05 + stage) > 3000.0 + 33.0 * n_pred;
 }
 
 }  // namespace
