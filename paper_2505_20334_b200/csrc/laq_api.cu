@@ -96,23 +96,35 @@ static laq_status check_strides_vo(const laq_params* p, bool need_v) {
   return LAQ_OK;
 }
 
+constexpr int kLongUnit = 400;  // tiles of a unit from which its tasks are always long ones (see below)
+
 int choose_tiles_per_task(const Dims& d) {
   const int n_tiles = (d.L + TILE_KEYS - 1) / TILE_KEYS;
   int t = d.tiles_per_task;
   if (t <= 0) {
-    // Measured on B200: 16 tiles (2048 keys) per task where there is much to do. With little, 8: the end
-    // of the launch, when SMs wait for the last tasks, weighs less (128 rows, 16 x 8 units of 12001 to
-    // 2311 keys: 475 -> 434 us; 256 units of 8192 keys 333 -> 320 us), at the price of more hand-offs
-    // (1024 units of 32768 keys: 3.79 -> 3.82 ms). Very long prompts stay with 16: sweep 2 has to trail
-    // by a unit, and twice the tasks would put it out of L2's reach (65536 keys: 770 -> 910 us).
+    // Tasks of 16 tiles (2048 keys) or of 8. Short ones make the end of the launch, when SMs wait for the
+    // last tasks, weigh less; long ones have fewer hand-offs. So the line lies at an amount of work per SM.
+    // Measured on B200 (time with 16 over time with 8, scoring, 128 / 256 rows): 30 tiles per SM 1.14-1.21 /
+    // 1.09-1.26, 60 1.02-1.09 / 1.03-1.12, 100 1.01-1.04 / 1.02-1.06, 150 0.98-1.01 / 1.02, 200 0.96-1.02 /
+    // 0.98-1.01, 300 0.95-0.98 / 0.97-1.01, 700 0.93-0.96 / 0.94-0.98, alike for 4096 to 32768 keys: 160.
+    constexpr int64_t kMuchWork = 24000;  // tiles: 160 for each of the 148 SMs
+    // kLongUnit: a second-sweep task merges the partial statistics of all its unit's first-sweep tasks, so their cost
+    // grows with the unit's length over the square of the task's: 65536 keys 1.07 at 30 tiles per SM, 0.92-0.95
+    // at 55, 0.84-0.87 at 300; 100000 keys 0.69-0.90 throughout; 49152 0.97-1.2 at 20, 1.00 at 60, 0.91 at 300.
+    // uneven: where a batch holds many prompts much shorter than its longest, units end in odd pieces of 16 tiles
+    // and long tasks lose at any amount of work (lengths drawn between 700 and L, 4 prompts: L 6000 1.02-1.25
+    // / 0.98-1.13, 12001 1.04-1.19 / 1.03-1.19, 30000 1.01-1.13 / 0.94-1.11 from 40 to 700 tiles per SM);
+    // lengths within 10 % of each other behave like equal ones (200 tiles per SM 1.00, 600 0.97-0.98). Units
+    // of more than 32768 keys again want the long ones (49152 0.92-0.97 from 150 on).
     int64_t tiles = d.U * (int64_t)n_tiles;
+    bool uneven = false;
     if (d.sl.n > 0) {
       int64_t per_layer = 0;
       for (int b = 0; b < d.Bt; ++b) per_layer += (d.sl.len[b] + TILE_KEYS - 1) / TILE_KEYS;
       tiles = per_layer * d.Hkv * d.NL;
+      uneven = n_tiles <= 256 && 8 * per_layer < 7 * (int64_t)d.Bt * n_tiles;
     }
-    const int64_t much = d.sl.n > 0 ? 40000 : 24000;
-    t = n_tiles >= 400 || (n_tiles >= 64 && tiles >= much) ? 16 : 8;
+    t = n_tiles >= kLongUnit || (n_tiles >= 64 && !uneven && tiles >= kMuchWork) ? 16 : 8;
   }
   if (t > n_tiles) t = n_tiles;
   return t;
@@ -122,7 +134,7 @@ int choose_tiles_per_task(const Dims& d) {
 // units and the lengths of their prompts.
 static int shortest_tiles_per_task(const Dims& d) {
   const int n_tiles = (d.L + TILE_KEYS - 1) / TILE_KEYS;
-  const int t = d.tiles_per_task > 0 ? d.tiles_per_task : (n_tiles >= 400 ? 16 : 8);
+  const int t = d.tiles_per_task > 0 ? d.tiles_per_task : (n_tiles >= kLongUnit ? 16 : 8);
   return t < n_tiles ? t : n_tiles;
 }
 static int longest_tiles_per_task(const Dims& d) {
