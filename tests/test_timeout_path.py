@@ -105,3 +105,38 @@ def test_wait_that_runs_out_in_one_piece_of_a_host_call_is_reported(W):
         hooked.laq_test_withhold_unit(-1)
         hooked.laq_test_withhold_launches(-1)
     assert run() == laq.LAQ_OK and torch.equal(he.h_idx, want)             # the next call starts afresh
+
+
+@pytest.mark.parametrize("G,W,tiles,group", [(4, 16, 2, 0), (4, 32, 0, 0), (8, 32, 0, 0), (4, 32, 0, 2), (4, 16, 0, 2)])
+def test_wait_that_runs_out_in_the_other_scoring_kernels(G, W, tiles, group):
+    # two sweeps with every row held twice (64 rows, tasks sized by the caller), 128 and 256 rows, one column
+    # sum per head; and the cluster kernel with one column sum per head
+    from paper_2505_20334_b200 import binding as laq
+
+    hooked = hooked_library()
+    NL, Bt, Hkv, D, L, kernel, B = 1, 1, 2, 128, 1024, 7, 100
+    g = torch.Generator().manual_seed(W)
+    q = torch.randn((NL, Bt, G * Hkv, W, D), generator=g).to(torch.bfloat16).cuda()
+    k = torch.randn((NL, Bt, Hkv, L, D), generator=g).to(torch.bfloat16).cuda()
+    p = laq.params_for(q, k, W, kernel, B)
+    p.tiles_per_task, p.group_mode = tiles, group
+    ws = laq.alloc_workspace(p, "cuda")
+    scores = torch.zeros((NL, Bt, Hkv * (G if group == 2 else 1), L - W), dtype=torch.float32, device="cuda")
+    stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+
+    def run(lib):
+        assert lib.laq_score(ctypes.byref(p), q.data_ptr(), k.data_ptr(), scores.data_ptr(), ws.data_ptr(),
+                             ws.numel(), stream) == laq.LAQ_OK
+        return lib.laq_last_device_status(ctypes.byref(p), ws.data_ptr(), ws.numel(), stream)
+
+    assert run(hooked) == laq.LAQ_OK
+    want = scores.clone()
+    hooked.laq_test_withhold_unit(1)
+    try:
+        assert run(hooked) == laq.LAQ_ERR_TIMEOUT
+    finally:
+        hooked.laq_test_withhold_unit(-1)
+    for lib in (hooked, laq.lib):
+        scores.zero_()
+        assert run(lib) == laq.LAQ_OK
+        assert torch.equal(scores, want)

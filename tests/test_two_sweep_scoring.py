@@ -5,7 +5,8 @@ import pytest
 import torch
 
 from oracle import laq_oracle as orc
-from test_gpu_parity import laq, rand_inputs  # noqa: F401 (laq is a fixture)
+from parity_util import SCORE_RTOL, score_rel_err
+from test_gpu_parity import compare_all_units, laq, rand_inputs  # noqa: F401 (laq is a fixture)
 
 pytestmark = pytest.mark.gpu
 
@@ -64,3 +65,126 @@ def test_static_scratch_takes_longer_tasks_where_shorter_ones_do_not_fit(laq):  
     # and what does not fit even so (108 units) is refused
     p = laq.make_params(27, 1, 8 * Hkv, Hkv, D, L, W, W, 7, B)
     assert laq.laq_score_static(p, q, k, got, check=False) == laq.LAQ_ERR_WORKSPACE
+
+
+# ------------------------------------------------------------------ which kernel scores
+def evict_with(laq, q, k, v, R, kernel, B, tiles_per_task=0, local_window=0, lens=None, group=0, want=None):  # noqa: F811
+    """laq_evict with the scheduling knob set (a nonzero one keeps units of up to 64 rows with the two
+    sweeps), in the form that compare_all_units takes. `want`: part of the name of the kernel that scores."""
+    qd, kd, vd = q.cuda(), k.cuda(), v.cuda()
+    NL, Bt, Hq, D = q.shape[0], q.shape[1], q.shape[2], q.shape[4]
+    H = Hq if group == laq.LAQ_GROUP_PER_HEAD else k.shape[2]
+    out = {"k_out": torch.empty((NL, Bt, H, B, D), dtype=torch.bfloat16, device="cuda"),
+           "idx": torch.empty((NL, Bt, H, B), dtype=torch.int32, device="cuda"),
+           "scores": torch.empty((NL, Bt, H, k.shape[3] - R), dtype=torch.float32, device="cuda")}
+    out["v_out"] = torch.empty_like(out["k_out"])
+    p = laq.params_for(qd, kd, R, kernel, B, v=vd, out=out["k_out"])
+    p.tiles_per_task, p.local_window, p.group_mode = tiles_per_task, local_window, group
+    p.set_seq_lens(lens)
+    ws = laq.alloc_workspace(p, "cuda")
+
+    def call():
+        laq.laq_evict(p, qd, kd, vd, out["k_out"], out["v_out"], out["idx"], out["scores"], ws)
+        assert laq.laq_last_device_status(p, ws) == laq.LAQ_OK
+    call()
+    if want is not None:
+        assert want in scoring_kernels(call)
+    return dict(out, params=p, ws=ws)
+
+
+def scoring_kernels(call):
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        call()
+        torch.cuda.synchronize()
+    names = " ".join(e.key for e in prof.key_averages())
+    return {n for n in ("score_cluster_kernel", "score_tc_kernel", "simt_stats_kernel") if n in names}
+
+
+TWO_SWEEP = [
+    # NL Bt Hq Hkv D    L     W  W_local k  B  tiles lens        group
+    (1, 1, 4, 1, 8, 700, 17, 0, 3, 60, 0, None, 0),              # head dims below 128, 68 rows
+    (1, 2, 8, 2, 64, 1300, 32, 16, 7, 90, 0, (1300, 401), 0),    # 128 rows
+    (1, 1, 8, 1, 80, 900, 17, 17, 5, 60, 0, None, 0),            # 136 rows: two row blocks
+    (1, 1, 8, 1, 112, 2300, 32, 0, 7, 100, 0, None, 0),          # 256 rows, several tasks
+    (1, 1, 8, 2, 64, 1100, 32, 0, 7, 90, 0, None, 2),            # one column sum per head
+    (1, 1, 4, 1, 96, 640, 64, 0, 7, 100, 0, None, 1),
+    (1, 1, 2, 2, 128, 1500, 1, 0, 7, 60, 4, None, 0),            # up to 64 rows: every row held twice
+    (1, 2, 8, 2, 128, 1030, 16, 8, 7, 90, 1, (1030, 129), 0),
+    (2, 1, 8, 2, 64, 2500, 8, 0, 5, 90, 3, None, 0),
+    (1, 1, 8, 2, 128, 1300, 16, 0, 7, 90, 4, None, 1),           # and one column sum per head
+    (1, 2, 8, 2, 128, 1300, 8, 0, 7, 90, 4, (1300, 500), 2),
+    (1, 1, 4, 2, 72, 900, 32, 0, 7, 90, 2, None, 2),
+    (1, 1, 8, 2, 128, 16385, 16, 0, 5, 64, 0, None, 0),          # too long for a cluster's tensor memory
+]
+
+
+@pytest.mark.parametrize("case", TWO_SWEEP, ids=[f"D{c[4]}-M{c[2] // c[3] * c[6]}-L{c[5]}-g{c[12]}" for c in TWO_SWEEP])
+def test_two_sweeps_match_oracle(laq, case):  # noqa: F811
+    NL, Bt, Hq, Hkv, D, L, W, Wl, kernel, B, tiles, lens, group = case
+    q, k, v = rand_inputs(NL, Bt, Hq, Hkv, D, L, W, seed=L + D + W, kscale=1.5)
+    if lens is not None:
+        for b, Lb in enumerate(lens):
+            k[:, b, :, Lb:] = float("nan")
+    out = evict_with(laq, q, k, v, W, kernel, B, tiles, Wl, lens, group, want="score_tc_kernel")
+    compare_all_units(laq, q, k, v, W, kernel, B, out=out, local_window=Wl, seq_lens=lens, group_mode=group)
+
+
+CUDA_CORES = [
+    (1, 1, 3, 1, 136, 500, 32, 0, 7, 60, None, 0),               # head dims above 128 with more than 64 rows
+    (1, 2, 8, 2, 192, 900, 32, 16, 5, 90, (900, 333), 0),
+    (1, 1, 8, 1, 256, 300, 32, 32, 7, 64, None, 0),              # 256 rows of 256 dims
+    (1, 1, 8, 1, 128, 700, 9, 0, 7, 60, None, 1),                # windows that straddle the groups of four rows
+    (1, 2, 4, 1, 128, 1200, 25, 5, 3, 60, (1200, 130), 2),
+    (1, 1, 8, 2, 200, 600, 20, 0, 7, 60, None, 2),
+]
+
+
+@pytest.mark.parametrize("case", CUDA_CORES, ids=[f"D{c[4]}-M{c[2] // c[3] * c[6]}-g{c[11]}" for c in CUDA_CORES])
+def test_cuda_cores_match_oracle(laq, case):  # noqa: F811
+    NL, Bt, Hq, Hkv, D, L, W, Wl, kernel, B, lens, group = case
+    q, k, v = rand_inputs(NL, Bt, Hq, Hkv, D, L, W, seed=L + D + W, kscale=1.5)
+    if lens is not None:
+        for b, Lb in enumerate(lens):
+            k[:, b, :, Lb:] = float("nan")
+    out = evict_with(laq, q, k, v, W, kernel, B, 0, Wl, lens, group, want="simt_stats_kernel")
+    compare_all_units(laq, q, k, v, W, kernel, B, out=out, local_window=Wl, seq_lens=lens, group_mode=group)
+    # and on the library's own scratch, whose last contents another problem left there
+    if group == 0:
+        qd, kd = q.cuda(), k.cuda()
+        got = torch.full_like(out["scores"], float("nan"))
+        laq.laq_score_static(out["params"], qd, kd, got)
+        assert torch.equal(got, out["scores"])
+
+
+def test_layout_that_tma_cannot_describe_is_scored_on_cuda_cores(laq):  # noqa: F811
+    # strides of 2^40 bytes and more are beyond a tensor map; with one layer the stride is never used
+    for W in (8, 32):
+        q, k, v = rand_inputs(1, 1, 8, 2, 128, 500, W, seed=W, kscale=1.5)
+        out = laq.evict(q.cuda(), k.cuda(), v.cuda(), 70, want_scores=True)
+        p, qd, kd = out["params"], q.cuda(), k.cuda()
+        p.k_stride_layer = 1 << 40
+        got = torch.zeros_like(out["scores"])
+
+        def call():
+            laq.laq_score(p, qd, kd, got, out["ws"])
+        call()
+        assert "simt_stats_kernel" in scoring_kernels(call)
+        want = orc.evict(q, k, None, W, 7, 70, want_idx=False)["scores"]
+        assert score_rel_err(got.cpu().numpy(), want) <= SCORE_RTOL
+
+
+@pytest.mark.parametrize("W,G,tiles", [(16, 4, 4), (2, 4, 8), (32, 4, 0), (32, 8, 0)])
+def test_extreme_logits_and_late_maximum_in_two_sweeps(laq, W, G, tiles):  # noqa: F811
+    # logits of +-hundreds and a very large key late in the prompt: the reference of sweep 1 has to move
+    # several times, also in the middle of a task, and sweep 2 sees probabilities below the smallest normal
+    Hkv, D, L, kernel, B = 2, 128, 4200, 7, 150
+    g = torch.Generator().manual_seed(404 + W)
+    q = torch.randn((1, 1, G * Hkv, W, D), generator=g).to(torch.bfloat16)
+    k = (torch.randn((1, 1, Hkv, L, D), generator=g) * 12.0).to(torch.bfloat16)
+    v = torch.randn((1, 1, Hkv, L, D), generator=g).to(torch.bfloat16)
+    for h in range(Hkv):
+        qbar = q[0, 0, h * G:(h + 1) * G].float().mean(dim=(0, 1))
+        k[0, 0, h, 3900] = (qbar * 60.0).to(torch.bfloat16)
+    for Wl in (0, min(W, 1)):
+        out = evict_with(laq, q, k, v, W, kernel, B, tiles, Wl, want="score_tc_kernel")
+        compare_all_units(laq, q, k, v, W, kernel, B, out=out, local_window=Wl)
