@@ -308,6 +308,15 @@ def config_dict(cfg, B, args, lens=None):
             "l2": "inputs (K+V) far larger than the 126 MB L2; no flush needed"}
 
 
+def scored_in_a_cluster(rows: int, prompt_len: int, args) -> bool:
+    """Whether units of this size take the one-sweep kernel (head_dim 128): no scheduling knobs, up to 64
+    rows, and their 128-key tiles fit the tensor memory of 16 SMs (512 columns each, one per row rounded up
+    to a power of two of at least 16)."""
+    stride = max(16, 1 << (rows - 1).bit_length())
+    return (rows <= 64 and not (args.tiles_per_task or args.lag_tasks) and
+            -(-prompt_len // 128) <= 16 * (512 // stride))
+
+
 def main():
     args = parse_args()
     if args.gpus > 1 and "WORLD_SIZE" not in os.environ:
@@ -442,7 +451,9 @@ def main():
         traffic = NCU_TRAFFIC_BYTES_RAW if captured and not args.layers else None
     else:
         traffic = NCU_SMALL_CASE_DRAM_BYTES * cfg.units / NCU_SMALL_CASE_UNITS if captured else None
-    roofline = {"bound": "hbm", "kernel": "score_raw_d128_kernel" if raw else "score_tc_kernel",
+    one_sweep = not raw and scored_in_a_cluster(cfg.rows, L, args)
+    roofline = {"bound": "hbm", "kernel": ("score_raw_d128_kernel" if raw else
+                                           "score_cluster_kernel" if one_sweep else "score_tc_kernel"),
                 "achieved": achieved, "peak": peak,
                 "unit": "GB/s", "frac": achieved / peak, "traffic": traffic,
                 "traffic_source": None if traffic is None else (
@@ -452,12 +463,14 @@ def main():
                 "kernel_ms": score_ms, "frac_of_nominal_8TBs": achieved / NOMINAL_HBM_GBS}
     if kernel_ns > 0 and not raw:
         sms_ = torch.cuda.get_device_properties(dev).multi_processor_count
-        tile_sweeps = 2.0 * NL * Hkv * sum(-(-x // 128) for x in (lens or [L] * Bt)) / sms_
+        sweeps = 1.0 if one_sweep else 2.0
+        tile_sweeps = sweeps * NL * Hkv * sum(-(-x // 128) for x in (lens or [L] * Bt)) / sms_
         roofline["in_kernel"] = {"sm_mhz": kernel_cycles / kernel_ns * 1e3, "sm_cycles": kernel_cycles,
+                                 "sweeps": int(sweeps),
                                  "cycles_per_128key_tile_and_sweep_per_sm": kernel_cycles / tile_sweeps,
                                  "source": "clock64 / globaltimer of the kernel's first block, last step"}
     # The scoring kernel's busiest unit is the MUFU: two base-2 exponentials per (row, key) pair
-    # (one per sweep) at 16 per clock and SM.
+    # (one per sweep or pass) at 16 per clock and SM.
     n_exp = 2.0 * NL * Hkv * cfg.rows * tokens_per_step
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     mufu_peak = 16.0 * sms * (clocks.get("sm_max_mhz") or 1965) * 1e6
