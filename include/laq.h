@@ -108,7 +108,7 @@ typedef struct {
   int32_t batch;       /* Bt >= 1 */
   int32_t n_q_heads;   /* Hq, a multiple of n_kv_heads */
   int32_t n_kv_heads;  /* Hkv >= 1; query head h reads KV head h / G */
-  int32_t head_dim;    /* D, a multiple of 8 up to 256 (up to 128 on tensor cores) */
+  int32_t head_dim;    /* D, a multiple of 8 up to 256 (on tensor cores up to 128, above that with G*W <= 64) */
   int32_t prompt_len;  /* L */
   int32_t window_len;  /* W >= 1 lookahead queries per query head; G*W <= 256 */
   int32_t keep_tail;   /* R, 0 <= R < B: last R positions always kept and never scored */
@@ -336,7 +336,8 @@ LAQ_API void laq_set_stage_events(void* score_begin, void* score_end);
  * recorded about itself: the SM clock cycles and the wall-clock nanoseconds its first thread block
  * ran for (the block is resident for the whole launch). cycles / nanoseconds is the SM clock the
  * kernel really ran at; the board lowers it under load, so cycle counts and times are reported
- * separately. Both read 0 if the call took another scoring path (head_dim other than 128, raw mode).
+ * separately. Both read 0 if the call took another scoring path (CUDA cores, raw mode).
+ * After laq_evict_host in pieces they are the last piece's.
  *   ws, ws_bytes   the workspace of that call (device)
  *   sm_cycles, nanoseconds   HOST, out
  * Errors: LAQ_ERR_INVALID_ARG, LAQ_ERR_CUDA.

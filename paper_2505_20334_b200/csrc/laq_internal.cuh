@@ -122,7 +122,7 @@ int64_t test_withhold_unit();
 // Raw-logit mode (Eq. 4 read literally): one streaming pass over K on CUDA cores.
 laq_status score_raw_launch(const laq_params& p, const Dims& d, const Workspace& w, const void* q,
                             const void* k, char* ws, cudaStream_t stream, int* launches);
-// CUDA-core path for every other shape.
+// CUDA-core path for every other shape and layout.
 laq_status score_simt_launch(const laq_params& p, const Dims& d, const Workspace& w,
                              const void* q, const void* k, char* ws, cudaStream_t stream,
                              int* launches);

@@ -6,8 +6,9 @@
 // logits twice (two sweeps over K). Here a cluster of C CTAs (one per SM) owns a whole unit: CTA r
 // takes the 128-key tiles r, r + C, r + 2C, ... and keeps their logits S^T = K Q^T (keys on the TMEM
 // lanes, fp32) in tensor memory while the row sums are formed and exchanged:
-//   pass 1   every thread owns one key of a tile and adds 2^(t[r][j] - ref_r) into one accumulator
-//            per row; the cross-lane sum is taken once per unit, not once per tile;
+//   pass 1   adds 2^(t[r][j] - ref_r) over the keys. The logits are read in the fragment layout: a
+//            thread holds a quarter of the rows, one accumulator each, for a quarter of its warp's
+//            keys, and the cross-lane sum is taken once per unit, not once per tile;
 //   exchange each CTA sends its (ref, sum) pairs to every CTA of the cluster through distributed
 //            shared memory (st.async), and each merges them into b_r = m_r + log2(l_r);
 //   pass 2   reads the same logits from tensor memory again and sums 2^(t[r][j] - b_r) over the rows.
@@ -19,17 +20,17 @@
 // tile's TMEM slot goes back to the MMA issuer when pass 2 has read it, whatever unit comes next.
 // 512 TMEM columns hold 512 / stride tiles, stride = rows rounded up to a power of two >= 16.
 //
-// The reference ref_r of a warp is the logit of the first key its first lane holds. Sums are scale
+// The reference ref_r of a warp is the logit of its first key. Sums are scale
 // free in fp32, so any reference within 2^100 of the largest logit will do; a warp whose sums
 // overflow that (a key 69 nats above the reference) takes the maximum from tensor memory and redoes
 // its sums.
 //
 // Warp roles (640 threads):
 //   warp 0       TMA producer (one lane)
-//   warp 1       tcgen05.mma issuer (one lane); owns the tensor memory
+//   warp 1       tcgen05.mma issuer (an elected lane of the converged warp); owns the tensor memory
 //   warps 2-3    exchange: merge the warps' pairs, send them, wait for the cluster's, publish -b_r
-//   warps 4-11   pass 1, two warpgroups on alternate tiles, all rows of a key in one thread
-//   warps 12-19  pass 2, likewise
+//   warps 4-11   pass 1, two warpgroups on alternate tiles
+//   warps 12-19  pass 2, likewise, all rows of a key in one thread
 // Every wait is bounded, as in score_tc.cu; clusters meet at a cluster barrier before they leave, so
 // that no CTA exits while another may still write into its shared memory.
 #include <cuda.h>

@@ -1,5 +1,7 @@
 // CUDA-core scoring path (steps 1-3 of the unit computation, Eq. 4 read as attention weights)
-// for the shapes the tensor-core kernel does not take (head_dim other than 128).
+// for what the tensor-core kernels do not take: head dims above 128 with more than 64 rows or units too long
+// for a cluster, per-head sums of more than 64 rows whose windows straddle the groups of four, and layouts
+// beyond a tensor map.
 // Three launches: partial row statistics per key chunk, their merge into one offset per row,
 // and the normalised column sums. fp32 arithmetic from bf16 inputs.
 #include <cuda_bf16.h>

@@ -82,8 +82,8 @@ SHAPES = [
     (1, 1, 2, 2, 128, 300, 8, 3, 40),      # G = 1, M = 8
     (1, 1, 6, 2, 128, 640, 5, 3, 33),      # M = 15 (not a multiple of 16)
     (1, 1, 4, 2, 128, 50, 4, 7, 20),       # L smaller than one tile
-    (1, 1, 8, 2, 64, 500, 8, 7, 90),       # head_dim 64: CUDA-core path
-    (1, 1, 4, 1, 256, 260, 8, 5, 48),      # head_dim 256: CUDA-core path
+    (1, 1, 8, 2, 64, 500, 8, 7, 90),       # head_dim 64
+    (1, 1, 4, 1, 256, 260, 8, 5, 48),      # head_dim 256
     (2, 2, 8, 2, 128, 4500, 1, 7, 64),     # one lookahead step (Section 6.2): M = 4
     (1, 1, 8, 2, 128, 2500, 2, 5, 40),     # two lookahead steps: M = 8
     (1, 1, 16, 2, 128, 1100, 2, 3, 50),    # M = 16
@@ -218,7 +218,7 @@ LOCAL_SHAPES = [
     (1, 1, 4, 1, 128, 777, 32, 16, 7, 200),   # M = 128, ragged last tile
     (1, 1, 8, 1, 128, 1536, 32, 32, 5, 64),   # M = 256, local queries only (SnapKV-style window)
     (1, 1, 4, 2, 128, 200, 6, 5, 3, 30),      # window length that is not a power of two
-    (1, 1, 8, 2, 64, 500, 8, 4, 7, 90),       # head_dim 64: CUDA-core path
+    (1, 1, 8, 2, 64, 500, 8, 4, 7, 90),       # head_dim 64
 ]
 
 
@@ -292,7 +292,7 @@ RAGGED_SHAPES = [
     (2, 2, 4, 1, 128, 3000, 32, 16, 5, 200, (2049, 3000)),       # M = 128, LAQ++ window at each prompt's own end
     (1, 2, 8, 1, 128, 1536, 32, 0, 7, 64, (700, 1536)),          # M = 256
     (1, 4, 4, 2, 128, 600, 8, 8, 3, 40, (41, 128, 129, 600)),    # shortest legal prompt, tile edges
-    (1, 2, 8, 2, 64, 500, 8, 4, 7, 90, (500, 200)),              # head_dim 64: CUDA-core path
+    (1, 2, 8, 2, 64, 500, 8, 4, 7, 90, (500, 200)),              # head_dim 64
 ]
 
 
@@ -373,7 +373,7 @@ def test_host_buffer_entry_point_equals_device_run(laq):
 
 
 def test_evict_can_be_captured_in_a_cuda_graph(laq):
-    # laq_evict only enqueues stream work (a memset and kernels): after one eager call it can be
+    # laq_evict only enqueues stream work (kernels, for some sizes after a memset): after one eager call it can be
     # captured and replayed, and the replay gives the eager call's bits on new inputs
     NL, Bt, Hq, Hkv, D, L, W, kernel, B = 2, 2, 8, 2, 128, 1500, 16, 7, 100
     q, k, v = (t.cuda() for t in rand_inputs(NL, Bt, Hq, Hkv, D, L, W, seed=91))
@@ -626,8 +626,8 @@ GROUP_SHAPES = [
     (2, 1, 8, 2, 128, 900, 8, 5, 64),      # four heads per chunk, M = 32
     (1, 1, 8, 2, 128, 700, 16, 7, 90),     # two heads per chunk, M = 64
     (1, 1, 4, 1, 128, 640, 64, 7, 100),    # a head spans two chunks, M = 256
-    (1, 1, 6, 2, 128, 500, 5, 3, 33),      # W = 5: heads straddle the groups of four -> CUDA-core path
-    (1, 1, 8, 2, 64, 400, 8, 7, 60),       # head_dim 64: CUDA-core path
+    (1, 1, 6, 2, 128, 500, 5, 3, 33),      # W = 5: heads straddle the groups of four
+    (1, 1, 8, 2, 64, 400, 8, 7, 60),       # head_dim 64
 ]
 
 

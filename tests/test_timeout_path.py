@@ -1,7 +1,7 @@
-"""The bounded device-side waits of the scoring kernel, exercised the only way that is safe on a
+"""The bounded device-side waits of the scoring kernels, exercised the only way that is safe on a
 shared GPU: a wait is made to run out by a flag that nothing sets. A copy of the library built with
-a test hook and a ~1.5 ms wait limit withholds the row statistics of one unit; the second sweep of
-that unit then waits for them in vain, gives up, the whole kernel returns, the host reads
+a test hook and a ~1.5 ms wait limit withholds the row statistics of one unit; whoever waits for
+them (the unit's second sweep, or the other CTAs of its cluster) gives up, the whole kernel returns, the host reads
 LAQ_ERR_TIMEOUT, and the next ordinary call on the same workspace works. Nothing traps or faults."""
 import ctypes
 

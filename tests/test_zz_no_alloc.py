@@ -68,7 +68,7 @@ def test_static_scratch_matches_workspace_entry_point_twice_in_a_row(laq):
     assert score_rel_err(got, want) <= SCORE_RTOL
     # and against the CPU oracle, so that a mistake shared by both entry points cannot pass
     assert score_rel_err(got, _oracle_scores(q, k, 8, 5, 64).reshape(got.shape)) <= SCORE_RTOL
-    # and the CUDA-core path (head_dim 64) shares the same scratch
+    # and head_dim 64 shares the same scratch
     q, k = _inputs(1, 1, 8, 2, 64, 500, 8, seed=103)
     got, want = _both(laq, q, k, 8, 7, 90)  # first use of these kernels: they load here
     assert score_rel_err(got, want) <= SCORE_RTOL
