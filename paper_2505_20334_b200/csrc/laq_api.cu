@@ -96,8 +96,6 @@ static laq_status check_strides_vo(const laq_params* p, bool need_v) {
   return LAQ_OK;
 }
 
-constexpr int kLongUnit = 400;  // tiles of a unit from which its tasks are always long ones (see below)
-
 int choose_tiles_per_task(const Dims& d) {
   const int n_tiles = (d.L + TILE_KEYS - 1) / TILE_KEYS;
   int t = d.tiles_per_task;
@@ -108,14 +106,16 @@ int choose_tiles_per_task(const Dims& d) {
     // 1.09-1.26, 60 1.02-1.09 / 1.03-1.12, 100 1.01-1.04 / 1.02-1.06, 150 0.98-1.01 / 1.02, 200 0.96-1.02 /
     // 0.98-1.01, 300 0.95-0.98 / 0.97-1.01, 700 0.93-0.96 / 0.94-0.98, alike for 4096 to 32768 keys: 160.
     constexpr int64_t kMuchWork = 24000;  // tiles: 160 for each of the 148 SMs
-    // kLongUnit: a second-sweep task merges the partial statistics of all its unit's first-sweep tasks, so their cost
+    // A second-sweep task merges the partial statistics of all its unit's first-sweep tasks, so their cost
     // grows with the unit's length over the square of the task's: 65536 keys 1.07 at 30 tiles per SM, 0.92-0.95
     // at 55, 0.84-0.87 at 300; 100000 keys 0.69-0.90 throughout; 49152 0.97-1.2 at 20, 1.00 at 60, 0.91 at 300.
-    // uneven: where a batch holds many prompts much shorter than its longest, units end in odd pieces of 16 tiles
+    constexpr int kLongUnit = 400;  // tiles of a unit from which its tasks are always long ones
+    // Where a batch holds many prompts much shorter than its longest, units end in odd pieces of 16 tiles
     // and long tasks lose at any amount of work (lengths drawn between 700 and L, 4 prompts: L 6000 1.02-1.25
     // / 0.98-1.13, 12001 1.04-1.19 / 1.03-1.19, 30000 1.01-1.13 / 0.94-1.11 from 40 to 700 tiles per SM);
     // lengths within 10 % of each other behave like equal ones (200 tiles per SM 1.00, 600 0.97-0.98). Units
-    // of more than 32768 keys again want the long ones (49152 0.92-0.97 from 150 on).
+    // of more than 32768 keys again want the long ones (49152 0.92-0.97 from 150 on). So batches count as
+    // uneven that hold less than 7/8 of their allocated tiles, up to 256 tiles per unit.
     int64_t tiles = d.U * (int64_t)n_tiles;
     bool uneven = false;
     if (d.sl.n > 0) {
@@ -128,26 +128,6 @@ int choose_tiles_per_task(const Dims& d) {
   }
   if (t > n_tiles) t = n_tiles;
   return t;
-}
-
-// The bounds of what choose_tiles_per_task may return for units of d.L positions, whatever the number of
-// units and the lengths of their prompts.
-static int shortest_tiles_per_task(const Dims& d) {
-  const int n_tiles = (d.L + TILE_KEYS - 1) / TILE_KEYS;
-  const int t = d.tiles_per_task > 0 ? d.tiles_per_task : (n_tiles >= kLongUnit ? 16 : 8);
-  return t < n_tiles ? t : n_tiles;
-}
-static int longest_tiles_per_task(const Dims& d) {
-  const int n_tiles = (d.L + TILE_KEYS - 1) / TILE_KEYS;
-  const int t = d.tiles_per_task > 0 ? d.tiles_per_task : (n_tiles >= 64 ? 16 : 8);
-  return t < n_tiles ? t : n_tiles;
-}
-
-bool plan_workspace_within(const Dims& d, size_t bytes, size_t Workspace::*end, Workspace* w) {
-  plan_workspace(d, choose_tiles_per_task(d), w);
-  if (w->*end <= bytes) return true;
-  plan_workspace(d, longest_tiles_per_task(d), w);
-  return w->*end <= bytes;
 }
 
 void plan_workspace(const Dims& d, int tiles_per_task, Workspace* w) {
@@ -179,6 +159,17 @@ void plan_workspace(const Dims& d, int tiles_per_task, Workspace* w) {
   w->off_idx = off;
   off = align_up(off + sel_units * d.B * sizeof(int32_t), 256);
   w->total = off;
+}
+
+// The size is that of the shortest tasks choose_tiles_per_task may pick for any number of units and any
+// lengths of their prompts: a workspace is sized once and kept for other batches.
+size_t workspace_bytes(const Dims& d) {
+  constexpr int kShortest = 8;
+  const int n_tiles = (d.L + TILE_KEYS - 1) / TILE_KEYS;
+  const int t = d.tiles_per_task > 0 ? d.tiles_per_task : kShortest;
+  Workspace w;
+  plan_workspace(d, t < n_tiles ? t : n_tiles, &w);
+  return w.total;
 }
 
 static bool use_tensor_core_path(const Dims& d) { return d.D <= 128 && d.M <= 256; }
@@ -233,9 +224,9 @@ laq_status selection_source(const Dims& d, const Workspace& w, char* ws, cudaStr
 
 // Plans the workspace of a call inside the caller's `ws`.
 static laq_status plan_in_ws(const Dims& d, const void* ws, size_t ws_bytes, Workspace* w) {
-  if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0 ||
-      !plan_workspace_within(d, ws_bytes, &Workspace::total, w))
+  if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0 || ws_bytes < workspace_bytes(d))
     return LAQ_ERR_WORKSPACE;
+  plan_workspace(d, choose_tiles_per_task(d), w);  // (no larger)
   return LAQ_OK;
 }
 
@@ -269,9 +260,7 @@ void laq_params_dense_strides(laq_params* p) {
 size_t laq_workspace_bytes(const laq_params* p) {
   Dims d;
   if (derive_dims(p, &d) != LAQ_OK) return 0;
-  Workspace w;
-  plan_workspace(d, shortest_tiles_per_task(d), &w);
-  return w.total;
+  return workspace_bytes(d);
 }
 
 laq_status laq_score(const laq_params* p, const void* q, const void* k, float* scores, void* ws,

@@ -88,13 +88,10 @@ constexpr int TILE_KEYS = 128;
 
 laq_status derive_dims(const laq_params* p, Dims* d);
 void plan_workspace(const Dims& d, int tiles_per_task, Workspace* w);
-// Tiles per task of a call. It may look at the number of units and at the prompts' lengths; the size
-// laq_workspace_bytes reports may not, because a workspace is sized once and kept for later batches. That
-// one is therefore planned with the shortest tasks (the most partial statistics) the units may get.
+// Tiles per task of a call: looks at the number of units and at the prompts' lengths.
 int choose_tiles_per_task(const Dims& d);
-// Plans a call's workspace so that `end` (total or one of the offsets) lies within `bytes`: with the tasks
-// it would choose, or else with the longest, which leave the fewest partial statistics. False: neither fits.
-bool plan_workspace_within(const Dims& d, size_t bytes, size_t Workspace::*end, Workspace* w);
+// What a caller's workspace must hold: depends on the allocated sizes only.
+size_t workspace_bytes(const Dims& d);
 
 // Host-side checks and the scoring dispatch shared by every entry point that scores.
 laq_status check_strides_qk(const laq_params* p);

@@ -53,9 +53,12 @@ extern "C" laq_status laq_score_static(const laq_params* p, const void* q, const
       (reinterpret_cast<uintptr_t>(k) & 15u) || (reinterpret_cast<uintptr_t>(scores) & 3u))
     return LAQ_ERR_INVALID_ARG;
   if ((st = check_strides_qk(p)) != LAQ_OK) return st;
-  // everything up to and including the column sums is needed; the caller supplies the scores
   Workspace w;
-  if (!plan_workspace_within(d, kStaticScratchBytes, &Workspace::off_pooled, &w)) return LAQ_ERR_WORKSPACE;
+  plan_workspace(d, choose_tiles_per_task(d), &w);
+  // longer tasks leave fewer partial statistics: what does not fit otherwise may fit with them
+  if (w.off_pooled > kStaticScratchBytes && d.tiles_per_task <= 0) plan_workspace(d, 16, &w);
+  // everything up to and including the column sums is needed; the caller supplies the scores
+  if (w.off_pooled > kStaticScratchBytes) return LAQ_ERR_WORKSPACE;
   void* base = nullptr;
   if ((st = static_scratch(&base)) != LAQ_OK) return st;
   char* ws = static_cast<char*>(base);

@@ -157,7 +157,7 @@ def test_group_mode_and_streaming_arguments_are_checked_on_the_host(binding):
 
 @pytest.mark.parametrize("rows", [32, 128, 256])
 @pytest.mark.parametrize("layers,batch,length", [(1, 4, 1000), (12, 4, 12001), (16, 4, 12001), (60, 4, 12001),
-                                                 (3, 2, 8192), (8, 1, 32768), (4, 4, 51000), (4, 4, 65536)])
+                                                 (3, 2, 8192), (8, 1, 32768), (4, 4, 51000), (4, 4, 51200), (4, 4, 65536)])
 def test_workspace_depends_on_allocated_sizes_only(binding, rows, layers, batch, length):
     # a workspace is sized once and kept for later batches: shorter prompts, fewer layers and shorter
     # allocations must not need more of it
@@ -173,5 +173,7 @@ def test_workspace_depends_on_allocated_sizes_only(binding, rows, layers, batch,
         assert binding.laq_workspace_bytes(p) == base
     for n in range(1, layers):
         assert binding.laq_workspace_bytes(params(n, batch, length)) < base
-    for n_pos in range(200, length, 997):
-        assert binding.laq_workspace_bytes(params(layers, batch, n_pos)) < base
+    fake = ctypes.c_void_p(4096)                     # refused on the host: nothing is read
+    assert binding.lib.laq_score(ctypes.byref(p), fake, fake, fake, fake, base - 1, None) == binding.LAQ_ERR_WORKSPACE
+    for n_pos in [*range(200, length, 997), length - 1]:
+        assert binding.laq_workspace_bytes(params(layers, batch, n_pos)) <= base
