@@ -110,21 +110,25 @@ int choose_tiles_per_task(const Dims& d) {
     // grows with the unit's length over the square of the task's: 65536 keys 1.07 at 30 tiles per SM, 0.92-0.95
     // at 55, 0.84-0.87 at 300; 100000 keys 0.69-0.90 throughout; 49152 0.97-1.2 at 20, 1.00 at 60, 0.91 at 300.
     constexpr int kLongUnit = 400;  // tiles of a unit from which its tasks are always long ones
-    // Where a batch holds many prompts much shorter than its longest, units end in odd pieces of 16 tiles
-    // and long tasks lose at any amount of work (lengths drawn between 700 and L, 4 prompts: L 6000 1.02-1.25
-    // / 0.98-1.13, 12001 1.04-1.19 / 1.03-1.19, 30000 1.01-1.13 / 0.94-1.11 from 40 to 700 tiles per SM);
-    // lengths within 10 % of each other behave like equal ones (200 tiles per SM 1.00, 600 0.97-0.98). Units
-    // of more than 32768 keys again want the long ones (49152 0.92-0.97 from 150 on). So batches count as
-    // uneven that hold less than 7/8 of their allocated tiles, up to 256 tiles per unit.
-    int64_t tiles = d.U * (int64_t)n_tiles;
-    bool uneven = false;
+    // In batches of different lengths units end in odd pieces, which costs long tasks more. Where many prompts
+    // are much shorter than the longest (together less than 3/4 of it), 8 wins at any amount of work (4 prompts
+    // drawn between 700 and L keys: L 6000 1.02-1.25 / 0.98-1.13, 12001 1.04-1.19 / 1.03-1.19, 30000 1.01-1.13 /
+    // 0.94-1.11 from 40 to 700 tiles per SM); else the line lies higher (lengths within 10 to 25 %: 200 tiles
+    // per SM 1.00-1.14, 290 0.98-1.09, 500 0.96, 600 0.97-0.98: 270). Not so for units of more than 32768 keys,
+    // where the merges weigh more (49152 0.92-0.97 from 150 on).
+    int64_t tiles = d.U * (int64_t)n_tiles, much = kMuchWork;
     if (d.sl.n > 0) {
-      int64_t per_layer = 0;
-      for (int b = 0; b < d.Bt; ++b) per_layer += (d.sl.len[b] + TILE_KEYS - 1) / TILE_KEYS;
+      int64_t per_layer = 0, longest = 0;
+      for (int b = 0; b < d.Bt; ++b) {
+        const int64_t n = (d.sl.len[b] + TILE_KEYS - 1) / TILE_KEYS;
+        per_layer += n;
+        if (n > longest) longest = n;
+      }
       tiles = per_layer * d.Hkv * d.NL;
-      uneven = n_tiles <= 256 && 8 * per_layer < 7 * (int64_t)d.Bt * n_tiles;
+      if (n_tiles <= 256 && 4 * per_layer < 3 * d.Bt * longest) much = INT64_MAX;
+      else if (n_tiles <= 256 && per_layer < d.Bt * longest) much = 40000;
     }
-    t = n_tiles >= kLongUnit || (n_tiles >= 64 && !uneven && tiles >= kMuchWork) ? 16 : 8;
+    t = n_tiles >= kLongUnit || (n_tiles >= 64 && tiles >= much) ? 16 : 8;
   }
   if (t > n_tiles) t = n_tiles;
   return t;
