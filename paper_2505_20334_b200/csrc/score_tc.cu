@@ -16,7 +16,7 @@
 // for any grid size. Every wait is bounded.
 // For M <= 64 sweep 1 holds the query rows twice (TMEM lanes r and 64 + r) and the warps on the
 // two copies split the key columns; for 128 < M <= 256 a tile has two row blocks and takes a
-// 256-column accumulator buffer (two K stages / buffers instead of four).
+// 256-column accumulator buffer (two buffers instead of four, a row block handed over at a time).
 //
 // Warp roles (768 threads):
 //   warp 0       ticket fetch + TMA producer (one lane)
@@ -58,7 +58,8 @@ constexpr int kThreads = 32 * (kMmaWarpB + kStatInWarps);
 // ring depths of the task hand-off and of the two statistics hand-offs (measured: 6 and 3 are
 // 0.5-1 % faster than 4 and 2; deeper rings do not fit the shared memory next to the K stages)
 constexpr int kTaskSlots = 6;
-constexpr int kMaxSlots = 4;  // K stages in shared memory = TMEM accumulator buffers
+constexpr int kMaxSlots = 4;  // TMEM accumulators of 128 columns
+constexpr int kKStages = 4;   // K stages in shared memory
 constexpr int kStatSlots = 3;
 constexpr uint32_t kKStageBytes = TILE_KEYS * 128 * 2;  // 128 keys x 128 dims x bf16
 constexpr uint32_t kCtlBytes = 34816;
@@ -112,15 +113,18 @@ struct Task {
 // Control block at the start of dynamic shared memory.
 struct Ctl {
   uint64_t q_full[2], q_empty[2];
-  uint64_t k_full[kMaxSlots];
-  // Tile t uses K stage t mod n_slots and accumulator buffer t mod n_slots, so one barrier per
-  // slot tells the producer that the stage is free and the softmax warps that the logits are ready.
+  uint64_t k_full[kKStages];
+  // Tile t uses K stage t mod 4 and accumulator buffer t mod n_slots. Up to 128 rows n_slots is 4 too, and
+  // one barrier per slot tells the producer that the stage is free and the softmax warps that the logits
+  // are ready. With more, n_slots is 2, a buffer consists of two row blocks with barriers of their own, and
+  // the stages have theirs.
   // n_slots is even: tiles t and t - n_slots then belong to the same MMA issuer and the same
   // softmax pair, which is what makes the parity waits sound (a waiter is never two phases ahead).
   // With five slots the second issuer can complete tile t - 2 before the first has issued tile
   // t - 5, and the pair waiting for tile t then sees a stale phase (seen as a wait that ran out).
   uint64_t mma_done[kMaxSlots];
   uint64_t tmem_empty[kMaxSlots];
+  uint64_t k_empty[kKStages];
   uint64_t drain[2];  // one per MMA issuer: completion of everything it has issued (abort path)
   uint64_t task_full[kTaskSlots], task_empty[kTaskSlots];
   uint64_t stat_full[kStatSlots], stat_empty[kStatSlots];
@@ -294,27 +298,35 @@ __device__ __noinline__ float2 stats_cols_ragged(uint32_t taddr, int valid_max, 
 
 // Sweep 1, this warpgroup's 64 key columns of one row block of a full tile. If `release`, the
 // accumulator buffer is handed back to the MMA warp as soon as the last chunk is in registers.
-template <int kPoly>
+template <int kPoly, bool kPrecise>
 __device__ __forceinline__ void stats_cols64(uint32_t taddr, float c, float& m, float& l, float* v,
                                              bool release, uint32_t empty_bar, int lane) {
   tmem_ld32(taddr, v);
   tmem_ld_wait(v);
-  stats_chunk<kPoly>(v, c, m, l);
+  stats_chunk<kPoly, kPrecise>(v, c, m, l);
   tmem_ld32(taddr + 32u, v);
   tmem_ld_wait(v);
   if (release) release_buffer(empty_bar, lane);
-  stats_chunk<kPoly>(v, c, m, l);
+  stats_chunk<kPoly, kPrecise>(v, c, m, l);
 }
 
 // ------------------------------------------------------------------ the kernel
 // kDup: M <= 64, sweep 1 holds every query row twice (on TMEM lanes r and 64 + r).
 // kWide: 128 < M <= 256, two row blocks per tile, so an accumulator buffer takes 256 TMEM columns
-// and there are two K stages / buffers instead of four.
+// and there are two of them instead of four. A row block's 128 columns are handed over and given back on
+// their own, in both sweeps, so that the MMAs of a pair's next tile run while it is at the second block of
+// this one; and there is one Q stage and room for four K stages, since a stage is now wanted half a tile
+// earlier (the next task's Q arrives while two tiles of this one are still to be exponentiated). 256 rows, us
+// with buffers and stages handed over whole, two of each: 65536 keys, 640 units 7589 -> 7136 (other boards
+// 7431 -> 7122); 16384 keys, 160 units 479 -> 458; 5000 keys 166 -> 157; row blocks alone 7214, 467, 161.
 // kPerHead: sweep 2 keeps one column sum per query head (colsum is [U*G][L_pad]); the launcher
 // only picks it when a head's rows never straddle a group of four rows or a 32-row chunk unevenly
 // (W a multiple of 4 that divides 32, or 32 or 64).
-// kPolyS1: share of sweep 1's exponentials on the FMA pipe (of every 8 pairs), measured to pay only for
-// 64 < M <= 128. Its polynomial has a relative error of 7.5e-5, which leaves the scores within 1e-6 of the
+// kPolyS1: share of sweep 1's exponentials on the FMA pipe (of every 8 pairs). With more than 128 rows it is
+// 1, of the exponential that is as precise as the MUFU's (scores 1.2e-7 from fp64 in the 2-norm either way):
+// the MUFU alone would take 2048 of a tile's 2570 cycles a sweep (256 rows: 65536 keys, 640 units 7136 -> 6894
+// us; 5000 keys, 160 units 161 -> 156; 64 dims 419 -> 404; 2 of 8 7031, 153, 403; one column sum per head no
+// faster, so none there). With up to 64 rows none pays. For 64 < M <= 128 it is a cheaper one. Its polynomial has a relative error of 7.5e-5, which leaves the scores within 1e-6 of the
 // exact ones in the 2-norm; on the MUFU alone they are within 2e-7. Head dims other than 128 take none, so
 // that their scores are as precise as on CUDA cores, where they used to be formed (64 dims, 128 rows, 128
 // units of 32768 keys: 324 us, with the polynomial 310; 256 units of 4096: 95.4 and 93.9).
@@ -323,9 +335,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
                 const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ TcArgs a) {
   constexpr uint32_t kQRows = kWide ? 256u : 128u;   // rows per 64-dim half of a Q stage
-  constexpr uint32_t kSlotShift = kWide ? 1u : 2u;   // log2 of the K stages = accumulator buffers
+  constexpr uint32_t kSlotShift = kWide ? 1u : 2u;   // log2 of the accumulator buffers
+  constexpr uint32_t kQStages = kWide ? 1u : 2u;
   constexpr uint32_t kTbCols = kWide ? 256u : 128u;  // TMEM columns per accumulator buffer
-  constexpr int RB = kWide ? 2 : 1;                  // 128-row blocks per tile in sweep 1
+  constexpr int RB = kWide ? 2 : 1;                  // 128-row blocks per tile, each with barriers of its own
   long long clk0 = 0;
   unsigned long long ns0 = 0;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -338,7 +351,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
   const uint32_t smem_base = smem_u32(smem_raw);
   const uint32_t q_stage_bytes = kQRows * 256u;
   const uint32_t q_base = smem_base + kCtlBytes;
-  const uint32_t k_base = q_base + 2u * q_stage_bytes;
+  const uint32_t k_base = q_base + kQStages * q_stage_bytes;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr uint32_t slot_mask = (1u << kSlotShift) - 1u;
 
@@ -354,8 +367,11 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
       mbar_init(smem_u32(&ctl->q_full[i]), 1);
       mbar_init(smem_u32(&ctl->q_empty[i]), 2);  // both MMA issuers
     }
-    for (int i = 0; i < kMaxSlots; ++i) {
+    for (int i = 0; i < kKStages; ++i) {
       mbar_init(smem_u32(&ctl->k_full[i]), 1);
+      mbar_init(smem_u32(&ctl->k_empty[i]), 1);
+    }
+    for (int i = 0; i < kMaxSlots; ++i) {
       mbar_init(smem_u32(&ctl->mma_done[i]), 1);
       mbar_init(smem_u32(&ctl->tmem_empty[i]), 8);  // the 8 warps of one warpgroup pair
     }
@@ -376,7 +392,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
   }
   {
     uint4* qz = reinterpret_cast<uint4*>(smem_raw + kCtlBytes);
-    const int n16 = (int)(2u * q_stage_bytes / 16u);
+    const int n16 = (int)(kQStages * q_stage_bytes / 16u);
     for (int i = threadIdx.x; i < n16; i += kThreads) qz[i] = make_uint4(0, 0, 0, 0);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -427,8 +443,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
         if (task.sweep < 0) break;
         // Q of the unit: box (64 dims, W queries, G heads) per half
         {
-          const uint32_t qs = qcount & 1u;
-          if (!mbar_wait(a, ctl, smem_u32(&ctl->q_empty[qs]), ((qcount >> 1) & 1u) ^ 1u, 3)) break;
+          const uint32_t qs = qcount % kQStages;
+          if (!mbar_wait(a, ctl, smem_u32(&ctl->q_empty[qs]), ((qcount / kQStages) & 1u) ^ 1u, 3)) break;
           const uint32_t bar = smem_u32(&ctl->q_full[qs]);
           mbar_expect_tx(bar, (uint32_t)(a.M * a.boxes) * 128u * (kDup ? 2u : 1u));
           for (int j = 0; j < a.boxes; ++j) {
@@ -444,9 +460,10 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
         const uint64_t pol = task.sweep == 0 ? pol_keep : pol_drop;
         Task next = stop;
         for (int i = 0; i < task.n_tiles; ++i) {
-          const uint32_t s = kcount & slot_mask;
+          const uint32_t s = kcount % kKStages;
           // the stage is free once the MMAs of the tile that used it last have completed
-          if (!mbar_wait(a, ctl, smem_u32(&ctl->mma_done[s]), ((kcount >> kSlotShift) & 1u) ^ 1u, 4)) {
+          if (!mbar_wait(a, ctl, smem_u32(kWide ? &ctl->k_empty[s] : &ctl->mma_done[s]),
+                         ((kcount / kKStages) & 1u) ^ 1u, 4)) {
             ok = false;
             break;
           }
@@ -467,11 +484,10 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
         // A wait ran out somewhere in this CTA. Loads that this lane has requested may still be
         // on their way into shared memory: wait (bounded) for the full-barrier of every K stage
         // and Q stage armed last, so that nothing is written into the CTA's memory after it exits.
-        const uint32_t n_slots = slot_mask + 1u;
-        for (uint32_t t = kcount > n_slots ? kcount - n_slots : 0u; t < kcount; ++t)
-          mbar_drain(smem_u32(&ctl->k_full[t & slot_mask]), (t >> kSlotShift) & 1u);
-        for (uint32_t t = qcount > 2u ? qcount - 2u : 0u; t < qcount; ++t)
-          mbar_drain(smem_u32(&ctl->q_full[t & 1u]), (t >> 1) & 1u);
+        for (uint32_t t = kcount > kKStages ? kcount - kKStages : 0u; t < kcount; ++t)
+          mbar_drain(smem_u32(&ctl->k_full[t % kKStages]), (t / kKStages) & 1u);
+        for (uint32_t t = qcount > kQStages ? qcount - kQStages : 0u; t < qcount; ++t)
+          mbar_drain(smem_u32(&ctl->q_full[t % kQStages]), (t / kQStages) & 1u);
       }
     }
   } else if (warp == 1 || warp == kMmaWarpB) {
@@ -485,7 +501,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
       const uint32_t issuer = warp == 1 ? 0u : 1u;
       uint32_t tc_base = 0, my_next = issuer, qc = 0, tk = 0;
       const uint32_t idesc_s1 = instr_desc(128, TILE_KEYS);
-      const uint32_t idesc_s2 = instr_desc(128, a.M_pad);
+      const uint32_t idesc_s2 = instr_desc(128, kWide ? 128 : a.M_pad);
+      const uint32_t idesc_s2b = instr_desc(128, kWide ? a.M_pad - 128 : 128);  // the second row block
       const uint32_t q_half16 = kQRows * 8u;  // (q_rows * 128 bytes) >> 4
       const uint32_t k_lo0 = smem_desc_lo(k_base), q_lo0 = smem_desc_lo(q_base);
       bool ok = true;
@@ -493,39 +510,46 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
         Task task;
         if (!next_task(a, ctl, tk, 0, true, 10, task)) break;
         if (task.sweep < 0) break;
-        const uint32_t qs = qc & 1u;
-        if (!mbar_wait(a, ctl, smem_u32(&ctl->q_full[qs]), (qc >> 1) & 1u, 11)) break;
+        const uint32_t qs = qc % kQStages;
+        if (!mbar_wait(a, ctl, smem_u32(&ctl->q_full[qs]), (qc / kQStages) & 1u, 11)) break;
         const uint32_t q_lo = q_lo0 + qs * (q_stage_bytes >> 4);
         int i = (int)(my_next - tc_base);
         for (; i < task.n_tiles; i += 2) {
           const uint32_t tc = tc_base + (uint32_t)i;
           const uint32_t s = tc & slot_mask;
           const uint32_t ph = (tc >> kSlotShift) & 1u;
-          if (!mbar_wait(a, ctl, smem_u32(&ctl->k_full[s]), ph, 12) ||
-              !mbar_wait(a, ctl, smem_u32(&ctl->tmem_empty[s]), ph ^ 1u, 13)) {
+          const uint32_t ks = tc % kKStages;
+          if (!mbar_wait(a, ctl, smem_u32(&ctl->k_full[ks]), (tc / kKStages) & 1u, 12)) {
             ok = false;
             break;
           }
-          tc_fence_after();
-          const uint32_t k_lo = k_lo0 + s * (kKStageBytes >> 4);
-          const uint32_t d_tmem = tmem_base + s * kTbCols;
-          // k-step kk covers dims [16 kk, 16 kk + 16): 32 bytes inside the 64-dim half (kk >> 2)
-          if (task.sweep == 0) {
-            for (int rb = 0; rb < RB; ++rb) {
+          const uint32_t k_lo = k_lo0 + ks * (kKStageBytes >> 4);
+#pragma unroll
+          for (int rb = 0; rb < RB; ++rb) {
+            if (!mbar_wait(a, ctl, smem_u32(&ctl->tmem_empty[s * RB + rb]), ph ^ 1u, 13)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint32_t d_tmem = tmem_base + s * kTbCols + (uint32_t)rb * 128u;
+            const uint32_t q_rb = q_lo + (uint32_t)rb * 1024u;
+            // k-step kk covers dims [16 kk, 16 kk + 16): 32 bytes inside the 64-dim half (kk >> 2)
+            if (task.sweep == 0) {
 #pragma unroll
               for (int kk = 0; kk < 8; ++kk)
-                if (kk < a.ksteps) umma_bf16(d_tmem + (uint32_t)rb * 128u,
-                          q_lo + (kk >> 2) * q_half16 + (uint32_t)rb * 1024u + (kk & 3) * 2u,
-                          k_lo + (kk >> 2) * (kKStageBytes >> 5) + (kk & 3) * 2u, kSmemDescHi,
-                          idesc_s1, kk > 0);
-            }
-          } else {
+                if (kk < a.ksteps) umma_bf16(d_tmem, q_rb + (kk >> 2) * q_half16 + (kk & 3) * 2u,
+                          k_lo + (kk >> 2) * (kKStageBytes >> 5) + (kk & 3) * 2u, kSmemDescHi, idesc_s1, kk > 0);
+            } else {
+              const uint32_t idesc = rb == 0 ? idesc_s2 : idesc_s2b;
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk)
-              if (kk < a.ksteps) umma_bf16(d_tmem, k_lo + (kk >> 2) * (kKStageBytes >> 5) + (kk & 3) * 2u,
-                        q_lo + (kk >> 2) * q_half16 + (kk & 3) * 2u, kSmemDescHi, idesc_s2, kk > 0);
+              for (int kk = 0; kk < 8; ++kk)
+                if (kk < a.ksteps) umma_bf16(d_tmem, k_lo + (kk >> 2) * (kKStageBytes >> 5) + (kk & 3) * 2u,
+                          q_rb + (kk >> 2) * q_half16 + (kk & 3) * 2u, kSmemDescHi, idesc, kk > 0);
+            }
+            umma_commit(smem_u32(&ctl->mma_done[s * RB + rb]));
           }
-          umma_commit(smem_u32(&ctl->mma_done[s]));
+          if (!ok) break;
+          if (kWide) umma_commit(smem_u32(&ctl->k_empty[ks]));
         }
         if (!ok) break;
         my_next = tc_base + (uint32_t)i;
@@ -656,10 +680,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
     const int row_in_wg = quad * 32 + lane;  // TMEM lane this thread reads
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
     const float c = a.scale_log2;
-    // sweep 2: this warpgroup's share of the M_pad / 32 row chunks
-    const int n_chunks2 = a.M_pad / 32;
-    const int ch_lo = half == 0 ? 0 : (n_chunks2 + 1) / 2;
-    const int ch_hi = half == 0 ? (n_chunks2 + 1) / 2 : n_chunks2;
+    const int n_chunks2 = a.M_pad / 32;  // sweep 2: row chunks of 32
     const uint32_t col0 = 64u * (uint32_t)half;  // sweep 1: this warpgroup's 64 key columns
     // Sweep 1 with M <= 64: lanes 64.. hold a second copy of the rows, so the warps on lanes r and
     // 64 + r share row r's 64 key columns of this warpgroup (32 each) and all four quadrants of
@@ -696,7 +717,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
       for (; i < task.n_tiles; i += 2) {
         const uint32_t tc = tc_base + (uint32_t)i;
         const uint32_t s = tc & slot_mask;
-        if (!mbar_wait(a, ctl, smem_u32(&ctl->mma_done[s]), (tc >> kSlotShift) & 1u, 21)) {
+        const uint32_t ph = (tc >> kSlotShift) & 1u;
+        if (!mbar_wait(a, ctl, smem_u32(&ctl->mma_done[s * RB]), ph, 21)) {
           ok = false;
           break;
         }
@@ -704,7 +726,14 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
         tc_fence_after();
         const int key0 = (task.tile0 + i) * TILE_KEYS;
         const uint32_t taddr = lane_addr + s * kTbCols;
-        const uint32_t empty_bar = smem_u32(&ctl->tmem_empty[s]);
+        const uint32_t empty_bar = smem_u32(&ctl->tmem_empty[s * RB]), empty_bar1 = empty_bar + 8u;
+        // the second row block's logits
+        auto second_block = [&]() -> bool {
+          if (!mbar_wait(a, ctl, smem_u32(&ctl->mma_done[s * RB + 1]), ph, 24)) return false;
+          __syncwarp();
+          tc_fence_after();
+          return true;
+        };
         float v[32];
         if (task.sweep == 0) {
           const int valid = min(TILE_KEYS, Lu - key0);
@@ -718,7 +747,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
               tmem_ld32(taddr + col_d, v);
               tmem_ld_wait(v);
               release_buffer(empty_bar, lane);
-              stats_chunk<kPolyS1>(v, c, m0, l0);
+              stats_chunk<kPolyS1, kWide>(v, c, m0, l0);
             } else {
               const int vq = min(32, valid - (int)col_d);
               const float2 r =
@@ -727,25 +756,38 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
               l0 = r.y;
               release_buffer(empty_bar, lane);
             }
-          } else if (valid == TILE_KEYS && key0 + TILE_KEYS <= Lu - a.W_local) {
-            // every column is a real key that every row sees
-            if (rows0) stats_cols64<kPolyS1>(taddr + col0, c, m0, l0, v, !rows1, empty_bar, lane);
-            if (rows1) stats_cols64<kPolyS1>(taddr + 128u + col0, c, m1, l1, v, true, empty_bar, lane);
-            if (!rows0) release_buffer(empty_bar, lane);
           } else {
+            // (every column is a real key that every row sees, but for the last tiles of a unit)
+            const bool whole = valid == TILE_KEYS && key0 + TILE_KEYS <= Lu - a.W_local;
             const int vh = min(64, valid - (int)col0);
             if (rows0) {
-              const float2 r = stats_cols_ragged(taddr + col0, vh, min(vh, vis0 - key0 - (int)col0), c, m0, l0);
-              m0 = r.x;
-              l0 = r.y;
+              if (whole) {
+                stats_cols64<kPolyS1, kWide>(taddr + col0, c, m0, l0, v, true, empty_bar, lane);
+              } else {
+                const float2 r =
+                    stats_cols_ragged(taddr + col0, vh, min(vh, vis0 - key0 - (int)col0), c, m0, l0);
+                m0 = r.x;
+                l0 = r.y;
+              }
             }
-            if (rows1) {
-              const float2 r =
-                  stats_cols_ragged(taddr + 128u + col0, vh, min(vh, vis1 - key0 - (int)col0), c, m1, l1);
-              m1 = r.x;
-              l1 = r.y;
+            if (!rows0 || !whole) release_buffer(empty_bar, lane);
+            if (kWide) {
+              if (!second_block()) {
+                ok = false;
+                break;
+              }
+              if (rows1) {
+                if (whole) {
+                  stats_cols64<kPolyS1, kWide>(taddr + 128u + col0, c, m1, l1, v, true, empty_bar1, lane);
+                } else {
+                  const float2 r =
+                      stats_cols_ragged(taddr + 128u + col0, vh, min(vh, vis1 - key0 - (int)col0), c, m1, l1);
+                  m1 = r.x;
+                  l1 = r.y;
+                }
+              }
+              if (!rows1 || !whole) release_buffer(empty_bar1, lane);
             }
-            release_buffer(empty_bar, lane);
           }
         } else if (kPerHead) {
           // one column sum per query head: the chunk's 32 rows come as eight groups of four, a
@@ -753,40 +795,64 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
           const int gph = (a.W < 32 ? a.W : 32) >> 2;
           const int key = key0 + row_in_wg;
 #pragma unroll 1
-          for (int ch = ch_lo; ch < ch_hi; ++ch) {
-            tmem_ld32(taddr + (uint32_t)ch * 32u, v);
-            tmem_ld_wait(v);
-            if (ch + 1 == ch_hi) release_buffer(empty_bar, lane);
-            float hs[8];
-            colsum_groups(v, c, nboff + ch * 32, hs);
-            float run = 0.f;
+          for (int rb = 0; rb < RB; ++rb) {
+            if (rb == 1 && !second_block()) {
+              ok = false;
+              break;
+            }
+            const uint32_t bar = rb == 0 ? empty_bar : empty_bar1;
+            const int n_ch = min(4, n_chunks2 - 4 * rb), mid = (n_ch + 1) / 2;
+            const int ch_lo = 4 * rb + (half == 0 ? 0 : mid), ch_hi = 4 * rb + (half == 0 ? mid : n_ch);
+#pragma unroll 1
+            for (int ch = ch_lo; ch < ch_hi; ++ch) {
+              tmem_ld32(taddr + (uint32_t)ch * 32u, v);
+              tmem_ld_wait(v);
+              if (ch + 1 == ch_hi) release_buffer(bar, lane);
+              float hs[8];
+              colsum_groups(v, c, nboff + ch * 32, hs);
+              float run = 0.f;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              run += hs[i];
-              if (((i + 1) & (gph - 1)) == 0) {
-                const int g = (ch * 32 + 4 * i) / a.W;
-                if (key < Lu && g < a.G) red_add(&a.colsum[(u * a.G + g) * a.L_pad + key], run);
-                run = 0.f;
+              for (int i = 0; i < 8; ++i) {
+                run += hs[i];
+                if (((i + 1) & (gph - 1)) == 0) {
+                  const int g = (ch * 32 + 4 * i) / a.W;
+                  if (key < Lu && g < a.G) red_add(&a.colsum[(u * a.G + g) * a.L_pad + key], run);
+                  run = 0.f;
+                }
               }
             }
+            if (ch_lo == ch_hi) release_buffer(bar, lane);
           }
-          if (ch_lo == ch_hi) release_buffer(empty_bar, lane);
+          if (!ok) break;
         } else {
           float2 acc[4];
 #pragma unroll
           for (int k = 0; k < 4; ++k) acc[k] = make_float2(0.f, 0.f);
+          bool any = false;
 #pragma unroll 1
-          for (int ch = ch_lo; ch < ch_hi; ++ch) {
-            tmem_ld32(taddr + (uint32_t)ch * 32u, v);
-            tmem_ld_wait(v);
-            if (ch + 1 == ch_hi) release_buffer(empty_bar, lane);
-            colsum_chunk<LAQ_POLY_PAIRS_S2>(v, c, nboff + ch * 32, nbsat + ch * 32, acc);
+          for (int rb = 0; rb < RB; ++rb) {
+            if (rb == 1 && !second_block()) {
+              ok = false;
+              break;
+            }
+            const uint32_t bar = rb == 0 ? empty_bar : empty_bar1;
+            // the row block's chunks that this warpgroup takes
+            const int n_ch = min(4, n_chunks2 - 4 * rb), mid = (n_ch + 1) / 2;
+            const int ch_lo = 4 * rb + (half == 0 ? 0 : mid), ch_hi = 4 * rb + (half == 0 ? mid : n_ch);
+#pragma unroll 1
+            for (int ch = ch_lo; ch < ch_hi; ++ch) {
+              tmem_ld32(taddr + (uint32_t)ch * 32u, v);
+              tmem_ld_wait(v);
+              if (ch + 1 == ch_hi) release_buffer(bar, lane);
+              colsum_chunk<LAQ_POLY_PAIRS_S2>(v, c, nboff + ch * 32, nbsat + ch * 32, acc);
+            }
+            if (ch_lo == ch_hi) release_buffer(bar, lane);
+            any = any || ch_lo < ch_hi;
           }
-          if (ch_lo == ch_hi) {
-            release_buffer(empty_bar, lane);
-          } else {
-            // The two warpgroups of the pair each add their rows' share into the zeroed column
-            // sum; with at most two addends the result does not depend on the order.
+          if (!ok) break;
+          // The two warpgroups of the pair each add their rows' share into the zeroed column
+          // sum; with at most two addends the result does not depend on the order.
+          if (any) {
             const float2 s2 = __fadd2_rn(__fadd2_rn(acc[0], acc[1]), __fadd2_rn(acc[2], acc[3]));
             const int key = key0 + row_in_wg;
             if (key < Lu) red_add(&a.colsum[u * a.L_pad + key], s2.x + s2.y);
@@ -964,7 +1030,6 @@ laq_status score_tc_launch(const laq_params& p, const Dims& d, const Workspace& 
   a.sl = d.sl;
   a.withhold_unit = test_withhold_unit();
   const bool wide = d.M > 128;
-  const int q_rows = wide ? 256 : 128, n_slots = wide ? 2 : 4;
   const bool dup = w.M_pad <= 64;  // sweep 1 holds every query row twice, on lanes r and 64 + r
 
   CUtensorMap tmap_q, tmap_k;
@@ -977,12 +1042,12 @@ laq_status score_tc_launch(const laq_params& p, const Dims& d, const Workspace& 
   if (!make_tensor_map(&tmap_q, q, qdims, qstr, qbox) || !make_tensor_map(&tmap_k, k, kdims, kstr, kbox))
     return score_simt_launch(p, d, w, q, k, ws, stream, launches);  // layout TMA cannot describe
 
-  const size_t smem = kCtlBytes + 2u * (size_t)q_rows * 256u + (size_t)n_slots * kKStageBytes;
+  const size_t smem = kCtlBytes + 65536u + (size_t)kKStages * kKStageBytes;  // one Q stage of 256 rows or two of 128
   const bool per_head = d.group_mode != LAQ_GROUP_SUM;
   typedef void (*Kernel)(const CUtensorMap, const CUtensorMap, const TcArgs);
   // [per head][dup, wide, neither, neither with other head dims]
   static const Kernel kernels[2][4] = {
-      {score_tc_kernel<true, false, false, 0>, score_tc_kernel<false, true, false, 0>,
+      {score_tc_kernel<true, false, false, 0>, score_tc_kernel<false, true, false, 1>,
        score_tc_kernel<false, false, false, LAQ_POLY_PAIRS_S1>, score_tc_kernel<false, false, false, 0>},
       {score_tc_kernel<true, false, true, 0>, score_tc_kernel<false, true, true, 0>,
        score_tc_kernel<false, false, true, LAQ_POLY_PAIRS_S1>, score_tc_kernel<false, false, true, 0>}};

@@ -11,8 +11,8 @@
 // Of every 8 element pairs, how many take the FMA-pipe exp2 instead of the MUFU. Alone, the
 // arithmetic is fastest at 2-3 of 8 (MUFU-bound below, FMA-bound above). Inside the kernel on a
 // B200 (measured in alternating builds, 20- and 150-step runs): in sweep 1, 2 of 8 is 1.3 % faster
-// than 0 of 8 for 64 < M <= 128 (3 of 8 is equal to 0, 4 of 8 is slower), equal for M = 256 and
-// 1 % slower for M = 64, so the kernel uses it for 64 < M <= 128 only; in sweep 2, where every
+// than 0 of 8 for 64 < M <= 128 (3 of 8 is equal to 0, 4 of 8 is slower) and 1 % slower for M = 64, so the
+// kernel uses it for 64 < M <= 128 only; in sweep 2, where every
 // chunk also loads its row offsets from shared memory, any share is slower.
 #define LAQ_POLY_PAIRS_S1 2
 #endif
@@ -88,8 +88,8 @@ __device__ __forceinline__ float2 exp2_mufu_pair(float2 x) { return make_float2(
 constexpr float kChunkSumLimit = 1.152921504606846976e18f;  // 2^60
 
 // One full 32-column chunk of this thread's row. Of every 8 element pairs, the first kPolyPairs
-// use the FMA-pipe exponential and the rest the MUFU.
-template <int kPolyPairs>
+// use the FMA-pipe exponential (kPrecise: the one as precise as the MUFU's) and the rest the MUFU.
+template <int kPolyPairs, bool kPrecise = false>
 __device__ __forceinline__ void stats_chunk(const float* v, float c, float& m, float& l) {
   const float2 c2 = make_float2(c, c), nm2 = make_float2(-m, -m);
   const float a_s = c * kSatInv, b_s = fmaf(-m, kSatInv, 0.5f);
@@ -98,10 +98,15 @@ __device__ __forceinline__ void stats_chunk(const float* v, float c, float& m, f
   for (int k = 0; k < 4; ++k) acc[k] = make_float2(0.f, 0.f);
 #pragma unroll
   for (int p = 0; p < 16; ++p) {
-    const float2 e =
-        ((p & 7) < kPolyPairs)
-            ? exp2_fma_pair_sat(v[2 * p], v[2 * p + 1], a_s, b_s, b_s)
-            : exp2_mufu_pair(__ffma2_rn(make_float2(v[2 * p], v[2 * p + 1]), c2, nm2));
+    float2 e;
+    if ((p & 7) >= kPolyPairs) {
+      e = exp2_mufu_pair(__ffma2_rn(make_float2(v[2 * p], v[2 * p + 1]), c2, nm2));
+    } else if (kPrecise) {
+      const float2 t = __ffma2_rn(make_float2(v[2 * p], v[2 * p + 1]), c2, nm2);
+      e = exp2_fma_pair(make_float2(fminf(t.x, 126.0f), fminf(t.y, 126.0f)));  // (2^126 is above the limit below)
+    } else {
+      e = exp2_fma_pair_sat(v[2 * p], v[2 * p + 1], a_s, b_s, b_s);
+    }
     acc[p & 3] = __fadd2_rn(acc[p & 3], e);
   }
   const float2 s2 = __fadd2_rn(__fadd2_rn(acc[0], acc[1]), __fadd2_rn(acc[2], acc[3]));

@@ -129,6 +129,33 @@ def test_two_sweeps_match_oracle(laq, case):  # noqa: F811
     compare_all_units(laq, q, k, v, W, kernel, B, out=out, local_window=Wl, seq_lens=lens, group_mode=group)
 
 
+# More than 128 rows: a tile's two row blocks change hands on their own, so the edges are the rows of the
+# second block (one group, one chunk, odd numbers of chunks), units of one to five tiles (fewer than the K
+# stages, odd numbers for a pair of warpgroups), tasks of one tile, and tiles that are masked in part.
+TWO_BLOCKS = [
+    # NL Bt G   L     W  W_local tiles lens          group
+    (1, 1, 3, 128, 43, 0, 0, None, 0),            # 129 rows, one tile
+    (2, 1, 5, 257, 32, 16, 0, None, 0),           # 160 rows, two tiles and a key
+    (1, 2, 7, 640, 32, 32, 1, (640, 130), 0),     # 224 rows, a task per tile, all queries local
+    (1, 1, 8, 1153, 32, 0, 3, None, 0),           # 256 rows, tasks of three tiles
+    (3, 2, 6, 4500, 32, 5, 0, (4500, 1000), 0),   # 192 rows, several tasks, CTAs with several units
+    (1, 1, 5, 900, 32, 0, 0, None, 2),            # one column sum per head, second block of one chunk
+    (1, 1, 4, 1300, 64, 8, 2, None, 1),           # heads of two chunks
+]
+
+
+@pytest.mark.parametrize("case", TWO_BLOCKS, ids=[f"M{c[2] * c[4]}-L{c[3]}-g{c[8]}" for c in TWO_BLOCKS])
+def test_two_row_blocks_match_oracle(laq, case):  # noqa: F811
+    NL, Bt, G, L, W, Wl, tiles, lens, group = case
+    q, k, v = rand_inputs(NL, Bt, 2 * G, 2, 128, L, W, seed=L + G, kscale=1.5)
+    if lens is not None:
+        for b, Lb in enumerate(lens):
+            k[:, b, :, Lb:] = float("nan")
+    B = W + 20
+    out = evict_with(laq, q, k, v, W, 7, B, tiles, Wl, lens, group, want="score_tc_kernel")
+    compare_all_units(laq, q, k, v, W, 7, B, out=out, local_window=Wl, seq_lens=lens, group_mode=group)
+
+
 CUDA_CORES = [
     (1, 1, 3, 1, 136, 500, 32, 0, 7, 60, None, 0),               # head dims above 128 with more than 64 rows
     (1, 2, 8, 2, 192, 900, 32, 16, 5, 90, (900, 333), 0),
