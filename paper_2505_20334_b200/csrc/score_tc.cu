@@ -680,7 +680,10 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
     const int row_in_wg = quad * 32 + lane;  // TMEM lane this thread reads
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
     const float c = a.scale_log2;
-    const int n_chunks2 = a.M_pad / 32;  // sweep 2: row chunks of 32
+    // sweep 2: this warpgroup's share of the row blocks' M_pad / 32 chunks of rows
+    const int n_chunks2 = a.M_pad / 32, n_first = min(4, n_chunks2), n_second = n_chunks2 - n_first;
+    const int ch_lo0 = half == 0 ? 0 : (n_first + 1) / 2, ch_hi0 = half == 0 ? (n_first + 1) / 2 : n_first;
+    const int ch_lo1 = 4 + (half == 0 ? 0 : (n_second + 1) / 2), ch_hi1 = 4 + (half == 0 ? (n_second + 1) / 2 : n_second);
     const uint32_t col0 = 64u * (uint32_t)half;  // sweep 1: this warpgroup's 64 key columns
     // Sweep 1 with M <= 64: lanes 64.. hold a second copy of the rows, so the warps on lanes r and
     // 64 + r share row r's 64 key columns of this warpgroup (32 each) and all four quadrants of
@@ -801,8 +804,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
               break;
             }
             const uint32_t bar = rb == 0 ? empty_bar : empty_bar1;
-            const int n_ch = min(4, n_chunks2 - 4 * rb), mid = (n_ch + 1) / 2;
-            const int ch_lo = 4 * rb + (half == 0 ? 0 : mid), ch_hi = 4 * rb + (half == 0 ? mid : n_ch);
+            const int ch_lo = rb == 0 ? ch_lo0 : ch_lo1, ch_hi = rb == 0 ? ch_hi0 : ch_hi1;
 #pragma unroll 1
             for (int ch = ch_lo; ch < ch_hi; ++ch) {
               tmem_ld32(taddr + (uint32_t)ch * 32u, v);
@@ -828,7 +830,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
           float2 acc[4];
 #pragma unroll
           for (int k = 0; k < 4; ++k) acc[k] = make_float2(0.f, 0.f);
-          bool any = false;
 #pragma unroll 1
           for (int rb = 0; rb < RB; ++rb) {
             if (rb == 1 && !second_block()) {
@@ -836,9 +837,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
               break;
             }
             const uint32_t bar = rb == 0 ? empty_bar : empty_bar1;
-            // the row block's chunks that this warpgroup takes
-            const int n_ch = min(4, n_chunks2 - 4 * rb), mid = (n_ch + 1) / 2;
-            const int ch_lo = 4 * rb + (half == 0 ? 0 : mid), ch_hi = 4 * rb + (half == 0 ? mid : n_ch);
+            const int ch_lo = rb == 0 ? ch_lo0 : ch_lo1, ch_hi = rb == 0 ? ch_hi0 : ch_hi1;
 #pragma unroll 1
             for (int ch = ch_lo; ch < ch_hi; ++ch) {
               tmem_ld32(taddr + (uint32_t)ch * 32u, v);
@@ -847,12 +846,11 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
               colsum_chunk<LAQ_POLY_PAIRS_S2>(v, c, nboff + ch * 32, nbsat + ch * 32, acc);
             }
             if (ch_lo == ch_hi) release_buffer(bar, lane);
-            any = any || ch_lo < ch_hi;
           }
           if (!ok) break;
           // The two warpgroups of the pair each add their rows' share into the zeroed column
           // sum; with at most two addends the result does not depend on the order.
-          if (any) {
+          if (ch_lo0 < ch_hi0) {
             const float2 s2 = __fadd2_rn(__fadd2_rn(acc[0], acc[1]), __fadd2_rn(acc[2], acc[3]));
             const int key = key0 + row_in_wg;
             if (key < Lu) red_add(&a.colsum[u * a.L_pad + key], s2.x + s2.y);
