@@ -84,7 +84,8 @@ struct ClArgs {
   int n_stages;      // K stages
   int slots_log2;    // TMEM tiles
   int stride_log2;   // TMEM columns per tile
-  int c_log2;        // log2 of the cluster size
+  int C, c_log2;     // CTAs per cluster; log2 of it where that is a whole number
+  int full_tiles, more_tiles;  // prompts of L positions: tiles of every CTA; CTAs that have one more
   float scale_log2;
   int keep_status;    // the status words keep what an earlier piece of the call recorded
   int withhold_unit;  // test hook: this unit's statistics are never sent (-1: none)
@@ -115,6 +116,16 @@ constexpr uint32_t kCtlBytes = (sizeof(Ctl) + 127u) / 128u * 128u;
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_index() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_count() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%nclusterid.x;" : "=r"(r));
   return r;
 }
 __device__ __forceinline__ void cluster_sync() {
@@ -179,10 +190,22 @@ struct Unit {
   int Lu;     // length of the unit's prompt
   int tiles;  // tiles of the unit that this CTA holds
 };
+// kShift: the cluster size is a power of two, c_log2 its logarithm. (Kernels of their own: with a product in place of the shift and
+// a division of the tiles the others took up to 4 % longer, 256 units of 12000 keys and 64 rows 190 -> 197 us.)
+// Place in the unit of the i-th tile of the CTA of that rank.
+template <bool kShift>
+__device__ __forceinline__ int tile_at(const ClArgs& a, int rank, int i) {
+  return rank + (kShift ? i << a.c_log2 : i * a.C);
+}
+template <bool kShift>
 __device__ __forceinline__ Unit unit_at(const ClArgs& a, int u, int rank) {
   Unit x;
   x.u = u;
   x.Lu = a.L;
+  if (!kShift) {  // (all prompts have L positions)
+    x.tiles = a.full_tiles + (rank < a.more_tiles ? 1 : 0);
+    return x;
+  }
   if (a.sl.n > 0) x.Lu = a.sl.len[((uint32_t)u / (uint32_t)a.Hkv) % (uint32_t)a.Bt];
   const int n_tiles = (x.Lu + TILE_KEYS - 1) / TILE_KEYS;
   x.tiles = rank < n_tiles ? (int)((uint32_t)(n_tiles - rank - 1) >> a.c_log2) + 1 : 0;
@@ -268,16 +291,17 @@ __device__ __forceinline__ Warp1 make_warp1(uint32_t tmem_base) {
 // Pass 1 again for a warp whose sums overflowed: the largest logit of every row becomes its
 // reference. Rare (a key more than 69 nats above the first one), so eight rows at a time; writes the
 // warp's pairs.
+template <bool kShift>
 __device__ __noinline__ void redo_sums(const ClArgs& a, Ctl* ctl, int u, int rank, uint32_t tile0, int buf) {
   const Warp1 w = make_warp1(ctl->tmem_base);
-  const Unit x = unit_at(a, u, rank);
+  const Unit x = unit_at<kShift>(a, u, rank);
   const float c = a.scale_log2;
   const uint32_t slot_mask = (1u << a.slots_log2) - 1u;
   for (int g = 0; g < a.groups; ++g) {
     float m[2] = {-3.0e38f, -3.0e38f}, s[2] = {0.f, 0.f};
     for (int sweep = 0; sweep < 2; ++sweep) {
       for (int i = w.index >> 2; i < x.tiles; i += 2) {
-        const int key0 = (rank + (i << a.c_log2)) * TILE_KEYS + w.quad * 32;
+        const int key0 = tile_at<kShift>(a, rank, i) * TILE_KEYS + w.quad * 32;
         if (key0 >= x.Lu) continue;
         const uint32_t slot = (tile0 + (uint32_t)i) & slot_mask;
         for (int half = 0; half < 2; ++half) {
@@ -310,7 +334,7 @@ __device__ __noinline__ void redo_sums(const ClArgs& a, Ctl* ctl, int u, int ran
 
 // Pass 1 over this warp's tiles of a unit; tile0 is the CTA's running number of the unit's first
 // tile, n the running number of the unit.
-template <int kGroups>
+template <int kGroups, bool kShift>
 __device__ __forceinline__ bool pass1(const ClArgs& a, Ctl* ctl, const Warp1& w, const Unit& x, int rank,
                                       uint32_t tile0, int n) {
   const float c = a.scale_log2;
@@ -326,7 +350,7 @@ __device__ __forceinline__ bool pass1(const ClArgs& a, Ctl* ctl, const Warp1& w,
     if (!bounded_wait(a, ctl, &ctl->slot_full[slot], (t >> a.slots_log2) & 1u, 21)) return false;
     __syncwarp();
     tc_fence_after();
-    const int key0 = (rank + (i << a.c_log2)) * TILE_KEYS + w.quad * 32;
+    const int key0 = tile_at<kShift>(a, rank, i) * TILE_KEYS + w.quad * 32;
     if (key0 >= x.Lu) continue;  // warp-uniform: the prompt ends before this warp's keys
     const uint32_t taddr = w.lane_addr + (slot << a.stride_log2);
     const bool masked = key0 + 32 > x.Lu - a.W_local;
@@ -364,7 +388,7 @@ __device__ __forceinline__ bool pass1(const ClArgs& a, Ctl* ctl, const Warp1& w,
     *reinterpret_cast<float4*>(&ctl->part[buf][w.index][row]) =
         make_float4(-nref[0].x, acc[0].x, -nref[0].y, acc[0].y);
   __syncwarp();
-  if (__any_sync(0xffffffffu, high)) redo_sums(a, ctl, x.u, rank, tile0, buf);
+  if (__any_sync(0xffffffffu, high)) redo_sums<kShift>(a, ctl, x.u, rank, tile0, buf);
   tc_fence_before();
   __syncwarp();
   if (w.lane == 0) mbar_arrive(smem_u32(&ctl->stat_full[buf]));
@@ -446,7 +470,7 @@ __device__ __forceinline__ void release_slot(Ctl* ctl, uint32_t slot, int lane) 
   if (lane == 0) mbar_arrive(smem_u32(&ctl->slot_empty[slot]));
 }
 
-template <int kGroups, bool kPerHead>
+template <int kGroups, bool kPerHead, bool kShift>
 __device__ __forceinline__ bool pass2(const ClArgs& a, Ctl* ctl, uint32_t tmem_base, const Unit& x, int rank,
                                       uint32_t tile0, int n) {
   constexpr int kFirst = kGroups < 4 ? kGroups : 4, kRest = kGroups - kFirst;  // one or two loads
@@ -463,7 +487,7 @@ __device__ __forceinline__ bool pass2(const ClArgs& a, Ctl* ctl, uint32_t tmem_b
   // the unit's tiles are all complete: pass 1 has been through them
   for (int i = wg; i < x.tiles; i += 2) {
     const uint32_t slot = (tile0 + (uint32_t)i) & slot_mask;
-    const int key = (rank + (i << a.c_log2)) * TILE_KEYS + quad * 32 + lane;
+    const int key = tile_at<kShift>(a, rank, i) * TILE_KEYS + quad * 32 + lane;
     const bool any = key - lane < x.Lu;  // warp-uniform: the prompt reaches this warp's keys
     float2 acc[4];
     HeadSums hs;
@@ -510,7 +534,7 @@ __device__ __forceinline__ bool pass2(const ClArgs& a, Ctl* ctl, uint32_t tmem_b
 }
 
 // ------------------------------------------------------------------ the kernel
-template <int kGroups, bool kPerHead>
+template <int kGroups, bool kPerHead, bool kShift>
 __global__ void __launch_bounds__(kThreads, 1)
 score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                      const __grid_constant__ ClArgs a) {
@@ -532,7 +556,9 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
   float2* lse_in = reinterpret_cast<float2*>(smem_raw + ctl_off + kCtlBytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = (int)cluster_rank();
-  const int C = 1 << a.c_log2, n_clusters = (int)(gridDim.x >> a.c_log2), u_first = (int)(blockIdx.x >> a.c_log2);
+  const int C = kShift ? 1 << a.c_log2 : a.C;
+  const int n_clusters = (int)(kShift ? gridDim.x >> a.c_log2 : cluster_count());
+  const int u_first = (int)(kShift ? blockIdx.x >> a.c_log2 : cluster_index());
   const int rows8 = a.groups * 8;
 
   if ((smem_base & 1023u) != 0) {  // the same in every CTA
@@ -601,7 +627,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
       const uint64_t pol = l2_policy_evict_first();
       bool ok = true;
       for (int u = u_first; ok && u < a.U; u += n_clusters) {
-        const Unit x = unit_at(a, u, rank);
+        const Unit x = unit_at<kShift>(a, u, rank);
         const int h = u % a.Hkv, b = (u / a.Hkv) % a.Bt, layer = u / (a.Hkv * a.Bt);
         {
           const uint32_t qs = qc & 1u;
@@ -621,7 +647,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
           const uint32_t bar = smem_u32(&ctl->k_full[stage]);
           mbar_expect_tx(bar, k_stage_bytes);
           const uint32_t dst = smem_base + stage * k_stage_bytes;
-          const int key0 = (rank + (i << a.c_log2)) * TILE_KEYS;
+          const int key0 = tile_at<kShift>(a, rank, i) * TILE_KEYS;
           for (int j = 0; j < a.boxes; ++j)
             tma_load_5d_hint(dst + (uint32_t)j * kBoxBytes, &tmap_k, bar, 64 * j, key0, h, b, layer, pol);
           ++kc;
@@ -646,7 +672,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
     uint32_t qc = 0, stage = 0, phase = 0, t = 0;
     bool ok = true;
     for (int u = u_first; ok && u < a.U; u += n_clusters) {
-      const Unit x = unit_at(a, u, rank);
+      const Unit x = unit_at<kShift>(a, u, rank);
       const uint32_t qs = qc & 1u;
       if (!bounded_wait(a, ctl, &ctl->q_full[qs], (qc >> 1) & 1u, 11)) break;
       const uint32_t q_lo = q_lo0 + qs * (q_stage_bytes >> 4);
@@ -748,8 +774,8 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
     uint32_t tile0 = 0;
     int n = 0;
     for (int u = u_first; u < a.U; u += n_clusters, ++n) {
-      const Unit x = unit_at(a, u, rank);
-      if (!pass1<kGroups>(a, ctl, w, x, rank, tile0, n)) break;
+      const Unit x = unit_at<kShift>(a, u, rank);
+      if (!pass1<kGroups, kShift>(a, ctl, w, x, rank, tile0, n)) break;
       tile0 += (uint32_t)x.tiles;
     }
   } else {
@@ -757,8 +783,8 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
     uint32_t tile0 = 0;
     int n = 0;
     for (int u = u_first; u < a.U; u += n_clusters, ++n) {
-      const Unit x = unit_at(a, u, rank);
-      if (!pass2<kGroups, kPerHead>(a, ctl, tmem_base, x, rank, tile0, n)) break;
+      const Unit x = unit_at<kShift>(a, u, rank);
+      if (!pass2<kGroups, kPerHead, kShift>(a, ctl, tmem_base, x, rank, tile0, n)) break;
       tile0 += (uint32_t)x.tiles;
     }
   }
@@ -783,19 +809,21 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
 }
 
 typedef void (*ClusterKernel)(const CUtensorMap, const CUtensorMap, const ClArgs);
-// [per head][groups of eight rows - 1] (seven groups run as eight)
+// [power of two][per head][groups of eight rows - 1] (seven groups run as eight)
 constexpr int kVariants = 8;
-#define LAQ_VARIANTS(H)                                                                           \
-  {score_cluster_kernel<1, H>, score_cluster_kernel<2, H>, score_cluster_kernel<3, H>,            \
-   score_cluster_kernel<4, H>, score_cluster_kernel<5, H>, score_cluster_kernel<6, H>,            \
-   score_cluster_kernel<8, H>, score_cluster_kernel<8, H>}
-const ClusterKernel kKernels[2][kVariants] = {LAQ_VARIANTS(false), LAQ_VARIANTS(true)};
+#define LAQ_VARIANTS(H, P)                                                                                \
+  {score_cluster_kernel<1, H, P>, score_cluster_kernel<2, H, P>, score_cluster_kernel<3, H, P>,           \
+   score_cluster_kernel<4, H, P>, score_cluster_kernel<5, H, P>, score_cluster_kernel<6, H, P>,           \
+   score_cluster_kernel<8, H, P>, score_cluster_kernel<8, H, P>}
+const ClusterKernel kKernels[2][2][kVariants] = {{LAQ_VARIANTS(false, false), LAQ_VARIANTS(true, false)},
+                                                 {LAQ_VARIANTS(false, true), LAQ_VARIANTS(true, true)}};
 #undef LAQ_VARIANTS
 
-// Clusters of each size (1, 2, 4, 8, 16) that the device keeps resident with this kernel's resources,
-// one CTA per SM; looked up once per device. 0: that cluster size cannot be launched.
+// Clusters of each size that the device keeps resident with this kernel's resources, one CTA per SM;
+// looked up once per device. 0: that cluster size cannot be launched.
+constexpr int kMaxCluster = 16;
 struct ClusterCounts {
-  int resident[5];
+  int resident[kMaxCluster + 1];
 };
 constexpr size_t kSmemBytes = 227 * 1024;
 
@@ -807,25 +835,25 @@ bool cluster_counts(int dev, ClusterCounts* out) {
   if (!known[dev].load(std::memory_order_acquire)) {
     std::lock_guard<std::mutex> lock(mutex);
     if (!known[dev].load(std::memory_order_relaxed)) {
-      for (int i = 0; i < 2 * kVariants; ++i)
-        if (!cuda_ok(cudaFuncSetAttribute(kKernels[i / kVariants][i % kVariants],
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes)) ||
-            !cuda_ok(cudaFuncSetAttribute(kKernels[i / kVariants][i % kVariants],
-                                          cudaFuncAttributeNonPortableClusterSizeAllowed, 1)))
+      for (int i = 0; i < 4 * kVariants; ++i) {
+        const ClusterKernel kernel = kKernels[i / (2 * kVariants)][i / kVariants % 2][i % kVariants];
+        if (!cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes)) ||
+            !cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)))
           return false;
-      for (int i = 0; i < 5; ++i) {
+      }
+      for (int i = 1; i <= kMaxCluster; ++i) {
         cudaLaunchAttribute attr;
         attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = 1u << i;
+        attr.val.clusterDim.x = (unsigned)i;
         attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(1u << i);
+        cfg.gridDim = dim3((unsigned)i);
         cfg.blockDim = dim3(kThreads);
         cfg.dynamicSmemBytes = kSmemBytes;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
         int n = 0;
-        if (!cuda_ok(cudaOccupancyMaxActiveClusters(&n, kKernels[0][kVariants - 1], &cfg))) n = 0;
+        if (!cuda_ok(cudaOccupancyMaxActiveClusters(&n, kKernels[(i & (i - 1)) == 0][0][kVariants - 1], &cfg))) n = 0;
         cached[dev].resident[i] = n;
       }
       known[dev].store(true, std::memory_order_release);
@@ -867,24 +895,53 @@ laq_status score_cluster_launch(const laq_params& p, const Dims& d, const Worksp
   // SMs idle (15 of 8 CTAs and 7 of 16 fit the 148), small ones fit fewer keys.
   // L 6007, 64 rows, 256 units: 102 us with 8 CTAs, 121 with 16; L 4096: 67 / 63 us with 4 / 8; 64-dim
   // heads, 32 rows, L 4096, 128 units: 26.1 / 24.6 / 27.0 us with 2 / 4 / 8.
-  int best = -1;
+  int best = 0;
   double best_cost = 0.0;
-  for (int i = 0; i < 5; ++i) {
-    const int C = 1 << i, n = counts.resident[i], T = (n_tiles + C - 1) / C;
+  for (int C = 1; C <= kMaxCluster; C *= 2) {
+    const int n = counts.resident[C], T = (n_tiles + C - 1) / C;
     if (n < 1 || T > slots || C > n_tiles) continue;
     const double rounds = (double)((d.U + n - 1) / n);
     const double tile = fmax(200.0 + 20.0 * d.M, (double)(a.boxes * kBoxBytes) * fmax(n * C, 120.0) / 3600.0);
     const double exchange = 2 * T <= slots ? 60.0 * C : (T < slots ? 1000.0 : 3000.0);
     const double cost = rounds * (T * tile + exchange);
-    if (best < 0 || cost < best_cost) {
-      best = i;
+    if (best == 0 || cost < best_cost) {
+      best = C;
       best_cost = cost;
     }
   }
-  if (best < 0) return LAQ_OK;
-  a.c_log2 = best;
-  const int C = 1 << best;
-  const int64_t clusters = d.U < counts.resident[best] ? d.U : counts.resident[best];
+  // Sizes between the powers of two, where 3 % or more are expected of them: the 148 SMs hold 45 clusters of
+  // 3 CTAs, 26 of 5, 22 of 6, 15 of 7 to 9, 11 of 10, 7 of 11 to 16, and the units fill the tensor memory and the
+  // last round better or worse. Fitted to sizes of all kinds (a round is the arithmetic and the exposed part
+  // of the exchange, or the CTA's share of the HBM stream and its exposed end). us on 256 units, 64 rows:
+  // L 9000 142 with 9, 180 with 16; L 6007 99 / 101 / 105 with 6 / 9 / 8; L 2500 45 / 49 with 5 / 4; 40 rows, L 2850
+  // 43 / 47 with 6 / 4; 32 rows, 96 dims, L 15018 159 / 169 / 177 with 9 / 10 / 16; 512 units of 16 rows, L 11612 153 / 155
+  // / 180 with 7 / 8 / 4. Not for prompts of different lengths, which leave CTAs of a cluster without tiles in
+  // ways that this does not foresee (3 prompts of 1319 to 6597 keys: 4 % slower).
+  const auto round_cycles = [&](int C) {
+    const int n = counts.resident[C], T = (n_tiles + C - 1) / C;
+    const double rounds = (double)((d.U + n - 1) / n), sms = (double)(d.U < n ? d.U : n) * C;
+    const double full = (double)T / slots;
+    const double math = T * (200.0 + 20.0 * d.M) + fmax(0.0, 2200.0 * (2.0 * full - 1.0));
+    const double stream = T * (double)(a.boxes * kBoxBytes) * fmax(sms, 116.0) / 3830.0 + fmax(0.0, 8000.0 * (full - 0.75));
+    return rounds * (fmax(math, stream) + 20.0 * C);
+  };
+  best_cost = best > 0 ? round_cycles(best) : 0.0;
+  for (int C = 3; C < kMaxCluster && d.sl.n == 0; ++C) {
+    if ((C & (C - 1)) == 0 || counts.resident[C] < 1 || (n_tiles + C - 1) / C > slots || C > n_tiles) continue;
+    const double cost = round_cycles(C);
+    if (best == 0 || cost < 0.97 * best_cost) {
+      best = C;
+      best_cost = cost;
+    }
+  }
+  if (best == 0) return LAQ_OK;
+  const int C = best;
+  const bool pow2 = (C & (C - 1)) == 0;
+  a.C = C;
+  a.c_log2 = log2_ceil(C);
+  a.full_tiles = n_tiles / C;
+  a.more_tiles = n_tiles % C;
+  const int64_t clusters = d.U < counts.resident[C] ? d.U : counts.resident[C];
   const int variant = a.groups - 1;
   a.n16 = ((a.groups == 7 ? 64 : 8 * a.groups) + 15) / 16 * 16;
   const size_t stage = (size_t)a.boxes * kBoxBytes, qs = 2 * (size_t)a.boxes * a.n16 * 128;
@@ -925,7 +982,7 @@ laq_status score_cluster_launch(const laq_params& p, const Dims& d, const Worksp
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  if (!cuda_ok(cudaLaunchKernelEx(&cfg, kKernels[per_head ? 1 : 0][variant], tmap_q, tmap_k, a)))
+  if (!cuda_ok(cudaLaunchKernelEx(&cfg, kKernels[pow2 ? 1 : 0][per_head ? 1 : 0][variant], tmap_q, tmap_k, a)))
     return LAQ_ERR_CUDA;
   *launches += 1;
   *done = true;

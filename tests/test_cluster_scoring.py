@@ -77,3 +77,32 @@ def test_cluster_scoring_many_short_units_of_few_rows(laq, W, L, lens):
         out = laq.evict(qc, kc, vc, B, pool_kernel=kernel, want_scores=True, seq_lens=lens, ws=first["ws"])
     assert laq.laq_last_device_status(out["params"], out["ws"]) == laq.LAQ_OK
     assert torch.equal(out["scores"], first["scores"]) and torch.equal(out["idx"], first["idx"])
+
+
+@pytest.mark.parametrize("units,G,W,D,L,lens", [
+    (256, 4, 16, 128, 2500, None),                 # clusters of 5, four tiles a CTA
+    (256, 4, 16, 128, 6007, None),                 # of 6, all slots of the tensor memory
+    (256, 4, 16, 128, 9000, None),                 # of 9
+    (256, 4, 16, 128, 9000, (9000, 5001, 1153, 129)),  # (prompts of different lengths: of 16)
+    (64, 4, 12, 128, 3000, None),                  # of 6
+    (16, 2, 4, 64, 6646, None),
+    (1184, 4, 16, 128, 384, None),                 # of 1 or 3: odd numbers of tiles a unit, many rounds
+])
+def test_clusters_of_any_size(laq, units, G, W, D, L, lens):
+    # against the other tensor-core kernel (which a task size set by the caller selects). Both sum the same
+    # exponentials, arguments rounded to fp32, in other orders: 2^-21 in the 2-norm apiece.
+    Bt, Hkv = (len(lens) if lens else 1), 8
+    NL = max(1, units // (Bt * Hkv))
+    g = torch.Generator(device="cuda").manual_seed(L)
+    q = torch.randn((NL, Bt, G * Hkv, W, D), generator=g, device="cuda", dtype=torch.bfloat16)
+    k = torch.randn((NL, Bt, Hkv, L, D), generator=g, device="cuda", dtype=torch.bfloat16)
+    p = laq.params_for(q, k, W, 1, W + 20)
+    p.set_seq_lens(lens)
+    got = torch.full((NL, Bt, Hkv, L - W), float("nan"), device="cuda")
+    ws = laq.alloc_workspace(p, "cuda")
+    laq.laq_score(p, q, k, got, ws)
+    assert laq.laq_last_device_status(p, ws) == laq.LAQ_OK
+    p.tiles_per_task = 8
+    want = torch.empty_like(got)
+    laq.laq_score(p, q, k, want, laq.alloc_workspace(p, "cuda"))
+    assert float((got - want).norm() / want.norm()) < 1e-6
