@@ -124,7 +124,6 @@ struct Ctl {
   // t - 5, and the pair waiting for tile t then sees a stale phase (seen as a wait that ran out).
   uint64_t mma_done[kMaxSlots];
   uint64_t tmem_empty[kMaxSlots];
-  uint64_t k_empty[kKStages];
   uint64_t drain[2];  // one per MMA issuer: completion of everything it has issued (abort path)
   uint64_t task_full[kTaskSlots], task_empty[kTaskSlots];
   uint64_t stat_full[kStatSlots], stat_empty[kStatSlots];
@@ -143,6 +142,7 @@ struct Ctl {
   // per-prompt lengths: task_prefix[b] = sweep-1 tasks of one layer that belong to prompts < b
   // (written and read by the producer lane only)
   int task_prefix[LAQ_MAX_RAGGED_BATCH + 1];
+  uint64_t k_empty[kKStages];  // (more than 128 rows)
 };
 static_assert(sizeof(Ctl) <= kCtlBytes, "control block too large");
 
@@ -518,38 +518,62 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
           const uint32_t tc = tc_base + (uint32_t)i;
           const uint32_t s = tc & slot_mask;
           const uint32_t ph = (tc >> kSlotShift) & 1u;
-          const uint32_t ks = tc % kKStages;
-          if (!mbar_wait(a, ctl, smem_u32(&ctl->k_full[ks]), (tc / kKStages) & 1u, 12)) {
-            ok = false;
-            break;
-          }
-          const uint32_t k_lo = k_lo0 + ks * (kKStageBytes >> 4);
-#pragma unroll
-          for (int rb = 0; rb < RB; ++rb) {
-            if (!mbar_wait(a, ctl, smem_u32(&ctl->tmem_empty[s * RB + rb]), ph ^ 1u, 13)) {
+          if constexpr (!kWide) {
+            if (!mbar_wait(a, ctl, smem_u32(&ctl->k_full[s]), ph, 12) ||
+                !mbar_wait(a, ctl, smem_u32(&ctl->tmem_empty[s]), ph ^ 1u, 13)) {
               ok = false;
               break;
             }
             tc_fence_after();
-            const uint32_t d_tmem = tmem_base + s * kTbCols + (uint32_t)rb * 128u;
-            const uint32_t q_rb = q_lo + (uint32_t)rb * 1024u;
+            const uint32_t k_lo = k_lo0 + s * (kKStageBytes >> 4);
+            const uint32_t d_tmem = tmem_base + s * kTbCols;
             // k-step kk covers dims [16 kk, 16 kk + 16): 32 bytes inside the 64-dim half (kk >> 2)
             if (task.sweep == 0) {
 #pragma unroll
               for (int kk = 0; kk < 8; ++kk)
-                if (kk < a.ksteps) umma_bf16(d_tmem, q_rb + (kk >> 2) * q_half16 + (kk & 3) * 2u,
+                if (kk < a.ksteps) umma_bf16(d_tmem, q_lo + (kk >> 2) * q_half16 + (kk & 3) * 2u,
                           k_lo + (kk >> 2) * (kKStageBytes >> 5) + (kk & 3) * 2u, kSmemDescHi, idesc_s1, kk > 0);
             } else {
-              const uint32_t idesc = rb == 0 ? idesc_s2 : idesc_s2b;
 #pragma unroll
               for (int kk = 0; kk < 8; ++kk)
                 if (kk < a.ksteps) umma_bf16(d_tmem, k_lo + (kk >> 2) * (kKStageBytes >> 5) + (kk & 3) * 2u,
-                          q_rb + (kk >> 2) * q_half16 + (kk & 3) * 2u, kSmemDescHi, idesc, kk > 0);
+                          q_lo + (kk >> 2) * q_half16 + (kk & 3) * 2u, kSmemDescHi, idesc_s2, kk > 0);
             }
-            umma_commit(smem_u32(&ctl->mma_done[s * RB + rb]));
+            umma_commit(smem_u32(&ctl->mma_done[s]));
+          } else {
+            const uint32_t ks = tc % kKStages;
+            if (!mbar_wait(a, ctl, smem_u32(&ctl->k_full[ks]), (tc / kKStages) & 1u, 12)) {
+              ok = false;
+              break;
+            }
+            const uint32_t k_lo = k_lo0 + ks * (kKStageBytes >> 4);
+#pragma unroll
+            for (int rb = 0; rb < RB; ++rb) {
+              if (!mbar_wait(a, ctl, smem_u32(&ctl->tmem_empty[s * RB + rb]), ph ^ 1u, 13)) {
+                ok = false;
+                break;
+              }
+              tc_fence_after();
+              const uint32_t d_tmem = tmem_base + s * kTbCols + (uint32_t)rb * 128u;
+              const uint32_t q_rb = q_lo + (uint32_t)rb * 1024u;
+              // k-step kk covers dims [16 kk, 16 kk + 16): 32 bytes inside the 64-dim half (kk >> 2)
+              if (task.sweep == 0) {
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk)
+                  if (kk < a.ksteps) umma_bf16(d_tmem, q_rb + (kk >> 2) * q_half16 + (kk & 3) * 2u,
+                            k_lo + (kk >> 2) * (kKStageBytes >> 5) + (kk & 3) * 2u, kSmemDescHi, idesc_s1, kk > 0);
+              } else {
+                const uint32_t idesc = rb == 0 ? idesc_s2 : idesc_s2b;
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk)
+                  if (kk < a.ksteps) umma_bf16(d_tmem, k_lo + (kk >> 2) * (kKStageBytes >> 5) + (kk & 3) * 2u,
+                            q_rb + (kk >> 2) * q_half16 + (kk & 3) * 2u, kSmemDescHi, idesc, kk > 0);
+              }
+              umma_commit(smem_u32(&ctl->mma_done[s * RB + rb]));
+            }
+            if (!ok) break;
+            umma_commit(smem_u32(&ctl->k_empty[ks]));
           }
-          if (!ok) break;
-          if (kWide) umma_commit(smem_u32(&ctl->k_empty[ks]));
         }
         if (!ok) break;
         my_next = tc_base + (uint32_t)i;
@@ -759,7 +783,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
               l0 = r.y;
               release_buffer(empty_bar, lane);
             }
-          } else {
+          } else if (kWide) {
             // (every column is a real key that every row sees, but for the last tiles of a unit)
             const bool whole = valid == TILE_KEYS && key0 + TILE_KEYS <= Lu - a.W_local;
             const int vh = min(64, valid - (int)col0);
@@ -774,23 +798,33 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
               }
             }
             if (!rows0 || !whole) release_buffer(empty_bar, lane);
-            if (kWide) {
-              if (!second_block()) {
-                ok = false;
-                break;
-              }
-              if (rows1) {
-                if (whole) {
-                  stats_cols64<kPolyS1, kWide>(taddr + 128u + col0, c, m1, l1, v, true, empty_bar1, lane);
-                } else {
-                  const float2 r =
-                      stats_cols_ragged(taddr + 128u + col0, vh, min(vh, vis1 - key0 - (int)col0), c, m1, l1);
-                  m1 = r.x;
-                  l1 = r.y;
-                }
-              }
-              if (!rows1 || !whole) release_buffer(empty_bar1, lane);
+            if (!second_block()) {
+              ok = false;
+              break;
             }
+            if (rows1) {
+              if (whole) {
+                stats_cols64<kPolyS1, kWide>(taddr + 128u + col0, c, m1, l1, v, true, empty_bar1, lane);
+              } else {
+                const float2 r =
+                    stats_cols_ragged(taddr + 128u + col0, vh, min(vh, vis1 - key0 - (int)col0), c, m1, l1);
+                m1 = r.x;
+                l1 = r.y;
+              }
+            }
+            if (!rows1 || !whole) release_buffer(empty_bar1, lane);
+          } else if (valid == TILE_KEYS && key0 + TILE_KEYS <= Lu - a.W_local) {
+            // every column is a real key that every row sees
+            if (rows0) stats_cols64<kPolyS1, kWide>(taddr + col0, c, m0, l0, v, true, empty_bar, lane);
+            if (!rows0) release_buffer(empty_bar, lane);
+          } else {
+            const int vh = min(64, valid - (int)col0);
+            if (rows0) {
+              const float2 r = stats_cols_ragged(taddr + col0, vh, min(vh, vis0 - key0 - (int)col0), c, m0, l0);
+              m0 = r.x;
+              l0 = r.y;
+            }
+            release_buffer(empty_bar, lane);
           }
         } else if (kPerHead) {
           // one column sum per query head: the chunk's 32 rows come as eight groups of four, a
