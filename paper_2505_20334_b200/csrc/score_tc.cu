@@ -686,6 +686,9 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
             for (int i = 0; i < 8; ++i) merge_stat(m, l, pr[i]);
           }
           for (; c0 < n_partials; ++c0) merge_stat(m, l, __ldcg(pp + (int64_t)c0 * a.M_pad));
+          // A row whose logits are all -inf has moved no reference; the sum is 0 on the MUFU, but the FMA-pipe
+          // exponential leaves 2^-126 apiece. It has no softmax: b_r must be -inf and its scores NaN.
+          if (!(m > -1e29f)) l *= 0.f;
           nb = -(m + log2f(l));
         }
         ctl->nboff[s][row] = nb;

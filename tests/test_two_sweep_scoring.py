@@ -156,6 +156,23 @@ def test_two_row_blocks_match_oracle(laq, case):  # noqa: F811
     compare_all_units(laq, q, k, v, W, 7, B, out=out, local_window=Wl, seq_lens=lens, group_mode=group)
 
 
+@pytest.mark.parametrize("G,W,D", [(8, 32, 128), (5, 32, 128), (8, 17, 64), (4, 32, 128), (4, 32, 64)])
+@pytest.mark.parametrize("what", [float("-inf"), float("inf"), float("nan")])
+def test_row_without_a_softmax_is_not_left_out(laq, G, W, D, what):  # noqa: F811
+    # every logit of one row of KV head 0 is -inf, +inf or NaN: that row's attention weights, and with them every
+    # score of the head, are NaN (as in the fp64 definition), and the other head is not touched
+    q, k, v = rand_inputs(1, 1, 2 * G, 2, D, 1000, W, seed=W + D)
+    q[..., 0] = 0.0
+    k[..., 0] = 1.0
+    for row in (0, 2, G * W - 1):
+        bad = q.clone()
+        bad[0, 0, row // W, row % W, 0] = what
+        out = evict_with(laq, bad, k, v, W, 1, W + 20)
+        good = evict_with(laq, q, k, v, W, 1, W + 20)
+        assert out["scores"][0, 0, 0].isnan().all()
+        assert torch.equal(out["scores"][0, 0, 1], good["scores"][0, 0, 1])
+
+
 CUDA_CORES = [
     (1, 1, 3, 1, 136, 500, 32, 0, 7, 60, None, 0),               # head dims above 128 with more than 64 rows
     (1, 2, 8, 2, 192, 900, 32, 16, 5, 90, (900, 333), 0),
