@@ -156,6 +156,15 @@ def test_two_row_blocks_match_oracle(laq, case):  # noqa: F811
     compare_all_units(laq, q, k, v, W, 7, B, out=out, local_window=Wl, seq_lens=lens, group_mode=group)
 
 
+@pytest.mark.parametrize("W,G", [(4, 18), (4, 64), (8, 9), (8, 17), (16, 5), (16, 11), (32, 3), (32, 5), (64, 2), (64, 3)])
+def test_heads_of_every_window(laq, W, G):  # noqa: F811
+    # one column sum per head: every window that takes this path, with one row block (72 to 128 rows) and with
+    # two, heads that end inside a chunk of 32 rows, with it, and over two, and a last chunk that is not full
+    q, k, v = rand_inputs(1, 1, G, 1, 128, 700, W, seed=W + G, kscale=1.5)
+    out = evict_with(laq, q, k, v, W, 7, W + 20, group=2, want="score_tc_kernel")
+    compare_all_units(laq, q, k, v, W, 7, W + 20, out=out, group_mode=2)
+
+
 @pytest.mark.parametrize("G,W,D", [(8, 32, 128), (5, 32, 128), (8, 17, 64), (4, 32, 128), (4, 32, 64)])
 @pytest.mark.parametrize("what", [float("-inf"), float("inf"), float("nan")])
 def test_row_without_a_softmax_is_not_left_out(laq, G, W, D, what):  # noqa: F811
