@@ -84,14 +84,18 @@ struct ClArgs {
   int n_stages;      // K stages
   int slots_log2;    // TMEM tiles
   int stride_log2;   // TMEM columns per tile
-  int C, c_log2;     // CTAs per cluster; log2 of it where that is a whole number
-  int full_tiles, more_tiles;  // prompts of L positions: tiles of every CTA; CTAs that have one more
+  int c_log2;        // log2 of the cluster size where that is a whole number
   float scale_log2;
   int keep_status;    // the status words keep what an earlier piece of the call recorded
   int withhold_unit;  // test hook: this unit's statistics are never sent (-1: none)
   int32_t* hdr;
   float* colsum;
   SeqLens sl;
+  // For cluster sizes between the powers of two, and behind the rest: between the fields above they changed
+  // which of those one load fetches, and with it the registers of the kernels that never read them (64 rows
+  // 96 for 94, with spills; us, 32 units of 2943 keys 15.4, so 14.6; 16 units of 7353 keys, 64 dims 19.8 / 18.9).
+  int C;                       // CTAs per cluster
+  int full_tiles, more_tiles;  // prompts of L positions: tiles of every CTA; CTAs that have one more
 };
 
 // Control block in dynamic shared memory, behind the K and Q stages.
