@@ -867,17 +867,89 @@ bool cluster_counts(int dev, ClusterCounts* out) {
   return true;
 }
 
+// CTAs per cluster for a call whose units have up to n_tiles tiles; 0: no cluster holds a unit.
+int cluster_size(const Dims& d, int n_tiles, int slots, const ClusterCounts& counts) {
+  // Among the powers of two: ceil(U / clusters) rounds of T tiles per CTA. Cycles as measured on B200: a
+  // tile takes the arithmetic of both passes or the CTA's share of the HBM stream (3600 bytes per cycle, at
+  // most 30 per SM). The exchange of a unit is hidden where its tiles leave room for as many of the next
+  // unit's, costs about 1000 where they leave some, and 3000 where they leave none. Large clusters leave
+  // SMs idle (15 of 8 CTAs and 7 of 16 fit the 148), small ones fit fewer keys.
+  const int boxes = (d.D + 63) / 64;
+  int best = 0;
+  double best_cost = 0.0;
+  for (int C = 1; C <= kMaxCluster; C *= 2) {
+    const int n = counts.resident[C], T = (n_tiles + C - 1) / C;
+    if (n < 1 || T > slots || C > n_tiles) continue;
+    const double rounds = (double)((d.U + n - 1) / n);
+    const double tile = fmax(200.0 + 20.0 * d.M, (double)(boxes * kBoxBytes) * fmax(n * C, 120.0) / 3600.0);
+    const double exchange = 2 * T <= slots ? 60.0 * C : (T < slots ? 1000.0 : 3000.0);
+    const double cost = rounds * (T * tile + exchange);
+    if (best == 0 || cost < best_cost) {
+      best = C;
+      best_cost = cost;
+    }
+  }
+  if (best == 0 || d.sl.n > 0) return best;
+  // A size between the powers of two (the 148 SMs hold 45 clusters of 3 CTAs, 26 of 5, 22 of 6, 15 of 7 to
+  // 9, 11 of 10, 7 of 11 to 16) where 3 % or more are expected of it. A round takes the longest of: the HBM
+  // stream, shared by the clusters of an average round, with its end exposed where the tiles leave no room
+  // for the next unit's; the arithmetic, likewise; the chain from the first MMA of a unit through the exchange
+  // to the end of pass 2, of which two can be under way (what short units are bound by: without it 512
+  // units of 582 keys and 16 rows took 31.7 us in clusters of 5, 20.1 alone); and, with one sum per head,
+  // pass 2 of the busier of the two warpgroups, row by row where heads are no groups of four rows. The last unit's pass 2 ends the call. Fitted to the times of
+  // all sizes on 4500 shapes of up to 65536 keys, K from HBM: the size taken is 1.7 % above the best one on
+  // average, the powers of two alone 4.4 %. On 3700 other shapes it is 2.0 % faster than those on average;
+  // 57 are more than 1.5 % slower, 24 more than 3 %, two 15 %. To rank the powers of two by the same costs
+  // gains another 0.3 %, but makes 129 of the 4500 shapes slower than they were.
+  // Not for prompts of different lengths, which leave CTAs of a cluster without tiles in ways that this does
+  // not foresee (3 prompts of 1319 to 6597 keys: 4 % slower).
+  const auto cycles = [&](int C) {
+    const int n = counts.resident[C], T = (n_tiles + C - 1) / C;
+    const double rounds = (double)((d.U + n - 1) / n), full = (double)T / slots;
+    const double sms = (double)d.U / rounds * C;  // of an average round
+    const double stream = T * (d.D / 64.0) * fmax(426.0, kBoxBytes * sms / 3860.0) + fmax(0.0, 2800.0 * (full - 0.52));
+    const double math = T * (720.0 + 8.0 * d.M) + fmax(0.0, 2600.0 * (full - 0.516));
+    const double chain = 1900.0 + 39.0 * d.M + 33.0 * C;
+    const double heads = d.group_mode == LAQ_GROUP_SUM ? 0.0 : (T + 1) / 2 * (1200.0 + (d.W % 4 ? 30.0 : 5.5) * d.M);
+    return rounds * fmax(fmax(stream, math), fmax(chain, heads)) + T * (233.0 + 0.84 * d.M);
+  };
+  best_cost = 0.97 * cycles(best);
+  for (int C = 3; C < kMaxCluster; ++C) {
+    if ((C & (C - 1)) == 0 || counts.resident[C] < 1 || (n_tiles + C - 1) / C > slots || C > n_tiles) continue;
+    const double cost = cycles(C);
+    if (cost < best_cost) {
+      best = C;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
 int log2_ceil(int x) {
   int l = 0;
   while ((1 << l) < x) ++l;
   return l;
 }
 
-}  // namespace
+#ifdef LAQ_TEST_HOOKS
+std::atomic<int> g_last_cluster{0};
+#endif
 
+}  // namespace
+}  // namespace laq
+
+#ifdef LAQ_TEST_HOOKS
+// Test builds only: CTAs per cluster of the last scoring call that took this kernel, 0 if the last one did not.
+extern "C" __attribute__((visibility("default"))) int laq_test_last_cluster() { return laq::g_last_cluster.load(); }
+#endif
+
+namespace laq {
 laq_status score_cluster_launch(const laq_params& p, const Dims& d, const Workspace& w, const void* q,
                                 const void* k, char* ws, cudaStream_t stream, int* launches, bool* done) {
   *done = false;
+#ifdef LAQ_TEST_HOOKS
+  g_last_cluster = 0;
+#endif
   // the caller's scheduling knobs belong to the two-sweep kernel
   if (d.M > kMaxRows || d.U > 0x3fffffff || d.D > 256 || d.tiles_per_task > 0 || d.sched_lag_tasks > 0)
     return LAQ_OK;
@@ -892,52 +964,7 @@ laq_status score_cluster_launch(const laq_params& p, const Dims& d, const Worksp
   a.stride_log2 = d.M <= 16 ? 4 : log2_ceil(d.M);
   a.slots_log2 = 9 - a.stride_log2;
   const int n_tiles = w.L_pad / TILE_KEYS, slots = 1 << a.slots_log2;
-  // The cluster size: ceil(U / clusters) rounds of T tiles per CTA. Cycles as measured on B200: a tile
-  // takes the arithmetic of both passes or the CTA's share of the HBM stream (3600 bytes per cycle, at
-  // most 30 per SM). The exchange of a unit is hidden where its tiles leave room for as many of the next
-  // unit's, costs about 1000 where they leave some, and 3000 where they leave none. Large clusters leave
-  // SMs idle (15 of 8 CTAs and 7 of 16 fit the 148), small ones fit fewer keys.
-  // L 6007, 64 rows, 256 units: 102 us with 8 CTAs, 121 with 16; L 4096: 67 / 63 us with 4 / 8; 64-dim
-  // heads, 32 rows, L 4096, 128 units: 26.1 / 24.6 / 27.0 us with 2 / 4 / 8.
-  int best = 0;
-  double best_cost = 0.0;
-  for (int C = 1; C <= kMaxCluster; C *= 2) {
-    const int n = counts.resident[C], T = (n_tiles + C - 1) / C;
-    if (n < 1 || T > slots || C > n_tiles) continue;
-    const double rounds = (double)((d.U + n - 1) / n);
-    const double tile = fmax(200.0 + 20.0 * d.M, (double)(a.boxes * kBoxBytes) * fmax(n * C, 120.0) / 3600.0);
-    const double exchange = 2 * T <= slots ? 60.0 * C : (T < slots ? 1000.0 : 3000.0);
-    const double cost = rounds * (T * tile + exchange);
-    if (best == 0 || cost < best_cost) {
-      best = C;
-      best_cost = cost;
-    }
-  }
-  // Sizes between the powers of two, where 3 % or more are expected of them: the 148 SMs hold 45 clusters of
-  // 3 CTAs, 26 of 5, 22 of 6, 15 of 7 to 9, 11 of 10, 7 of 11 to 16, and the units fill the tensor memory and the
-  // last round better or worse. Fitted to sizes of all kinds (a round is the arithmetic and the exposed part
-  // of the exchange, or the CTA's share of the HBM stream and its exposed end). us on 256 units, 64 rows:
-  // L 9000 142 with 9, 180 with 16; L 6007 99 / 101 / 105 with 6 / 9 / 8; L 2500 45 / 49 with 5 / 4; 40 rows, L 2850
-  // 43 / 47 with 6 / 4; 32 rows, 96 dims, L 15018 159 / 169 / 177 with 9 / 10 / 16; 512 units of 16 rows, L 11612 153 / 155
-  // / 180 with 7 / 8 / 4. Not for prompts of different lengths, which leave CTAs of a cluster without tiles in
-  // ways that this does not foresee (3 prompts of 1319 to 6597 keys: 4 % slower).
-  const auto round_cycles = [&](int C) {
-    const int n = counts.resident[C], T = (n_tiles + C - 1) / C;
-    const double rounds = (double)((d.U + n - 1) / n), sms = (double)(d.U < n ? d.U : n) * C;
-    const double full = (double)T / slots;
-    const double math = T * (200.0 + 20.0 * d.M) + fmax(0.0, 2200.0 * (2.0 * full - 1.0));
-    const double stream = T * (double)(a.boxes * kBoxBytes) * fmax(sms, 116.0) / 3830.0 + fmax(0.0, 8000.0 * (full - 0.75));
-    return rounds * (fmax(math, stream) + 20.0 * C);
-  };
-  best_cost = best > 0 ? round_cycles(best) : 0.0;
-  for (int C = 3; C < kMaxCluster && d.sl.n == 0; ++C) {
-    if ((C & (C - 1)) == 0 || counts.resident[C] < 1 || (n_tiles + C - 1) / C > slots || C > n_tiles) continue;
-    const double cost = round_cycles(C);
-    if (best == 0 || cost < 0.97 * best_cost) {
-      best = C;
-      best_cost = cost;
-    }
-  }
+  const int best = cluster_size(d, n_tiles, slots, counts);
   if (best == 0) return LAQ_OK;
   const int C = best;
   const bool pow2 = (C & (C - 1)) == 0;
@@ -990,6 +1017,9 @@ laq_status score_cluster_launch(const laq_params& p, const Dims& d, const Worksp
     return LAQ_ERR_CUDA;
   *launches += 1;
   *done = true;
+#ifdef LAQ_TEST_HOOKS
+  g_last_cluster = C;
+#endif
   return LAQ_OK;
 }
 

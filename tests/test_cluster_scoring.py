@@ -1,12 +1,15 @@
 """Scoring with the logits of a unit kept in the tensor memory of a thread-block cluster (up to 64
 softmax rows): the sizes at which tiles, row groups, clusters and head dims end, against the fp64
 oracle with the tolerances of the other parity tests."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
 
 from parity_util import SCORE_RTOL
 from test_gpu_parity import compare_all_units, laq, rand_inputs  # noqa: F401 (laq is a fixture)
+from test_timeout_path import hooked_library
 
 pytestmark = pytest.mark.gpu
 
@@ -79,29 +82,45 @@ def test_cluster_scoring_many_short_units_of_few_rows(laq, W, L, lens):
     assert torch.equal(out["scores"], first["scores"]) and torch.equal(out["idx"], first["idx"])
 
 
-@pytest.mark.parametrize("units,G,W,D,L,lens", [
-    (256, 4, 16, 128, 2500, None),                 # clusters of 5, four tiles a CTA
-    (256, 4, 16, 128, 6007, None),                 # of 6, all slots of the tensor memory
-    (256, 4, 16, 128, 9000, None),                 # of 9
-    (256, 4, 16, 128, 9000, (9000, 5001, 1153, 129)),  # (prompts of different lengths: of 16)
-    (64, 4, 12, 128, 3000, None),                  # of 6
-    (16, 2, 4, 64, 6646, None),
-    (1184, 4, 16, 128, 384, None),                 # of 1 or 3: odd numbers of tiles a unit, many rounds
+@pytest.mark.parametrize("units,G,W,D,L,lens,group,C", [
+    # between the powers of two
+    (256, 4, 16, 128, 2500, None, 0, 5),                 # four tiles a CTA
+    (256, 4, 16, 128, 6007, None, 0, 6),                 # all slots of the tensor memory
+    (256, 4, 16, 128, 9000, None, 0, 9),
+    (64, 4, 12, 128, 3000, None, 0, 6),
+    (16, 2, 4, 64, 6646, None, 0, 6),
+    (40, 5, 8, 128, 3000, None, 2, 6),                   # one sum per head
+    # powers of two
+    (256, 4, 16, 128, 9000, (9000, 5001, 1153, 129), 0, 16),   # (prompts of different lengths take no other)
+    (256, 4, 16, 128, 4096, None, 0, 8),
+    (1184, 4, 16, 128, 384, None, 0, 1),                 # many rounds of short units: bound by the chain from a unit's
+    (512, 4, 4, 128, 582, None, 0, 1),                   # first MMA to the end of its pass 2, which a cluster does
+    (256, 1, 4, 96, 539, None, 0, 1),                    # not shorten
+    (224, 8, 8, 128, 639, None, 2, 1),
+    (896, 4, 12, 128, 555, None, 0, 2),
+    (56, 4, 8, 128, 2218, None, 0, 4),
 ])
-def test_clusters_of_any_size(laq, units, G, W, D, L, lens):
+def test_clusters_of_any_size(laq, units, G, W, D, L, lens, group, C):
     # against the other tensor-core kernel (which a task size set by the caller selects). Both sum the same
     # exponentials, arguments rounded to fp32, in other orders: 2^-21 in the 2-norm apiece.
     Bt, Hkv = (len(lens) if lens else 1), 8
-    NL = max(1, units // (Bt * Hkv))
+    NL = units // (Bt * Hkv)
     g = torch.Generator(device="cuda").manual_seed(L)
     q = torch.randn((NL, Bt, G * Hkv, W, D), generator=g, device="cuda", dtype=torch.bfloat16)
     k = torch.randn((NL, Bt, Hkv, L, D), generator=g, device="cuda", dtype=torch.bfloat16)
     p = laq.params_for(q, k, W, 1, W + 20)
     p.set_seq_lens(lens)
-    got = torch.full((NL, Bt, Hkv, L - W), float("nan"), device="cuda")
+    p.group_mode = group
+    got = torch.full((NL, Bt, Hkv * (G if group == 2 else 1), L - W), float("nan"), device="cuda")
     ws = laq.alloc_workspace(p, "cuda")
     laq.laq_score(p, q, k, got, ws)
     assert laq.laq_last_device_status(p, ws) == laq.LAQ_OK
+    hooked = hooked_library()               # (the same code, and says which size it launched)
+    again = torch.full_like(got, float("nan"))
+    assert hooked.laq_score(ctypes.byref(p), q.data_ptr(), k.data_ptr(), again.data_ptr(), ws.data_ptr(), ws.numel(),
+                            torch.cuda.current_stream().cuda_stream) == laq.LAQ_OK
+    assert hooked.laq_test_last_cluster() == C
+    assert torch.equal(got, again)
     p.tiles_per_task = 8
     want = torch.empty_like(got)
     laq.laq_score(p, q, k, want, laq.alloc_workspace(p, "cuda"))
