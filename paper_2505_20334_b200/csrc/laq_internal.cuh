@@ -114,6 +114,8 @@ laq_status score_tc_launch(const laq_params& p, const Dims& d, const Workspace& 
 // (*done says whether it was launched; if not, nothing was enqueued).
 laq_status score_cluster_launch(const laq_params& p, const Dims& d, const Workspace& w, const void* q,
                                 const void* k, char* ws, cudaStream_t stream, int* launches, bool* done);
+// Its kernels for cluster sizes between the powers of two (variant: groups of eight rows - 1).
+const void* cluster_kernel_between(bool per_head, int variant);
 // Unit whose statistics a test build withholds (-1 in the library).
 int64_t test_withhold_unit();
 // Raw-logit mode (Eq. 4 read literally): one streaming pass over K on CUDA cores.

@@ -812,24 +812,40 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
   }
 }
 
-typedef void (*ClusterKernel)(const CUtensorMap, const CUtensorMap, const ClArgs);
-// [power of two][per head][groups of eight rows - 1] (seven groups run as eight)
+#ifdef LAQ_SIZES_BETWEEN
+constexpr bool kPow2 = false;
+#else
+constexpr bool kPow2 = true;
+#endif
+// [per head][groups of eight rows - 1] (seven groups run as eight)
 constexpr int kVariants = 8;
-#define LAQ_VARIANTS(H, P)                                                                                \
-  {score_cluster_kernel<1, H, P>, score_cluster_kernel<2, H, P>, score_cluster_kernel<3, H, P>,           \
-   score_cluster_kernel<4, H, P>, score_cluster_kernel<5, H, P>, score_cluster_kernel<6, H, P>,           \
-   score_cluster_kernel<8, H, P>, score_cluster_kernel<8, H, P>}
-const ClusterKernel kKernels[2][2][kVariants] = {{LAQ_VARIANTS(false, false), LAQ_VARIANTS(true, false)},
-                                                 {LAQ_VARIANTS(false, true), LAQ_VARIANTS(true, true)}};
+#define LAQ_VARIANTS(H)                                                                                      \
+  {(const void*)score_cluster_kernel<1, H, kPow2>, (const void*)score_cluster_kernel<2, H, kPow2>,           \
+   (const void*)score_cluster_kernel<3, H, kPow2>, (const void*)score_cluster_kernel<4, H, kPow2>,           \
+   (const void*)score_cluster_kernel<5, H, kPow2>, (const void*)score_cluster_kernel<6, H, kPow2>,           \
+   (const void*)score_cluster_kernel<8, H, kPow2>, (const void*)score_cluster_kernel<8, H, kPow2>}
+const void* const kKernels[2][kVariants] = {LAQ_VARIANTS(false), LAQ_VARIANTS(true)};
 #undef LAQ_VARIANTS
 
-// Clusters of each size that the device keeps resident with this kernel's resources, one CTA per SM;
+#ifdef LAQ_SIZES_BETWEEN
+}  // namespace
+
+const void* cluster_kernel_between(bool per_head, int variant) { return kKernels[per_head ? 1 : 0][variant]; }
+#else
+
+// Clusters of each size that the device keeps resident with these kernels' resources, one CTA per SM;
 // looked up once per device. 0: that cluster size cannot be launched.
 constexpr int kMaxCluster = 16;
 struct ClusterCounts {
   int resident[kMaxCluster + 1];
 };
 constexpr size_t kSmemBytes = 227 * 1024;
+
+// What a kernel needs to be launched with all shared memory and in clusters of any size, per device.
+bool allow_launch(const void* kernel) {
+  return cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes)) &&
+         cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+}
 
 bool cluster_counts(int dev, ClusterCounts* out) {
   static std::mutex mutex;
@@ -839,12 +855,8 @@ bool cluster_counts(int dev, ClusterCounts* out) {
   if (!known[dev].load(std::memory_order_acquire)) {
     std::lock_guard<std::mutex> lock(mutex);
     if (!known[dev].load(std::memory_order_relaxed)) {
-      for (int i = 0; i < 4 * kVariants; ++i) {
-        const ClusterKernel kernel = kKernels[i / (2 * kVariants)][i / kVariants % 2][i % kVariants];
-        if (!cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes)) ||
-            !cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)))
-          return false;
-      }
+      for (int i = 0; i < 2 * kVariants; ++i)
+        if (!allow_launch(kKernels[i / kVariants][i % kVariants])) return false;
       for (int i = 1; i <= kMaxCluster; ++i) {
         cudaLaunchAttribute attr;
         attr.id = cudaLaunchAttributeClusterDimension;
@@ -857,7 +869,7 @@ bool cluster_counts(int dev, ClusterCounts* out) {
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
         int n = 0;
-        if (!cuda_ok(cudaOccupancyMaxActiveClusters(&n, kKernels[(i & (i - 1)) == 0][0][kVariants - 1], &cfg))) n = 0;
+        if (!cuda_ok(cudaOccupancyMaxActiveClusters(&n, kKernels[0][kVariants - 1], &cfg))) n = 0;
         cached[dev].resident[i] = n;
       }
       known[dev].store(true, std::memory_order_release);
@@ -923,6 +935,22 @@ int cluster_size(const Dims& d, int n_tiles, int slots, const ClusterCounts& cou
     }
   }
   return best;
+}
+
+// The kernel of these rows for a size, ready to be launched on this device (0 <= dev < kMaxDevices). Those for
+// sizes between the powers of two are a module of their own (score_cluster_between.cu), loaded when one of
+// them is first wanted: a process's first scoring call took 12.6 ms with all of them in one, and takes 10.3;
+// the first call of such a size 1.7.
+const void* use_size(int dev, bool pow2, bool per_head, int variant) {
+  if (pow2) return kKernels[per_head ? 1 : 0][variant];
+  static std::atomic<uint32_t> allowed[kMaxDevices];
+  const void* kernel = cluster_kernel_between(per_head, variant);
+  const uint32_t bit = 1u << (variant + (per_head ? kVariants : 0));
+  if (!(allowed[dev].load(std::memory_order_acquire) & bit)) {
+    if (!allow_launch(kernel)) return nullptr;
+    allowed[dev].fetch_or(bit, std::memory_order_release);
+  }
+  return kernel;
 }
 
 int log2_ceil(int x) {
@@ -1013,8 +1041,9 @@ laq_status score_cluster_launch(const laq_params& p, const Dims& d, const Worksp
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  if (!cuda_ok(cudaLaunchKernelEx(&cfg, kKernels[pow2 ? 1 : 0][per_head ? 1 : 0][variant], tmap_q, tmap_k, a)))
-    return LAQ_ERR_CUDA;
+  const void* kernel = use_size(dev, pow2, per_head, variant);
+  void* args[] = {&tmap_q, &tmap_k, &a};
+  if (!kernel || !cuda_ok(cudaLaunchKernelExC(&cfg, kernel, args))) return LAQ_ERR_CUDA;
   *launches += 1;
   *done = true;
 #ifdef LAQ_TEST_HOOKS
@@ -1022,5 +1051,6 @@ laq_status score_cluster_launch(const laq_params& p, const Dims& d, const Worksp
 #endif
   return LAQ_OK;
 }
+#endif  // !LAQ_SIZES_BETWEEN
 
 }  // namespace laq

@@ -2,6 +2,9 @@
 softmax rows): the sizes at which tiles, row groups, clusters and head dims end, against the fp64
 oracle with the tolerances of the other parity tests."""
 import ctypes
+import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -125,3 +128,40 @@ def test_clusters_of_any_size(laq, units, G, W, D, L, lens, group, C):
     want = torch.empty_like(got)
     laq.laq_score(p, q, k, want, laq.alloc_workspace(p, "cuda"))
     assert float((got - want).norm() / want.norm()) < 1e-6
+
+
+FIRST_USE = """
+import sys
+sys.path.insert(0, {root!r})
+import torch
+from paper_2505_20334_b200 import binding as laq
+g = torch.Generator(device="cuda").manual_seed(1)
+def problem(L, group):
+    q = torch.randn((4, 1, 8, 8, 128), generator=g, device="cuda", dtype=torch.bfloat16)
+    k = torch.randn((4, 1, 2, L, 128), generator=g, device="cuda", dtype=torch.bfloat16)
+    p = laq.params_for(q, k, 8, 7, 40)
+    p.group_mode = group
+    s = torch.full((4, 1, 8 if group == 2 else 2, L - 8), float("nan"), device="cuda")
+    return p, q, k, s, laq.alloc_workspace(p, "cuda")
+laq.laq_score(*problem(512, 0))                 # a cluster of 4 CTAs: the library is up
+for group in (0, 2):
+    p, q, k, s, ws = problem(1100, group)       # of 9
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        laq.laq_score(p, q, k, s, ws)
+    assert s.isnan().all()                      # captured, not run
+    graph.replay()
+    torch.cuda.synchronize()
+    assert laq.laq_last_device_status(p, ws) == laq.LAQ_OK
+    again = torch.empty_like(s)
+    laq.laq_score(p, q, k, again, ws)
+    assert torch.equal(s, again)
+"""
+
+
+def test_first_use_of_a_cluster_size_may_be_captured():
+    # the kernels of sizes between the powers of two are loaded when first wanted, also under a capture
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", FIRST_USE.format(root=root)], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
