@@ -70,6 +70,50 @@ def test_cluster_scoring_sums_that_overflow(laq):
     assert np.isfinite(out["k_out"].float().cpu().numpy()).all()
 
 
+def launched_cluster(laq, q, k, R, kernel, B, group=0):  # noqa: F811
+    """CTAs per cluster of a scoring call of these sizes (0: another kernel takes it)."""
+    p = laq.params_for(q, k, R, kernel, B)
+    p.group_mode = group
+    ws = laq.alloc_workspace(p, "cuda")
+    H = q.shape[2] if group == 2 else k.shape[2]
+    scores = torch.empty((q.shape[0], q.shape[1], H, k.shape[3] - R), device="cuda")
+    hooked = hooked_library()
+    assert hooked.laq_score(ctypes.byref(p), q.cuda().data_ptr(), k.cuda().data_ptr(), scores.data_ptr(), ws.data_ptr(),
+                            ws.numel(), torch.cuda.current_stream().cuda_stream) == laq.LAQ_OK
+    torch.cuda.synchronize()
+    return hooked.laq_test_last_cluster()
+
+
+# clusters whose CTAs hold several tiles of a unit: nine with two tiles, sixteen with three and four
+SIZES = [(2304, 9), (8192, 16)]
+
+
+@pytest.mark.parametrize("L,C", SIZES)
+@pytest.mark.parametrize("G,W,group", [(4, 4, 0), (4, 16, 0), (3, 19, 0), (8, 8, 2), (4, 3, 2)])
+def test_sums_that_overflow_in_clusters_of(laq, L, C, G, W, group):
+    # as above, every warp with more than one tile: its reference lies 120 nats below the largest key, in
+    # some warps in their first tile and in some in a later one
+    Hkv, D, kernel, B = 2, 128, 7, W + 90
+    q, k, v = rand_inputs(1, 1, G * Hkv, Hkv, D, L, W, seed=L + W)
+    q[..., 0] = 12.0
+    k[..., 0] = 0.0
+    k[:, :, :, ::32, 0] = -56.0
+    for j in (5, 300, 1500, L - 200):
+        k[:, :, :, j, 0] = 56.0
+    assert launched_cluster(laq, q, k, W, kernel, B, group) == C
+    err, _ = compare_all_units(laq, q, k, v, W, kernel, B, group_mode=group)
+    assert err < SCORE_RTOL
+
+
+@pytest.mark.parametrize("L,C", SIZES)
+@pytest.mark.parametrize("W,G", [(1, 4), (3, 4), (5, 8), (6, 4), (8, 7), (16, 4)])
+def test_cluster_scoring_per_head_with_several_tiles(laq, L, C, W, G):
+    q, k, v = rand_inputs(1, 1, 2 * G, 2, 128, L, W, seed=L + W, kscale=1.5)
+    for mode in (1, 2):
+        assert launched_cluster(laq, q, k, W, 7, 80, mode) == C
+        compare_all_units(laq, q, k, v, W, 7, 80, group_mode=mode)
+
+
 @pytest.mark.parametrize("W,L,lens", [(1, 128, None), (2, 700, None), (4, 500, tuple([500, 131] * 16))])
 def test_cluster_scoring_many_short_units_of_few_rows(laq, W, L, lens):
     # At most 32 rows: one of the two exchange warps has no row of its own. Three and more units fit the

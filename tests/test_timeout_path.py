@@ -140,3 +140,39 @@ def test_wait_that_runs_out_in_the_other_scoring_kernels(G, W, tiles, group):
         scores.zero_()
         assert run(lib) == laq.LAQ_OK
         assert torch.equal(scores, want)
+
+
+@pytest.mark.parametrize("G,W", [(1, 8), (2, 8), (3, 8), (4, 8), (5, 8), (6, 8), (8, 8)])   # every group of eight rows
+@pytest.mark.parametrize("L,C", [(2304, 9), (8192, 16)])
+@pytest.mark.parametrize("group", [0, 2])
+def test_wait_that_runs_out_in_clusters(G, W, L, C, group):
+    # every variant of the cluster kernel, for a size between the powers of two and for one of them
+    from paper_2505_20334_b200 import binding as laq
+
+    hooked = hooked_library()
+    Hkv, D = 2, 128
+    g = torch.Generator(device="cuda").manual_seed(G + L)
+    q = torch.randn((1, 1, G * Hkv, W, D), generator=g, device="cuda", dtype=torch.bfloat16)
+    k = torch.randn((1, 1, Hkv, L, D), generator=g, device="cuda", dtype=torch.bfloat16)
+    p = laq.params_for(q, k, W, 7, 100)
+    p.group_mode = group
+    ws = laq.alloc_workspace(p, "cuda")
+    scores = torch.zeros((1, 1, Hkv * (G if group == 2 else 1), L - W), device="cuda")
+    stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+
+    def run():
+        scores.zero_()
+        assert hooked.laq_score(ctypes.byref(p), q.data_ptr(), k.data_ptr(), scores.data_ptr(), ws.data_ptr(),
+                                ws.numel(), stream) == laq.LAQ_OK
+        assert hooked.laq_test_last_cluster() == C
+        return hooked.laq_last_device_status(ctypes.byref(p), ws.data_ptr(), ws.numel(), stream)
+
+    assert run() == laq.LAQ_OK
+    want = scores.clone()
+    hooked.laq_test_withhold_unit(1)
+    try:
+        assert run() == laq.LAQ_ERR_TIMEOUT
+    finally:
+        hooked.laq_test_withhold_unit(-1)
+    assert run() == laq.LAQ_OK
+    assert torch.equal(scores, want)

@@ -25,6 +25,20 @@ def test_scores_of_other_head_dims_are_as_precise_as_fp32_sums(laq, D, W):  # no
     assert np.linalg.norm(got - ref) <= 4.8e-7 * np.linalg.norm(ref)
 
 
+@pytest.mark.parametrize("D", [64, 80, 128])
+@pytest.mark.parametrize("G,W,L", [(8, 17, 3000), (5, 32, 3000), (8, 32, 3000), (8, 32, 600)])     # 136, 160, 256 rows
+@pytest.mark.parametrize("group", [0, 2])
+def test_scores_of_two_row_blocks_are_as_precise_as_fp32_sums(laq, G, W, L, D, group):  # noqa: F811
+    # the same bound. An eighth of sweep 1's exponentials comes from a polynomial of degree 5 on the FMA pipe:
+    # the one of degree 3 that 65 to 128 rows of 128 dims take leaves 1e-6, and must not be in its place.
+    # One column sum per head with a window of 17 is formed on CUDA cores.
+    q, k, v = rand_inputs(1, 1, 2 * G, 2, D, L, W, seed=D + W + G)
+    out = laq.evict(q.cuda(), k.cuda(), v.cuda(), 100, want_scores=True, group_mode=group)
+    ref = orc.evict(q, k, v, W, 7, 100, group_mode=group)["scores"]
+    got = out["scores"].cpu().numpy().astype(np.float64)
+    assert np.linalg.norm(got - ref) <= 4.8e-7 * np.linalg.norm(ref)
+
+
 @pytest.mark.parametrize("W", [8, 32])          # 32 and 128 rows
 def test_one_workspace_serves_batches_of_other_lengths(laq, W):  # noqa: F811
     # sized for the allocated batch, then used for batches of shorter prompts and for fewer layers: the
@@ -138,7 +152,7 @@ TWO_BLOCKS = [
     (2, 1, 5, 257, 32, 16, 0, None, 0),           # 160 rows, two tiles and a key
     (1, 2, 7, 640, 32, 32, 1, (640, 130), 0),     # 224 rows, a task per tile, all queries local
     (1, 1, 8, 1153, 32, 0, 3, None, 0),           # 256 rows, tasks of three tiles
-    (3, 2, 6, 4500, 32, 5, 0, (4500, 1000), 0),   # 192 rows, several tasks, CTAs with several units
+    (3, 2, 6, 4500, 32, 5, 0, (4500, 1000), 0),   # 192 rows, several tasks a unit
     (1, 1, 5, 900, 32, 0, 0, None, 2),            # one column sum per head, second block of one chunk
     (1, 1, 4, 1300, 64, 8, 2, None, 1),           # heads of two chunks
 ]
@@ -180,6 +194,51 @@ def test_row_without_a_softmax_is_not_left_out(laq, G, W, D, what):  # noqa: F81
         good = evict_with(laq, q, k, v, W, 1, W + 20)
         assert out["scores"][0, 0, 0].isnan().all()
         assert torch.equal(out["scores"][0, 0, 1], good["scores"][0, 0, 1])
+
+
+# Batches of many more tasks than SMs, so that every CTA takes tasks of both sweeps and of several units in
+# turn: the one Q stage, the ring of K stages and the phases of the accumulators run on across them.
+MANY_TASKS = [
+    # Bt G  L     W  W_local tiles ragged group
+    (32, 5, 2300, 32, 0, 0, False, 0),            # 160 rows, 64 units
+    (32, 8, 3000, 32, 16, 0, False, 0),           # 256 rows, local queries
+    (40, 8, 1500, 32, 0, 1, True, 0),             # 256 rows, a task per tile, prompts of different lengths
+    (32, 6, 5000, 32, 5, 3, True, 0),             # 192 rows, tasks of three tiles
+    (24, 8, 4100, 17, 17, 5, False, 0),           # 136 rows, odd numbers of tiles a task
+    (32, 5, 2000, 32, 0, 0, True, 2),             # one column sum per head
+    (32, 8, 1700, 32, 8, 3, False, 1),
+]
+
+
+@pytest.mark.parametrize("case", MANY_TASKS, ids=[f"M{c[1] * c[3]}-L{c[2]}-t{c[5]}-g{c[7]}" for c in MANY_TASKS])
+def test_two_row_blocks_through_many_tasks(laq, case):  # noqa: F811
+    # Against the CUDA-core kernel, which a layer stride that no tensor map holds selects (with one layer it is
+    # never used): fp32 sums of the same terms in other orders, 2^-21 in the 2-norm apiece.
+    Bt, G, L, W, Wl, tiles, ragged, group = case
+    Hkv, D = 2, 128
+    g = torch.Generator(device="cuda").manual_seed(L)
+    q = torch.randn((1, Bt, G * Hkv, W, D), generator=g, device="cuda", dtype=torch.bfloat16)
+    k = torch.randn((1, Bt, Hkv, L, D), generator=g, device="cuda", dtype=torch.bfloat16)
+    lens = [L - b * (L - 2 * W) // Bt for b in range(Bt)] if ragged else None
+    for b, Lb in enumerate(lens or ()):
+        k[:, b, :, Lb:] = float("nan")
+    p = laq.params_for(q, k, W, 1, W + 20)
+    p.tiles_per_task, p.local_window, p.group_mode = tiles, Wl, group
+    p.set_seq_lens(lens)
+    got = torch.zeros((1, Bt, Hkv * (G if group == 2 else 1), L - W), device="cuda")
+    want = torch.zeros_like(got)
+    ws = laq.alloc_workspace(p, "cuda")
+
+    def call():
+        laq.laq_score(p, q, k, got, ws)
+    assert scoring_kernels(call) == {"score_tc_kernel"}
+    for _ in range(3):
+        call()
+        assert laq.laq_last_device_status(p, ws) == laq.LAQ_OK
+        p.k_stride_layer, stride = 1 << 40, p.k_stride_layer
+        laq.laq_score(p, q, k, want, ws)
+        p.k_stride_layer = stride
+        assert not got.isnan().any() and float((got - want).norm() / want.norm()) < 1e-6
 
 
 CUDA_CORES = [
