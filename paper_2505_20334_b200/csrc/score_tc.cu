@@ -296,40 +296,40 @@ __device__ __noinline__ float2 stats_cols_ragged(uint32_t taddr, int valid_max, 
   return make_float2(m, l);
 }
 
-// Sweep 1, this warpgroup's 64 key columns of one row block of a full tile. If `release`, the
-// accumulator buffer is handed back to the MMA warp as soon as the last chunk is in registers.
+// Sweep 1, this warpgroup's 64 key columns of one row block of a full tile. They are handed back to the
+// MMA warp as soon as the last chunk is in registers.
 template <int kPoly, bool kPrecise>
 __device__ __forceinline__ void stats_cols64(uint32_t taddr, float c, float& m, float& l, float* v,
-                                             bool release, uint32_t empty_bar, int lane) {
+                                             uint32_t empty_bar, int lane) {
   tmem_ld32(taddr, v);
   tmem_ld_wait(v);
   stats_chunk<kPoly, kPrecise>(v, c, m, l);
   tmem_ld32(taddr + 32u, v);
   tmem_ld_wait(v);
-  if (release) release_buffer(empty_bar, lane);
+  release_buffer(empty_bar, lane);
   stats_chunk<kPoly, kPrecise>(v, c, m, l);
 }
 
 // ------------------------------------------------------------------ the kernel
 // kDup: M <= 64, sweep 1 holds every query row twice (on TMEM lanes r and 64 + r).
-// kWide: 128 < M <= 256, two row blocks per tile, so an accumulator buffer takes 256 TMEM columns
-// and there are two of them instead of four. A row block's 128 columns are handed over and given back on
-// their own, in both sweeps, so that the MMAs of a pair's next tile run while it is at the second block of
-// this one; and there is one Q stage and room for four K stages, since a stage is now wanted half a tile
-// earlier (the next task's Q arrives while two tiles of this one are still to be exponentiated). 256 rows, us
-// with buffers and stages handed over whole, two of each: 65536 keys, 640 units 7589 -> 7136 (other boards
-// 7431 -> 7122); 16384 keys, 160 units 479 -> 458; 5000 keys 166 -> 157; row blocks alone 7214, 467, 161.
+// kWide: 128 < M <= 256, two row blocks per tile, so an accumulator buffer takes 256 TMEM columns and there
+// are two of them instead of four. A block's 128 columns change hands on their own, in both sweeps: the MMAs
+// of a pair's next tile run while it is at the second block of this one. A K stage is then wanted half a tile
+// earlier, so there are four, and one Q stage (the next task's Q arrives while two tiles of this one are still
+// to be exponentiated). 256 rows, us, all handed over whole, blocks alone, and with the stages: 65536 keys, 640
+// units 7589 / 7214 / 7136; 16384 keys, 160 units 479 / 467 / 458; 5000 keys 166 / 161 / 157.
 // kPerHead: sweep 2 keeps one column sum per query head (colsum is [U*G][L_pad]); the launcher
 // only picks it when a head's rows never straddle a group of four rows or a 32-row chunk unevenly
 // (W a multiple of 4 that divides 32, or 32 or 64).
-// kPolyS1: share of sweep 1's exponentials on the FMA pipe (of every 8 pairs). With more than 128 rows it is
-// 1, of the exponential that is as precise as the MUFU's (scores 1.2e-7 from fp64 in the 2-norm either way):
-// the MUFU alone would take 2048 of a tile's 2570 cycles a sweep (256 rows: 65536 keys, 640 units 7136 -> 6894
-// us; 5000 keys, 160 units 161 -> 156; 64 dims 419 -> 404; 2 of 8 7031, 153, 403; one column sum per head no
-// faster, so none there). With up to 64 rows none pays. For 64 < M <= 128 it is a cheaper one. Its polynomial has a relative error of 7.5e-5, which leaves the scores within 1e-6 of the
-// exact ones in the 2-norm; on the MUFU alone they are within 2e-7. Head dims other than 128 take none, so
-// that their scores are as precise as on CUDA cores, where they used to be formed (64 dims, 128 rows, 128
-// units of 32768 keys: 324 us, with the polynomial 310; 256 units of 4096: 95.4 and 93.9).
+// kPolyS1: of every 8 pairs of sweep 1, how many take an exponential on the FMA pipe.
+//   M > 128, one sum: 1, as precise as the MUFU's (scores 1.2e-7 from fp64 in the 2-norm either way). The MUFU
+//     alone takes 2048 of a tile's 2570 cycles a sweep: 65536 keys, 640 units 7136 -> 6894 us, 5000 keys, 160
+//     units 161 -> 156, 64 dims 419 -> 404 (2 of 8: 7031, 153, 403).
+//   M > 128, a sum per head: 0, it pays nothing there (160 rows 159 -> 164, 256 rows 141 -> 142).
+//   64 < M <= 128, 128 dims: LAQ_POLY_PAIRS_S1 of a cheaper one, 7.5e-5 off, which leaves the scores within
+//     1e-6 (on the MUFU alone 2e-7). Other head dims: 0, so that their scores are as precise as on the CUDA
+//     cores, where they used to be formed (64 dims, 128 rows, 128 units of 32768 keys 324 us, with it 310).
+//   M <= 64: 0, it pays nothing.
 template <bool kDup, bool kWide, bool kPerHead, int kPolyS1>
 __global__ void __launch_bounds__(kThreads, 1)
 score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
@@ -767,7 +767,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
         float v[32];
         if (task.sweep == 0) {
           const int valid = min(TILE_KEYS, Lu - key0);
-          // row blocks beyond the unit's rows are skipped (warp-uniform)
+          // rows beyond the unit's are skipped (warp-uniform; with two row blocks the first one is full)
           const bool rows0 = (kDup ? (quad & 1) : quad) * 32 < a.M;
           const bool rows1 = kWide && 128 + quad * 32 < a.M;
           if (kDup) {
@@ -790,24 +790,21 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
             // (every column is a real key that every row sees, but for the last tiles of a unit)
             const bool whole = valid == TILE_KEYS && key0 + TILE_KEYS <= Lu - a.W_local;
             const int vh = min(64, valid - (int)col0);
-            if (rows0) {
-              if (whole) {
-                stats_cols64<kPolyS1, kWide>(taddr + col0, c, m0, l0, v, true, empty_bar, lane);
-              } else {
-                const float2 r =
-                    stats_cols_ragged(taddr + col0, vh, min(vh, vis0 - key0 - (int)col0), c, m0, l0);
-                m0 = r.x;
-                l0 = r.y;
-              }
+            if (whole) {
+              stats_cols64<kPolyS1, kWide>(taddr + col0, c, m0, l0, v, empty_bar, lane);
+            } else {
+              const float2 r = stats_cols_ragged(taddr + col0, vh, min(vh, vis0 - key0 - (int)col0), c, m0, l0);
+              m0 = r.x;
+              l0 = r.y;
+              release_buffer(empty_bar, lane);
             }
-            if (!rows0 || !whole) release_buffer(empty_bar, lane);
             if (!second_block()) {
               ok = false;
               break;
             }
             if (rows1) {
               if (whole) {
-                stats_cols64<kPolyS1, kWide>(taddr + 128u + col0, c, m1, l1, v, true, empty_bar1, lane);
+                stats_cols64<kPolyS1, kWide>(taddr + 128u + col0, c, m1, l1, v, empty_bar1, lane);
               } else {
                 const float2 r =
                     stats_cols_ragged(taddr + 128u + col0, vh, min(vh, vis1 - key0 - (int)col0), c, m1, l1);
@@ -818,7 +815,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
             if (!rows1 || !whole) release_buffer(empty_bar1, lane);
           } else if (valid == TILE_KEYS && key0 + TILE_KEYS <= Lu - a.W_local) {
             // every column is a real key that every row sees
-            if (rows0) stats_cols64<kPolyS1, kWide>(taddr + col0, c, m0, l0, v, true, empty_bar, lane);
+            if (rows0) stats_cols64<kPolyS1, kWide>(taddr + col0, c, m0, l0, v, empty_bar, lane);
             if (!rows0) release_buffer(empty_bar, lane);
           } else {
             const int vh = min(64, valid - (int)col0);
