@@ -294,8 +294,10 @@ __device__ __forceinline__ Warp1 make_warp1(uint32_t tmem_base) {
 
 // Pass 1 again for a warp whose sums overflowed: the largest logit of every row becomes its
 // reference. Rare (a key more than 69 nats above the first one), so eight rows at a time; writes the
-// warp's pairs.
-template <bool kShift>
+// warp's pairs. A row whose logits hold NaN or +inf ends here too, with a sum that is NaN, as its scores are to be.
+// With one sum over the rows, pass 2 takes rows 2 and 3 of every four on the FMA pipe, whose exponential
+// makes 2^-126 of a NaN, so rows 0 and 1 of those four, which the MUFU takes, pass it on.
+template <bool kPerHead, bool kShift>
 __device__ __noinline__ void redo_sums(const ClArgs& a, Ctl* ctl, int u, int rank, uint32_t tile0, int buf) {
   const Warp1 w = make_warp1(ctl->tmem_base);
   const Unit x = unit_at<kShift>(a, u, rank);
@@ -329,6 +331,13 @@ __device__ __noinline__ void redo_sums(const ClArgs& a, Ctl* ctl, int u, int ran
         }
     }
     sum_lanes(s);
+    if (!kPerHead) {
+      const float s2 = __shfl_xor_sync(0xffffffffu, s[0], 1), s3 = __shfl_xor_sync(0xffffffffu, s[1], 1);
+      if ((w.lane & 1) == 0) {
+        s[0] += 0.f * s2;
+        s[1] += 0.f * s3;
+      }
+    }
     if (w.lane < 4) {
       ctl->part[buf][w.index][8 * g + 2 * w.lane] = make_float2(m[0], s[0]);
       ctl->part[buf][w.index][8 * g + 2 * w.lane + 1] = make_float2(m[1], s[1]);
@@ -338,7 +347,7 @@ __device__ __noinline__ void redo_sums(const ClArgs& a, Ctl* ctl, int u, int ran
 
 // Pass 1 over this warp's tiles of a unit; tile0 is the CTA's running number of the unit's first
 // tile, n the running number of the unit.
-template <int kGroups, bool kShift>
+template <int kGroups, bool kPerHead, bool kShift>
 __device__ __forceinline__ bool pass1(const ClArgs& a, Ctl* ctl, const Warp1& w, const Unit& x, int rank,
                                       uint32_t tile0, int n) {
   const float c = a.scale_log2;
@@ -392,7 +401,7 @@ __device__ __forceinline__ bool pass1(const ClArgs& a, Ctl* ctl, const Warp1& w,
     *reinterpret_cast<float4*>(&ctl->part[buf][w.index][row]) =
         make_float4(-nref[0].x, acc[0].x, -nref[0].y, acc[0].y);
   __syncwarp();
-  if (__any_sync(0xffffffffu, high)) redo_sums<kShift>(a, ctl, x.u, rank, tile0, buf);
+  if (__any_sync(0xffffffffu, high)) redo_sums<kPerHead, kShift>(a, ctl, x.u, rank, tile0, buf);
   tc_fence_before();
   __syncwarp();
   if (w.lane == 0) mbar_arrive(smem_u32(&ctl->stat_full[buf]));
@@ -779,7 +788,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
     int n = 0;
     for (int u = u_first; u < a.U; u += n_clusters, ++n) {
       const Unit x = unit_at<kShift>(a, u, rank);
-      if (!pass1<kGroups, kShift>(a, ctl, w, x, rank, tile0, n)) break;
+      if (!pass1<kGroups, kPerHead, kShift>(a, ctl, w, x, rank, tile0, n)) break;
       tile0 += (uint32_t)x.tiles;
     }
   } else {

@@ -11,7 +11,7 @@ import pytest
 import torch
 
 from parity_util import SCORE_RTOL
-from test_gpu_parity import compare_all_units, laq, rand_inputs  # noqa: F401 (laq is a fixture)
+from test_gpu_parity import compare_all_units, laq, rand_inputs, run_evict  # noqa: F401 (laq is a fixture)
 from test_timeout_path import hooked_library
 
 pytestmark = pytest.mark.gpu
@@ -112,6 +112,32 @@ def test_cluster_scoring_per_head_with_several_tiles(laq, L, C, W, G):
     for mode in (1, 2):
         assert launched_cluster(laq, q, k, W, 7, 80, mode) == C
         compare_all_units(laq, q, k, v, W, 7, 80, group_mode=mode)
+
+
+@pytest.mark.parametrize("G,W,group", [(1, 5, 0), (4, 2, 0), (4, 16, 0), (7, 8, 0), (4, 8, 1), (4, 3, 2)])
+@pytest.mark.parametrize("what", [float("inf"), float("nan")])
+def test_row_without_a_softmax_is_not_left_out_of_a_cluster(laq, G, W, group, what):
+    # every logit of one row of KV head 0 is +inf or NaN: its attention weights, and with them every score
+    # that adds or compares them, are NaN (as in the fp64 definition); the other KV head is not touched. Pass 2
+    # takes rows 2 and 3 of every four on another pipe than rows 0 and 1.
+    q, k, v = rand_inputs(1, 1, 2 * G, 2, 128, 1000, W, seed=W + G)
+    q[..., 0] = 0.0
+    k[..., 0] = 1.0
+    H = G if group == 2 else 1
+    good = run_evict(laq, q, k, v, W, 1, W + 20, group_mode=group)["scores"]
+    for row in sorted({0, 1, 2, 3, G * W - 2, G * W - 1} & set(range(G * W))):
+        bad = q.clone()
+        bad[0, 0, row // W, row % W, 0] = what
+        got = run_evict(laq, bad, k, v, W, 1, W + 20, group_mode=group)["scores"]
+        nan = got[0, 0].isnan()
+        if group == 1:                       # (the larger of a NaN and a number is the number)
+            assert torch.equal(got[0, 0, 1], good[0, 0, 1])
+        elif group == 2:
+            assert nan[row // W].all()
+            others = [h for h in range(2 * G) if h != row // W]
+            assert torch.equal(got[0, 0, others], good[0, 0, others])
+        else:
+            assert nan[0].all() and torch.equal(got[0, 0, H:], good[0, 0, H:])
 
 
 @pytest.mark.parametrize("W,L,lens", [(1, 128, None), (2, 700, None), (4, 500, tuple([500, 131] * 16))])
