@@ -59,7 +59,7 @@ constexpr int kThreads = 32 * (kMmaWarpB + kStatInWarps);
 // 0.5-1 % faster than 4 and 2; deeper rings do not fit the shared memory next to the K stages)
 constexpr int kTaskSlots = 6;
 constexpr int kMaxSlots = 4;  // TMEM accumulators of 128 columns
-constexpr int kKStages = 4;   // K stages in shared memory
+constexpr int kMaxKStages = 4;  // K stages in shared memory
 constexpr int kStatSlots = 3;
 constexpr uint32_t kKStageBytes = TILE_KEYS * 128 * 2;  // 128 keys x 128 dims x bf16
 constexpr uint32_t kCtlBytes = 34816;
@@ -113,11 +113,11 @@ struct Task {
 // Control block at the start of dynamic shared memory.
 struct Ctl {
   uint64_t q_full[2], q_empty[2];
-  uint64_t k_full[kKStages];
-  // Tile t uses K stage t mod 4 and accumulator buffer t mod n_slots. Up to 128 rows n_slots is 4 too, and
-  // one barrier per slot tells the producer that the stage is free and the softmax warps that the logits
-  // are ready. With more, n_slots is 2, a buffer consists of two row blocks with barriers of their own, and
-  // the stages have theirs.
+  uint64_t k_full[kMaxKStages];
+  // Tile t uses K stage t mod n_stages and accumulator buffer t mod n_slots. Both are 4 up to 128 rows and 2
+  // with more, and one barrier per slot tells the producer that the stage is free and the softmax warps that
+  // the logits are ready. Where row blocks change hands on their own they have barriers of their own, and
+  // there are 4 stages with theirs.
   // n_slots is even: tiles t and t - n_slots then belong to the same MMA issuer and the same
   // softmax pair, which is what makes the parity waits sound (a waiter is never two phases ahead).
   // With five slots the second issuer can complete tile t - 2 before the first has issued tile
@@ -142,7 +142,7 @@ struct Ctl {
   // per-prompt lengths: task_prefix[b] = sweep-1 tasks of one layer that belong to prompts < b
   // (written and read by the producer lane only)
   int task_prefix[LAQ_MAX_RAGGED_BATCH + 1];
-  uint64_t k_empty[kKStages];  // (more than 128 rows)
+  uint64_t k_empty[kMaxKStages];  // (row blocks on their own)
 };
 static_assert(sizeof(Ctl) <= kCtlBytes, "control block too large");
 
@@ -300,45 +300,48 @@ __device__ __noinline__ float2 stats_cols_ragged(uint32_t taddr, int valid_max, 
 // MMA warp as soon as the last chunk is in registers.
 template <int kPoly, bool kPrecise>
 __device__ __forceinline__ void stats_cols64(uint32_t taddr, float c, float& m, float& l, float* v,
-                                             uint32_t empty_bar, int lane) {
+                                             uint32_t empty_bar, int lane, bool release = true) {
   tmem_ld32(taddr, v);
   tmem_ld_wait(v);
   stats_chunk<kPoly, kPrecise>(v, c, m, l);
   tmem_ld32(taddr + 32u, v);
   tmem_ld_wait(v);
-  release_buffer(empty_bar, lane);
+  if (release) release_buffer(empty_bar, lane);
   stats_chunk<kPoly, kPrecise>(v, c, m, l);
 }
 
 // ------------------------------------------------------------------ the kernel
 // kDup: M <= 64, sweep 1 holds every query row twice (on TMEM lanes r and 64 + r).
 // kWide: 128 < M <= 256, two row blocks per tile, so an accumulator buffer takes 256 TMEM columns and there
-// are two of them instead of four. A block's 128 columns change hands on their own, in both sweeps: the MMAs
-// of a pair's next tile run while it is at the second block of this one. A K stage is then wanted half a tile
-// earlier, so there are four, and one Q stage (the next task's Q arrives while two tiles of this one are still
-// to be exponentiated). 256 rows, us, all handed over whole, blocks alone, and with the stages: 65536 keys, 640
-// units 7589 / 7214 / 7136; 16384 keys, 160 units 479 / 467 / 458; 5000 keys 166 / 161 / 157.
+// are two of them instead of four.
+// kSplit: a block's 128 columns change hands on their own, in both sweeps: the MMAs of a pair's next tile run
+// while it is at the second block of this one. A K stage is then wanted half a tile earlier, so there are four,
+// and one Q stage. 256 rows, us, all handed over whole, blocks alone, and with the stages: 65536 keys, 640
+// units 7589 / 7214 / 7136; 16384 keys, 160 units 479 / 467 / 458; 5000 keys 166 / 161 / 157. But the next
+// task's Q then comes late, which short tasks show; two stages of Q and of K, and tiles handed over whole, are
+// for them (split_blocks; three K stages beside two smaller ones of Q took 5 to 10 % longer).
 // kPerHead: sweep 2 keeps one column sum per query head (colsum is [U*G][L_pad]); the launcher
 // only picks it when a head's rows never straddle a group of four rows or a 32-row chunk unevenly
 // (W a multiple of 4 that divides 32, or 32 or 64).
 // kPolyS1: of every 8 pairs of sweep 1, how many take an exponential on the FMA pipe.
-//   M > 128, one sum: 1, as precise as the MUFU's (scores 1.2e-7 from fp64 in the 2-norm either way). The MUFU
+//   M > 128, one sum, kSplit: 1, as precise as the MUFU's (scores 1.2e-7 from fp64 in the 2-norm either way). The MUFU
 //     alone takes 2048 of a tile's 2570 cycles a sweep: 65536 keys, 640 units 7136 -> 6894 us, 5000 keys, 160
 //     units 161 -> 156, 64 dims 419 -> 404 (2 of 8: 7031, 153, 403).
-//   M > 128, a sum per head: 0 (1 of 8: 160 rows, 6000 keys 147 -> 150, 256 rows, 9001 keys 131 -> 130).
+//   M > 128, whole: 0 (1 of 8 -1 to +1 %). A sum per head: 0 (1 of 8: 160 rows, 6000 keys 147 -> 150, 256 rows, 9001 keys 131 -> 130).
 //   64 < M <= 128, 128 dims: LAQ_POLY_PAIRS_S1 of a cheaper one, 7.5e-5 off, which leaves the scores within
 //     1e-6 (on the MUFU alone 2e-7). Other head dims: 0, so that their scores are as precise as on the CUDA
 //     cores, where they used to be formed (64 dims, 128 rows, 128 units of 32768 keys 324 us, with it 310).
 //   M <= 64: 0, it pays nothing.
-template <bool kDup, bool kWide, bool kPerHead, int kPolyS1>
+template <bool kDup, bool kWide, bool kPerHead, int kPolyS1, bool kSplit = kWide>
 __global__ void __launch_bounds__(kThreads, 1)
 score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
                 const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ TcArgs a) {
   constexpr uint32_t kQRows = kWide ? 256u : 128u;   // rows per 64-dim half of a Q stage
   constexpr uint32_t kSlotShift = kWide ? 1u : 2u;   // log2 of the accumulator buffers
-  constexpr uint32_t kQStages = kWide ? 1u : 2u;
+  constexpr uint32_t kQStages = kSplit ? 1u : 2u, kKStages = kWide && !kSplit ? 2u : 4u;
   constexpr uint32_t kTbCols = kWide ? 256u : 128u;  // TMEM columns per accumulator buffer
-  constexpr int RB = kWide ? 2 : 1;                  // 128-row blocks per tile, each with barriers of its own
+  constexpr int RB = kWide ? 2 : 1;                  // 128-row blocks per tile
+  constexpr int kHand = kSplit ? 2 : 1;              // parts in which an accumulator buffer changes hands
   long long clk0 = 0;
   unsigned long long ns0 = 0;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -367,7 +370,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
       mbar_init(smem_u32(&ctl->q_full[i]), 1);
       mbar_init(smem_u32(&ctl->q_empty[i]), 2);  // both MMA issuers
     }
-    for (int i = 0; i < kKStages; ++i) {
+    for (int i = 0; i < kMaxKStages; ++i) {
       mbar_init(smem_u32(&ctl->k_full[i]), 1);
       mbar_init(smem_u32(&ctl->k_empty[i]), 1);
     }
@@ -462,7 +465,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
         for (int i = 0; i < task.n_tiles; ++i) {
           const uint32_t s = kcount % kKStages;
           // the stage is free once the MMAs of the tile that used it last have completed
-          if (!mbar_wait(a, ctl, smem_u32(kWide ? &ctl->k_empty[s] : &ctl->mma_done[s]),
+          if (!mbar_wait(a, ctl, smem_u32(kSplit ? &ctl->k_empty[s] : &ctl->mma_done[s]),
                          ((kcount / kKStages) & 1u) ^ 1u, 4)) {
             ok = false;
             break;
@@ -501,8 +504,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
       const uint32_t issuer = warp == 1 ? 0u : 1u;
       uint32_t tc_base = 0, my_next = issuer, qc = 0, tk = 0;
       const uint32_t idesc_s1 = instr_desc(128, TILE_KEYS);
-      const uint32_t idesc_s2 = instr_desc(128, kWide ? 128 : a.M_pad);
-      const uint32_t idesc_s2b = instr_desc(128, kWide ? a.M_pad - 128 : 128);  // the second row block
+      const uint32_t idesc_s2 = instr_desc(128, kSplit ? 128 : a.M_pad);
+      const uint32_t idesc_s2b = instr_desc(128, kSplit ? a.M_pad - 128 : 128);  // the second row block
       const uint32_t q_half16 = kQRows * 8u;  // (q_rows * 128 bytes) >> 4
       const uint32_t k_lo0 = smem_desc_lo(k_base), q_lo0 = smem_desc_lo(q_base);
       bool ok = true;
@@ -518,7 +521,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
           const uint32_t tc = tc_base + (uint32_t)i;
           const uint32_t s = tc & slot_mask;
           const uint32_t ph = (tc >> kSlotShift) & 1u;
-          if constexpr (!kWide) {
+          if constexpr (!kSplit) {
             if (!mbar_wait(a, ctl, smem_u32(&ctl->k_full[s]), ph, 12) ||
                 !mbar_wait(a, ctl, smem_u32(&ctl->tmem_empty[s]), ph ^ 1u, 13)) {
               ok = false;
@@ -529,10 +532,12 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
             const uint32_t d_tmem = tmem_base + s * kTbCols;
             // k-step kk covers dims [16 kk, 16 kk + 16): 32 bytes inside the 64-dim half (kk >> 2)
             if (task.sweep == 0) {
+              for (int rb = 0; rb < RB; ++rb)
 #pragma unroll
-              for (int kk = 0; kk < 8; ++kk)
-                if (kk < a.ksteps) umma_bf16(d_tmem, q_lo + (kk >> 2) * q_half16 + (kk & 3) * 2u,
-                          k_lo + (kk >> 2) * (kKStageBytes >> 5) + (kk & 3) * 2u, kSmemDescHi, idesc_s1, kk > 0);
+                for (int kk = 0; kk < 8; ++kk)
+                  if (kk < a.ksteps) umma_bf16(d_tmem + (uint32_t)rb * 128u,
+                            q_lo + (kk >> 2) * q_half16 + (uint32_t)rb * 1024u + (kk & 3) * 2u,
+                            k_lo + (kk >> 2) * (kKStageBytes >> 5) + (kk & 3) * 2u, kSmemDescHi, idesc_s1, kk > 0);
             } else {
 #pragma unroll
               for (int kk = 0; kk < 8; ++kk)
@@ -548,8 +553,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
             }
             const uint32_t k_lo = k_lo0 + ks * (kKStageBytes >> 4);
 #pragma unroll
-            for (int rb = 0; rb < RB; ++rb) {
-              if (!mbar_wait(a, ctl, smem_u32(&ctl->tmem_empty[s * RB + rb]), ph ^ 1u, 13)) {
+            for (int rb = 0; rb < kHand; ++rb) {
+              if (!mbar_wait(a, ctl, smem_u32(&ctl->tmem_empty[s * kHand + rb]), ph ^ 1u, 13)) {
                 ok = false;
                 break;
               }
@@ -569,7 +574,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
                   if (kk < a.ksteps) umma_bf16(d_tmem, k_lo + (kk >> 2) * (kKStageBytes >> 5) + (kk & 3) * 2u,
                             q_rb + (kk >> 2) * q_half16 + (kk & 3) * 2u, kSmemDescHi, idesc, kk > 0);
               }
-              umma_commit(smem_u32(&ctl->mma_done[s * RB + rb]));
+              umma_commit(smem_u32(&ctl->mma_done[s * kHand + rb]));
             }
             if (!ok) break;
             umma_commit(smem_u32(&ctl->k_empty[ks]));
@@ -707,8 +712,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
     const int row_in_wg = quad * 32 + lane;  // TMEM lane this thread reads
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
     const float c = a.scale_log2;
-    // sweep 2: this warpgroup's share of the row blocks' M_pad / 32 chunks of rows
-    const int n_chunks2 = a.M_pad / 32, n_first = min(4, n_chunks2), n_second = n_chunks2 - n_first;
+    // sweep 2: this warpgroup's share of the M_pad / 32 chunks of rows, or of each block's
+    const int n_chunks2 = a.M_pad / 32, n_first = kSplit ? 4 : n_chunks2, n_second = n_chunks2 - n_first;
     const int ch_lo0 = half == 0 ? 0 : (n_first + 1) / 2, ch_hi0 = half == 0 ? (n_first + 1) / 2 : n_first;
     const int ch_lo1 = 4 + (half == 0 ? 0 : (n_second + 1) / 2), ch_hi1 = 4 + (half == 0 ? (n_second + 1) / 2 : n_second);
     const uint32_t col0 = 64u * (uint32_t)half;  // sweep 1: this warpgroup's 64 key columns
@@ -748,7 +753,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
         const uint32_t tc = tc_base + (uint32_t)i;
         const uint32_t s = tc & slot_mask;
         const uint32_t ph = (tc >> kSlotShift) & 1u;
-        if (!mbar_wait(a, ctl, smem_u32(&ctl->mma_done[s * RB]), ph, 21)) {
+        if (!mbar_wait(a, ctl, smem_u32(&ctl->mma_done[s * kHand]), ph, 21)) {
           ok = false;
           break;
         }
@@ -756,10 +761,10 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
         tc_fence_after();
         const int key0 = (task.tile0 + i) * TILE_KEYS;
         const uint32_t taddr = lane_addr + s * kTbCols;
-        const uint32_t empty_bar = smem_u32(&ctl->tmem_empty[s * RB]), empty_bar1 = empty_bar + 8u;
+        const uint32_t empty_bar = smem_u32(&ctl->tmem_empty[s * kHand]), empty_bar1 = empty_bar + 8u;
         // the second row block's logits
         auto second_block = [&]() -> bool {
-          if (!mbar_wait(a, ctl, smem_u32(&ctl->mma_done[s * RB + 1]), ph, 24)) return false;
+          if (!mbar_wait(a, ctl, smem_u32(&ctl->mma_done[s * kHand + 1]), ph, 24)) return false;
           __syncwarp();
           tc_fence_after();
           return true;
@@ -786,7 +791,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
               l0 = r.y;
               release_buffer(empty_bar, lane);
             }
-          } else if (kWide) {
+          } else if (kSplit) {
             // (every column is a real key that every row sees, but for the last tiles of a unit)
             const bool whole = valid == TILE_KEYS && key0 + TILE_KEYS <= Lu - a.W_local;
             const int vh = min(64, valid - (int)col0);
@@ -815,7 +820,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
             if (!rows1 || !whole) release_buffer(empty_bar1, lane);
           } else if (valid == TILE_KEYS && key0 + TILE_KEYS <= Lu - a.W_local) {
             // every column is a real key that every row sees
-            if (rows0) stats_cols64<kPolyS1, kWide>(taddr + col0, c, m0, l0, v, empty_bar, lane);
+            if (rows0) stats_cols64<kPolyS1, kWide>(taddr + col0, c, m0, l0, v, empty_bar, lane, !rows1);
+            if (rows1) stats_cols64<kPolyS1, kWide>(taddr + 128u + col0, c, m1, l1, v, empty_bar, lane);
             if (!rows0) release_buffer(empty_bar, lane);
           } else {
             const int vh = min(64, valid - (int)col0);
@@ -823,6 +829,11 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
               const float2 r = stats_cols_ragged(taddr + col0, vh, min(vh, vis0 - key0 - (int)col0), c, m0, l0);
               m0 = r.x;
               l0 = r.y;
+            }
+            if (rows1) {
+              const float2 r = stats_cols_ragged(taddr + 128u + col0, vh, min(vh, vis1 - key0 - (int)col0), c, m1, l1);
+              m1 = r.x;
+              l1 = r.y;
             }
             release_buffer(empty_bar, lane);
           }
@@ -835,7 +846,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
           const int gph = (a.W < 32 ? a.W : 32) >> 2, w_log2 = 31 - __clz(a.W);
           const int key = key0 + row_in_wg;
 #pragma unroll 1
-          for (int rb = 0; rb < RB; ++rb) {
+          for (int rb = 0; rb < kHand; ++rb) {
             if (rb == 1 && !second_block()) {
               ok = false;
               break;
@@ -868,7 +879,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
 #pragma unroll
           for (int k = 0; k < 4; ++k) acc[k] = make_float2(0.f, 0.f);
 #pragma unroll 1
-          for (int rb = 0; rb < RB; ++rb) {
+          for (int rb = 0; rb < kHand; ++rb) {
             if (rb == 1 && !second_block()) {
               ok = false;
               break;
@@ -1000,6 +1011,27 @@ extern "C" __attribute__((visibility("default"))) void laq_test_withhold_launche
 #endif
 
 namespace laq {
+namespace {
+// Whether the row blocks of more than 128 rows change hands on their own. Where an SM has few tasks to take that
+// wins 2 to 12 %, and so do tasks of 8 tiles and more always (2 to 11 %). Where it has many and they are short,
+// tiles handed over whole do, whose Q is there in time (medians over 3492 shapes of one to 160 tiles; whole over
+// split, up to 192 rows / more): from 2.5 tasks on an SM, both sweeps counted, 1 tile 0.95-1.00 / 0.90-0.98,
+// 2 0.95-0.97 / 0.96-1.00, 3 0.93-0.98 / 0.93-1.01, 5 0.89-1.00 / 0.95-1.06; from 8 on also 4 0.93-0.95 /
+// 0.96, 6 0.97-0.98 / 1.00, 7 0.95-0.97 / 0.98-1.00 (4 to 8: 4 1.00, 6 1.01, 7 1.00). Prompts of different
+// lengths (1096 batches) go by the mean: up to 6.5 tiles a task 0.92-0.97, 6.5 to 7 0.99, more 1.03 / up to 4.5
+// 0.91-0.97, more 1.00-1.05. With one sum per head split wins or is equal.
+bool split_blocks(const Dims& d, const TcArgs& a, int64_t tasks, int sms) {
+  if (d.group_mode != LAQ_GROUP_SUM) return true;
+  const double per_sm = 2.0 * (double)tasks / sms;
+  if (per_sm < 2.5) return true;
+  const int t = a.tiles_per_task;
+  if (d.sl.n == 0) return !(t <= 3 || (d.M <= 192 && t == 5) || (per_sm >= 8.0 && t <= (d.M <= 192 ? 7 : 5)));
+  int64_t tiles = 0;
+  for (int b = 0; b < d.Bt; ++b) tiles += (d.sl.len[b] + TILE_KEYS - 1) / TILE_KEYS;
+  return (double)(tiles * d.Hkv * d.NL) >= (d.M <= 192 ? 7.0 : 5.0) * (double)tasks;
+}
+}  // namespace
+
 laq_status score_tc_launch(const laq_params& p, const Dims& d, const Workspace& w, const void* q,
                            const void* k, char* ws, cudaStream_t stream, int* launches) {
   TcArgs a;
@@ -1077,20 +1109,23 @@ laq_status score_tc_launch(const laq_params& p, const Dims& d, const Workspace& 
   if (!make_tensor_map(&tmap_q, q, qdims, qstr, qbox) || !make_tensor_map(&tmap_k, k, kdims, kstr, kbox))
     return score_simt_launch(p, d, w, q, k, ws, stream, launches);  // layout TMA cannot describe
 
-  const size_t smem = kCtlBytes + 65536u + (size_t)kKStages * kKStageBytes;  // one Q stage of 256 rows or two of 128
+  // one Q stage of 256 rows or two of 128 beside four K stages, or two of 256 beside two
+  const size_t smem = kCtlBytes + 65536u + (size_t)kMaxKStages * kKStageBytes;
   const bool per_head = d.group_mode != LAQ_GROUP_SUM;
   typedef void (*Kernel)(const CUtensorMap, const CUtensorMap, const TcArgs);
-  // [per head][dup, wide, neither, neither with other head dims]
-  static const Kernel kernels[2][4] = {
+  // [per head][dup, wide, neither, neither with other head dims, wide and whole]
+  static const Kernel kernels[2][5] = {
       {score_tc_kernel<true, false, false, 0>, score_tc_kernel<false, true, false, 1>,
-       score_tc_kernel<false, false, false, LAQ_POLY_PAIRS_S1>, score_tc_kernel<false, false, false, 0>},
+       score_tc_kernel<false, false, false, LAQ_POLY_PAIRS_S1>, score_tc_kernel<false, false, false, 0>,
+       score_tc_kernel<false, true, false, 0, false>},
       {score_tc_kernel<true, false, true, 0>, score_tc_kernel<false, true, true, 0>,
-       score_tc_kernel<false, false, true, LAQ_POLY_PAIRS_S1>, score_tc_kernel<false, false, true, 0>}};
-  const int variant = dup ? 0 : (wide ? 1 : (d.D == 128 ? 2 : 3));
+       score_tc_kernel<false, false, true, LAQ_POLY_PAIRS_S1>, score_tc_kernel<false, false, true, 0>,
+       score_tc_kernel<false, true, true, 0>}};
+  const int variant = dup ? 0 : (wide ? (split_blocks(d, a, n_stream, sms) ? 1 : 4) : (d.D == 128 ? 2 : 3));
   const Kernel kernel = kernels[per_head][variant];
   // the shared-memory opt-in is a per-device attribute of each kernel variant: set once
   static std::atomic<uint32_t> smem_opted_in[kMaxDevices];
-  const uint32_t variant_bit = 1u << (variant + (per_head ? 4 : 0));
+  const uint32_t variant_bit = 1u << (variant + (per_head ? 5 : 0));
   if (dev >= kMaxDevices || !(smem_opted_in[dev].load(std::memory_order_acquire) & variant_bit)) {
     if (!cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
       return LAQ_ERR_CUDA;

@@ -176,3 +176,36 @@ def test_wait_that_runs_out_in_clusters(G, W, L, C, group):
         hooked.laq_test_withhold_unit(-1)
     assert run() == laq.LAQ_OK
     assert torch.equal(scores, want)
+
+
+def test_wait_that_runs_out_where_tiles_are_handed_over_whole():
+    # 200 units of 160 rows and five tiles: more than two tasks an SM, short ones
+    from paper_2505_20334_b200 import binding as laq
+
+    hooked = hooked_library()
+    Bt, G, Hkv, W, D, L = 100, 5, 2, 32, 128, 600
+    g = torch.Generator(device="cuda").manual_seed(7)
+    q = torch.randn((1, Bt, G * Hkv, W, D), generator=g, device="cuda", dtype=torch.bfloat16)
+    k = torch.randn((1, Bt, Hkv, L, D), generator=g, device="cuda", dtype=torch.bfloat16)
+    p = laq.params_for(q, k, W, 7, 100)
+    ws = laq.alloc_workspace(p, "cuda")
+    scores = torch.zeros((1, Bt, Hkv, L - W), device="cuda")
+    stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+
+    def run(lib):
+        scores.zero_()
+        assert lib.laq_score(ctypes.byref(p), q.data_ptr(), k.data_ptr(), scores.data_ptr(), ws.data_ptr(), ws.numel(),
+                             stream) == laq.LAQ_OK
+        return lib.laq_last_device_status(ctypes.byref(p), ws.data_ptr(), ws.numel(), stream)
+
+    assert run(hooked) == laq.LAQ_OK
+    want = scores.clone()
+    for unit in (0, 1, 150, 199):
+        hooked.laq_test_withhold_unit(unit)
+        try:
+            assert run(hooked) == laq.LAQ_ERR_TIMEOUT
+        finally:
+            hooked.laq_test_withhold_unit(-1)
+    for lib in (hooked, laq.lib):
+        assert run(lib) == laq.LAQ_OK
+        assert float((scores - want).norm() / want.norm()) < 5e-7     # (tasks of an odd number of tiles)

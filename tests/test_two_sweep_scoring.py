@@ -106,12 +106,12 @@ def evict_with(laq, q, k, v, R, kernel, B, tiles_per_task=0, local_window=0, len
     return dict(out, params=p, ws=ws)
 
 
-def scoring_kernels(call):
+def scoring_kernels(call, *more):
     with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
         call()
         torch.cuda.synchronize()
     names = " ".join(e.key for e in prof.key_averages())
-    return {n for n in ("score_cluster_kernel", "score_tc_kernel", "simt_stats_kernel") if n in names}
+    return {n for n in ("score_cluster_kernel", "score_tc_kernel", "simt_stats_kernel", *more) if n in names}
 
 
 TWO_SWEEP = [
@@ -203,15 +203,34 @@ MANY_TASKS = [
     (32, 5, 2300, 32, 0, 0, False, 0),            # 160 rows, 64 units
     (32, 8, 3000, 32, 16, 0, False, 0),           # 256 rows, local queries
     (40, 8, 1500, 32, 0, 1, True, 0),             # 256 rows, a task per tile, prompts of different lengths
-    (32, 6, 5000, 32, 5, 3, True, 0),             # 192 rows, tasks of three tiles
-    (24, 8, 4100, 17, 17, 5, False, 0),           # 136 rows, odd numbers of tiles a task
+    (32, 6, 4900, 32, 5, 13, True, 0),            # 192 rows, tasks of thirteen tiles, prompts of different lengths
+    (32, 8, 4100, 32, 17, 5, False, 0),           # 256 rows, odd numbers of tiles a task
+    (32, 8, 3500, 17, 17, 7, False, 0),           # 136 rows, likewise
     (32, 5, 2000, 32, 0, 0, True, 2),             # one column sum per head
     (32, 8, 1700, 32, 8, 3, False, 1),
 ]
+# Many tasks of few tiles: these are handed over whole, both row blocks at once
+SHORT_TASKS = [
+    (100, 3, 300, 43, 0, 0, False, 0),            # 129 rows, three tiles a unit
+    (100, 5, 600, 32, 16, 0, False, 0),           # 160 rows, five tiles, local queries
+    (100, 8, 200, 32, 0, 0, False, 0),            # 256 rows, two tiles
+    (160, 6, 2600, 32, 0, 0, False, 0),           # 192 rows, three tasks of seven tiles
+    (100, 8, 900, 17, 17, 1, False, 0),           # 136 rows, a task per tile, all queries local
+    (100, 5, 1500, 32, 5, 0, True, 0),            # 160 rows, prompts of different lengths
+]
+
+
+@pytest.mark.parametrize("case", SHORT_TASKS, ids=[f"M{c[1] * c[3]}-L{c[2]}-t{c[5]}" for c in SHORT_TASKS])
+def test_two_row_blocks_handed_over_whole(laq, case):  # noqa: F811
+    check_many_tasks(laq, case, whole=True)
 
 
 @pytest.mark.parametrize("case", MANY_TASKS, ids=[f"M{c[1] * c[3]}-L{c[2]}-t{c[5]}-g{c[7]}" for c in MANY_TASKS])
 def test_two_row_blocks_through_many_tasks(laq, case):  # noqa: F811
+    check_many_tasks(laq, case, whole=case == MANY_TASKS[2])
+
+
+def check_many_tasks(laq, case, whole):  # noqa: F811
     # Against the CUDA-core kernel, which a layer stride that no tensor map holds selects (with one layer it is
     # never used): fp32 sums of the same terms in other orders, 2^-21 in the 2-norm apiece.
     Bt, G, L, W, Wl, tiles, ragged, group = case
@@ -231,7 +250,8 @@ def test_two_row_blocks_through_many_tasks(laq, case):  # noqa: F811
 
     def call():
         laq.laq_score(p, q, k, got, ws)
-    assert scoring_kernels(call) == {"score_tc_kernel"}
+    assert scoring_kernels(call, "score_tc_kernel<false, true, false, 0, false>") == (
+        {"score_tc_kernel", "score_tc_kernel<false, true, false, 0, false>"} if whole else {"score_tc_kernel"})
     for _ in range(3):
         call()
         assert laq.laq_last_device_status(p, ws) == laq.LAQ_OK
