@@ -917,24 +917,24 @@ int cluster_size(const Dims& d, int n_tiles, int slots, const ClusterCounts& cou
   // for the next unit's; the arithmetic, likewise; the chain from the first MMA of a unit through the exchange
   // to the end of pass 2, of which two can be under way (what short units are bound by: without it 512
   // units of 582 keys and 16 rows took 31.7 us in clusters of 5, 20.1 alone); and, with one sum per head,
-  // pass 2 of the busier of the two warpgroups, row by row where heads are no groups of four rows. The last unit's pass 2 ends the call. Fitted to the times of
-  // all sizes on 4500 shapes of up to 65536 keys, K from HBM: the size taken is 1.7 % above the best one on
-  // average, the powers of two alone 4.4 %. On 3700 other shapes it is 2.0 % faster than those on average;
-  // 57 are more than 1.5 % slower, 24 more than 3 %, two 15 %. To rank the powers of two by the same costs
-  // gains another 0.3 %, but makes 129 of the 4500 shapes slower than they were.
+  // pass 2 of the busier of the two warpgroups. The last unit's pass 2 ends the call. Fitted to the times of
+  // all sizes on 9500 shapes of up to 65536 keys, K from HBM in 4500 of them and from L2 in the others: 2 %
+  // faster than the powers of two alone on average, 48 shapes more than 1.5 % slower, the worst 7 %. With K from
+  // HBM the size taken is 2.1 % above the best one on average, powers of two 4.4 %. To rank those by the same
+  // costs gains another 0.3 %, but makes some 3 % of the shapes slower than they were.
   // Not for prompts of different lengths, which leave CTAs of a cluster without tiles in ways that this does
   // not foresee (3 prompts of 1319 to 6597 keys: 4 % slower).
   const auto cycles = [&](int C) {
     const int n = counts.resident[C], T = (n_tiles + C - 1) / C;
     const double rounds = (double)((d.U + n - 1) / n), full = (double)T / slots;
     const double sms = (double)d.U / rounds * C;  // of an average round
-    const double stream = T * (d.D / 64.0) * fmax(426.0, kBoxBytes * sms / 3860.0) + fmax(0.0, 2800.0 * (full - 0.52));
-    const double math = T * (720.0 + 8.0 * d.M) + fmax(0.0, 2600.0 * (full - 0.516));
-    const double chain = 1900.0 + 39.0 * d.M + 33.0 * C;
-    const double heads = d.group_mode == LAQ_GROUP_SUM ? 0.0 : (T + 1) / 2 * (1200.0 + (d.W % 4 ? 30.0 : 5.5) * d.M);
-    return rounds * fmax(fmax(stream, math), fmax(chain, heads)) + T * (233.0 + 0.84 * d.M);
+    const double stream = T * (d.D / 64.0) * fmax(477.0, kBoxBytes * sms / 3853.0) + fmax(0.0, 3400.0 * (full - 0.602));
+    const double math = T * (751.0 + 6.4 * d.M) + fmax(0.0, 2185.0 * (full - 0.505));
+    const double chain = 2467.0 + 30.0 * d.M + 7.2 * C;
+    const double heads = d.group_mode == LAQ_GROUP_SUM ? 0.0 : (T + 1) / 2 * (682.0 + 18.8 * d.M);
+    return rounds * fmax(fmax(stream, math), fmax(chain, heads)) + T * (122.0 + 0.7 * d.M);
   };
-  best_cost = 0.97 * cycles(best);
+  best_cost = 0.967 * cycles(best);
   for (int C = 3; C < kMaxCluster; ++C) {
     if ((C & (C - 1)) == 0 || counts.resident[C] < 1 || (n_tiles + C - 1) / C > slots || C > n_tiles) continue;
     const double cost = cycles(C);

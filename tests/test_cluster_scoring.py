@@ -84,17 +84,17 @@ def launched_cluster(laq, q, k, R, kernel, B, group=0):  # noqa: F811
     return hooked.laq_test_last_cluster()
 
 
-# clusters whose CTAs hold several tiles of a unit: nine with two tiles, sixteen with three and four
-SIZES = [(2304, 9), (8192, 16)]
+# clusters whose CTAs hold several tiles of a unit (layers, batch, keys, size): six with three tiles, sixteen with four
+SIZES = [(4, 2, 2000, 6), (1, 1, 8192, 16)]
 
 
-@pytest.mark.parametrize("L,C", SIZES)
+@pytest.mark.parametrize("NL,Bt,L,C", SIZES)
 @pytest.mark.parametrize("G,W,group", [(4, 4, 0), (4, 16, 0), (3, 19, 0), (8, 8, 2), (4, 3, 2)])
-def test_sums_that_overflow_in_clusters_of(laq, L, C, G, W, group):
+def test_sums_that_overflow_in_clusters_of(laq, NL, Bt, L, C, G, W, group):
     # as above, every warp with more than one tile: its reference lies 120 nats below the largest key, in
     # some warps in their first tile and in some in a later one
     Hkv, D, kernel, B = 2, 128, 7, W + 90
-    q, k, v = rand_inputs(1, 1, G * Hkv, Hkv, D, L, W, seed=L + W)
+    q, k, v = rand_inputs(NL, Bt, G * Hkv, Hkv, D, L, W, seed=L + W)
     q[..., 0] = 12.0
     k[..., 0] = 0.0
     k[:, :, :, ::32, 0] = -56.0
@@ -105,10 +105,10 @@ def test_sums_that_overflow_in_clusters_of(laq, L, C, G, W, group):
     assert err < SCORE_RTOL
 
 
-@pytest.mark.parametrize("L,C", SIZES)
+@pytest.mark.parametrize("NL,Bt,L,C", SIZES)
 @pytest.mark.parametrize("W,G", [(1, 4), (3, 4), (5, 8), (6, 4), (8, 7), (16, 4)])
-def test_cluster_scoring_per_head_with_several_tiles(laq, L, C, W, G):
-    q, k, v = rand_inputs(1, 1, 2 * G, 2, 128, L, W, seed=L + W, kscale=1.5)
+def test_cluster_scoring_per_head_with_several_tiles(laq, NL, Bt, L, C, W, G):
+    q, k, v = rand_inputs(NL, Bt, 2 * G, 2, 128, L, W, seed=L + W, kscale=1.5)
     for mode in (1, 2):
         assert launched_cluster(laq, q, k, W, 7, 80, mode) == C
         compare_all_units(laq, q, k, v, W, 7, 80, group_mode=mode)

@@ -143,21 +143,21 @@ def test_wait_that_runs_out_in_the_other_scoring_kernels(G, W, tiles, group):
 
 
 @pytest.mark.parametrize("G,W", [(1, 8), (2, 8), (3, 8), (4, 8), (5, 8), (6, 8), (8, 8)])   # every group of eight rows
-@pytest.mark.parametrize("L,C", [(2304, 9), (8192, 16)])
+@pytest.mark.parametrize("NL,Bt,L,C", [(4, 2, 2000, 6), (1, 1, 8192, 16)])
 @pytest.mark.parametrize("group", [0, 2])
-def test_wait_that_runs_out_in_clusters(G, W, L, C, group):
+def test_wait_that_runs_out_in_clusters(G, W, NL, Bt, L, C, group):
     # every variant of the cluster kernel, for a size between the powers of two and for one of them
     from paper_2505_20334_b200 import binding as laq
 
     hooked = hooked_library()
     Hkv, D = 2, 128
     g = torch.Generator(device="cuda").manual_seed(G + L)
-    q = torch.randn((1, 1, G * Hkv, W, D), generator=g, device="cuda", dtype=torch.bfloat16)
-    k = torch.randn((1, 1, Hkv, L, D), generator=g, device="cuda", dtype=torch.bfloat16)
+    q = torch.randn((NL, Bt, G * Hkv, W, D), generator=g, device="cuda", dtype=torch.bfloat16)
+    k = torch.randn((NL, Bt, Hkv, L, D), generator=g, device="cuda", dtype=torch.bfloat16)
     p = laq.params_for(q, k, W, 7, 100)
     p.group_mode = group
     ws = laq.alloc_workspace(p, "cuda")
-    scores = torch.zeros((1, 1, Hkv * (G if group == 2 else 1), L - W), device="cuda")
+    scores = torch.zeros((NL, Bt, Hkv * (G if group == 2 else 1), L - W), device="cuda")
     stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
 
     def run():
