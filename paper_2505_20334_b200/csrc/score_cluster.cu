@@ -194,8 +194,9 @@ struct Unit {
   int Lu;     // length of the unit's prompt
   int tiles;  // tiles of the unit that this CTA holds
 };
-// kShift: the cluster size is a power of two, c_log2 its logarithm. (Kernels of their own: with a product in place of the shift and
-// a division of the tiles the others took up to 4 % longer, 256 units of 12000 keys and 64 rows 190 -> 197 us.)
+// kShift: the cluster size is a power of two, c_log2 its logarithm. (Kernels of their own: with a product in
+// place of the shift and a division of the tiles the others took up to 4 % longer, 256 units of 12000 keys and
+// 64 rows 190 -> 197 us.)
 // Place in the unit of the i-th tile of the CTA of that rank.
 template <bool kShift>
 __device__ __forceinline__ int tile_at(const ClArgs& a, int rank, int i) {

@@ -327,7 +327,8 @@ __device__ __forceinline__ void stats_cols64(uint32_t taddr, float c, float& m, 
 //   M > 128, one sum, kSplit: 1, as precise as the MUFU's (scores 1.2e-7 from fp64 in the 2-norm either way). The MUFU
 //     alone takes 2048 of a tile's 2570 cycles a sweep: 65536 keys, 640 units 7136 -> 6894 us, 5000 keys, 160
 //     units 161 -> 156, 64 dims 419 -> 404 (2 of 8: 7031, 153, 403).
-//   M > 128, whole: 0 (1 of 8 -1 to +1 %). A sum per head: 0 (1 of 8: 160 rows, 6000 keys 147 -> 150, 256 rows, 9001 keys 131 -> 130).
+//   M > 128, whole: 0 (1 of 8 -1 to +1 %). A sum per head: 0 (1 of 8: 160 rows, 6000 keys 147 -> 150, 256
+//     rows, 9001 keys 131 -> 130).
 //   64 < M <= 128, 128 dims: LAQ_POLY_PAIRS_S1 of a cheaper one, 7.5e-5 off, which leaves the scores within
 //     1e-6 (on the MUFU alone 2e-7). Other head dims: 0, so that their scores are as precise as on the CUDA
 //     cores, where they used to be formed (64 dims, 128 rows, 128 units of 32768 keys 324 us, with it 310).
